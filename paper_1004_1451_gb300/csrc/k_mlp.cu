@@ -12,6 +12,8 @@
 // with the incoming gradient rounded to bf16; bias gradients and Adam stay in FP32.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <vector>
@@ -79,8 +81,8 @@ __global__ void k_mlp_to_bf16(const float* __restrict__ P, __nv_bfloat16* __rest
 
 // ------------------------------------------------------------------ forward (tensor cores)
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    const __nv_bfloat16 a = __float2bfloat16_rn(lo), b = __float2bfloat16_rn(hi);
-    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);  // one conversion instruction for both
+    return *reinterpret_cast<const uint32_t*>(&v);
 }
 template <typename TA>
 __device__ __forceinline__ uint32_t load_pair(const TA* p);  // elements p[0], p[1] as bf16x2
@@ -157,6 +159,178 @@ __global__ void __launch_bounds__(FWD_WARPS * 32)
         } else {
             if (va) *reinterpret_cast<float2*>(Yf + ra * N + c) = make_float2(v0, v1);
             if (vb) *reinterpret_cast<float2*>(Yf + rb * N + c) = make_float2(v2, v3);
+        }
+    }
+}
+
+// ------------------------------------------------------------------ the network in one kernel
+// All three layers of a row tile in one warp, the activations in registers: an m16n8
+// accumulator holds the same elements of a row as the m16k16 fragment of the next product
+// needs, so relu and the rounding to bf16 turn it into the next layer's A operand in place.
+// The k-steps run in the order of a layer on its own, so the values are those of three
+// separate layer kernels, bit for bit.
+//
+// What bounds it: the tensor pipe under mma.sync (29 us at its rate for 2^18 rows, ncu), then HBM
+// (134 MB in and out, 20 us of the copy rate).  Three layer kernels passed H1 and H2 through memory
+// (400 MB), loaded weight fragments four bytes at a time and staged the weights in every block of
+// 64 rows: 178 us.  Here one block per SM keeps all weights in shared memory (71 KB, staged once)
+// and its 12 warps walk the 16-row tiles; ldmatrix fetches four fragment registers at a time, and
+// each warp's next feature tile arrives by cp.async while the current one is computed: 47 us.
+// Measured besides: two row tiles a warp sharing each weight fragment, 52 us with 8 warps and 64
+// with 10 (registers), 58 with 12 and no feature staging; one row tile with 16 warps, 48 us.
+constexpr int NET_WARPS = 12;
+constexpr int NET_LD1 = MLP_F + 8, NET_LD2 = MLP_H + 8;  // padded strides: ldmatrix rows on distinct banks
+constexpr int NET_LDX = MLP_F + 8;  // of a feature tile: the fragment loads of a half warp on distinct banks
+struct NetSmem {
+    __nv_bfloat16 w1[MLP_H * NET_LD1];
+    __nv_bfloat16 w2[MLP_H * NET_LD2];
+    __nv_bfloat16 w3[MLP_S * NET_LD2];
+    float b1[MLP_H], b2[MLP_H], b3[MLP_S];
+};
+
+__device__ __forceinline__ void net_cp16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+// rows x K bf16 (row-major, contiguous) into rows of LD elements, by the whole block
+template <int K, int LD>
+__device__ __forceinline__ void net_stage(__nv_bfloat16* dst, const __nv_bfloat16* __restrict__ src, int rows) {
+    constexpr int C = K / 8;  // 16-byte pieces a row
+    for (int e = threadIdx.x; e < rows * C; e += blockDim.x) {
+        const int r = e / C, c = e - r * C;
+        net_cp16(dst + r * LD + 8 * c, src + (int64_t)r * K + 8 * c);
+    }
+}
+// All weights and biases into shared memory; every thread of the block calls it.
+__device__ __forceinline__ void net_stage_weights(NetSmem& sm, const __nv_bfloat16* __restrict__ Wb,
+                                                  const float* __restrict__ P) {
+    net_stage<MLP_F, NET_LD1>(sm.w1, Wb + BOFF_W1, MLP_H);
+    net_stage<MLP_H, NET_LD2>(sm.w2, Wb + BOFF_W2, MLP_H);
+    net_stage<MLP_H, NET_LD2>(sm.w3, Wb + BOFF_W3, MLP_S);
+    for (int e = threadIdx.x; e < MLP_H; e += blockDim.x) {
+        sm.b1[e] = P[OFF_B1 + e];
+        sm.b2[e] = P[OFF_B2 + e];
+        if (e < MLP_S) sm.b3[e] = P[OFF_B3 + e];
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+}
+
+// the fragments b0, b1 of two neighbouring n8 tiles at one k16 step: w = the element (n, k) of
+// the first tile's corner, rows of LD
+template <int LD>
+__device__ __forceinline__ void net_ldb(uint32_t (&b)[4], const __nv_bfloat16* w, int lane) {
+    const __nv_bfloat16* p = w + ((lane & 7) + ((lane >> 4) << 3)) * LD + ((lane >> 3) & 1) * 8;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+// acc (NT n8 tiles) = A W^T for the NT * 8 outputs whose weights start at w
+template <int NT, int KS, int LD>
+__device__ __forceinline__ void net_product(float (&acc)[NT][4], const uint32_t (&A)[KS][4], const __nv_bfloat16* w,
+                                            int lane) {
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[n][e] = 0.f;
+#pragma unroll
+    for (int k = 0; k < KS; ++k) {
+#pragma unroll
+        for (int n = 0; n < NT; n += 2) {
+            uint32_t b[4];
+            net_ldb<LD>(b, w + n * 8 * LD + k * 16, lane);
+            mma_bf16(acc[n], A[k][0], A[k][1], A[k][2], A[k][3], b[0], b[1]);
+            mma_bf16(acc[n + 1], A[k][0], A[k][1], A[k][2], A[k][3], b[2], b[3]);
+        }
+    }
+}
+// One hidden layer: the next layer's A operand from this one's (128 outputs in slices of 32)
+template <int KS, int LD>
+__device__ __forceinline__ void net_hidden(const uint32_t (&A)[KS][4], uint32_t (&H)[8][4], const __nv_bfloat16* w,
+                                           const float* bias, int lane) {
+    const int t = lane & 3;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        float acc[4][4];
+        net_product<4, KS, LD>(acc, A, w + c * 32 * LD, lane);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            const float2 bb = *reinterpret_cast<const float2*>(bias + c * 32 + n * 8 + 2 * t);
+            uint32_t* h = H[2 * c + (n >> 1)] + 2 * (n & 1);
+            h[0] = pack_bf16(fmaxf(acc[n][0] + bb.x, 0.f), fmaxf(acc[n][1] + bb.y, 0.f));
+            h[1] = pack_bf16(fmaxf(acc[n][2] + bb.x, 0.f), fmaxf(acc[n][3] + bb.y, 0.f));
+        }
+    }
+}
+
+// Copies the 16 rows of X from r0 (those < M; 448 bytes each, contiguous) into a warp's tile
+// buffer, asynchronously: 16-byte pieces where X allows them (wide), else 8-byte ones.
+__device__ __forceinline__ void net_fetch(float* buf, const float* __restrict__ X, int64_t r0, int64_t M, bool wide,
+                                          int lane) {
+    const int rows = (int)(M - r0 < 16 ? M - r0 : 16);
+    const float* src = X + r0 * MLP_F;
+    if (wide) {
+        constexpr int C = MLP_F / 4;
+#pragma unroll
+        for (int e = lane; e < 16 * C; e += 32) {
+            const int r = e / C, c = e - r * C;
+            if (r < rows) net_cp16(buf + r * NET_LDX + 4 * c, src + 4 * e);
+        }
+    } else {
+        constexpr int C = MLP_F / 2;
+        for (int e = lane; e < rows * C; e += 32) {
+            const int r = e / C, c = e - r * C;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                             (unsigned)__cvta_generic_to_shared(buf + r * NET_LDX + 2 * c)),
+                         "l"(src + 2 * e)
+                         : "memory");
+        }
+    }
+}
+
+__global__ void __launch_bounds__(NET_WARPS * 32)
+    k_mlp_net(int64_t M, const float* __restrict__ X, const __nv_bfloat16* __restrict__ Wb, const float* __restrict__ P,
+              float* __restrict__ Y) {
+    pdl_begin();
+    extern __shared__ __align__(16) unsigned char net_raw[];
+    NetSmem& sm = *reinterpret_cast<NetSmem*>(net_raw);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    float* buf = reinterpret_cast<float*>(net_raw + sizeof(NetSmem)) + warp * (16 * NET_LDX);
+    const int64_t tiles = (M + 15) / 16, step = (int64_t)gridDim.x * NET_WARPS;
+    const bool wide = (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    // neighbouring tiles on different SMs, so that few rows spread over the whole chip
+    int64_t q = blockIdx.x + (int64_t)gridDim.x * warp;
+    if (q < tiles) net_fetch(buf, X, q * 16, M, wide, lane);
+    net_stage_weights(sm, Wb, P);
+    for (; q < tiles; q += step) {
+        const int64_t ra = q * 16 + g, rb = ra + 8;
+        const bool va = ra < M, vb = rb < M;
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+        uint32_t H1[8][4], H2[8][4];
+        {
+            uint32_t A[MLP_F / 16][4];
+            const float* p = buf + g * NET_LDX + 2 * t;
+#pragma unroll
+            for (int k = 0; k < MLP_F / 16; ++k) {
+                A[k][0] = va ? load_pair<float>(p + 16 * k) : 0u;
+                A[k][1] = vb ? load_pair<float>(p + 8 * NET_LDX + 16 * k) : 0u;
+                A[k][2] = va ? load_pair<float>(p + 16 * k + 8) : 0u;
+                A[k][3] = vb ? load_pair<float>(p + 8 * NET_LDX + 16 * k + 8) : 0u;
+            }
+            __syncwarp();  // the tile is in registers: its buffer takes the next one meanwhile
+            if (q + step < tiles) net_fetch(buf, X, (q + step) * 16, M, wide, lane);
+            net_hidden<MLP_F / 16, NET_LD1>(A, H1, sm.w1, sm.b1, lane);
+        }
+        net_hidden<MLP_H / 16, NET_LD2>(H1, H2, sm.w2, sm.b2, lane);
+        float acc[2][4];
+        net_product<2, MLP_H / 16, NET_LD2>(acc, H2, sm.w3, lane);
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            const int c = n * 8 + 2 * t;
+            const float2 bb = *reinterpret_cast<const float2*>(sm.b3 + c);
+            if (va) *reinterpret_cast<float2*>(Y + ra * MLP_S + c) = make_float2(acc[n][0] + bb.x, acc[n][1] + bb.y);
+            if (vb) *reinterpret_cast<float2*>(Y + rb * MLP_S + c) = make_float2(acc[n][2] + bb.x, acc[n][3] + bb.y);
         }
     }
 }
@@ -422,10 +596,20 @@ static void forward_rows(const Model* m, int64_t rows, const float* feat, MlpWor
 
 void mlp_forward(const Model* m, int64_t rows, const float* feat, float* Y, cudaStream_t s) {
     if (rows <= 0) return;
-    AllocStream as_(s);
-    MlpWork w;
-    w.ensure(rows, false);
-    forward_rows(m, rows, feat, w, Y, s);
+    constexpr size_t smem = sizeof(NetSmem) + sizeof(float) * NET_WARPS * 16 * NET_LDX;
+    static_assert(smem <= 227 * 1024, "weights and feature tiles in shared memory");
+    static std::atomic<bool> allowed[256] = {};  // more than 48 KB: once per device (idempotent across threads)
+    int dev = 0, nsm = 0;
+    BAMG_CK(cudaGetDevice(&dev));
+    BAMG_REQUIRE(dev >= 0 && dev < 256, BAMG_EINVAL, "device ordinal out of range");
+    if (!allowed[dev]) {
+        BAMG_CK(cudaFuncSetAttribute(k_mlp_net, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        allowed[dev] = true;
+    }
+    BAMG_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const unsigned grid = (unsigned)std::min<int64_t>(nsm > 0 ? nsm : 1, (rows + 15) / 16);
+    BAMG_LAUNCH(k_mlp_net, grid, NET_WARPS * 32, smem, s, rows, feat, (const __nv_bfloat16*)m->Wb.get(),
+                (const float*)m->P.get(), Y);
 }
 
 // Gradients of the batch loss into m->G (zeroed first); the loss sum into w.loss.

@@ -1,0 +1,56 @@
+"""Kernels at the sizes where their tiling can go wrong: tile edges, remainders, the smallest
+and the largest launch shapes, and the alignments their wide loads distinguish."""
+
+import numpy as np
+import pytest
+
+from gpu_util import need_gpu
+from oracle import learned as ol
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    need_gpu()
+
+
+def _network(rows, seed=3):
+    """A model with random parameters, its FP32 parameters as FP64 arrays, and features."""
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+
+    rng = np.random.default_rng(seed)
+    p = ol.init_params(seed)
+    for k in ("b1", "b2", "b3"):
+        p[k] = rng.standard_normal(p[k].shape) * 0.05
+    flat = np.concatenate([p[k].ravel() for k in ("W1", "b1", "W2", "b2", "W3", "b3")]).astype(np.float32)
+    m = bamg.Model(0)
+    m.set(flat)
+    p32 = {k: v.astype(np.float32).astype(np.float64) for k, v in p.items()}
+    feat = rng.standard_normal((rows, 112)).astype(np.float32) * 0.5
+    feat[:, 0:96:6] = np.arange(16)[None, :] < rng.integers(1, 17, rows)[:, None]
+    return torch, m, p32, feat
+
+
+@pytest.mark.parametrize("rows", [1, 15, 16, 17, 33, 16 * 152 * 12 - 1, 16 * 152 * 12 + 17])
+def test_forward_at_tile_edges(rows):
+    """Every row equals the row on its own, bit for bit (a row's arithmetic does not depend on its
+    place), also from storage that is only 8-byte aligned; the first rows agree with the oracle, whose
+    sums are exact: a difference is a bf16 rounding that fell the other way (2^-8 of an activation)."""
+    base = min(rows, 40)
+    torch, m, p, f = _network(base)
+    idx = np.arange(rows) % base
+    Fd = torch.tensor(f, device="cuda")[torch.tensor(idx, device="cuda")].contiguous()
+    y = m.forward(Fd)
+    alone = torch.cat([m.forward(Fd[k:k + 1].contiguous()) for k in range(base)])
+    assert torch.equal(y, alone[torch.tensor(idx, device="cuda")])
+    shifted = torch.empty(rows * 112 + 2, dtype=torch.float32, device="cuda")[2:].view(rows, 112)
+    shifted.copy_(Fd)
+    assert shifted.data_ptr() % 16 == 8
+    assert torch.equal(m.forward(shifted), y)
+    y_o, _ = ol.forward(p, f.astype(np.float64), use_bf16=True)
+    err = np.abs(alone.cpu().numpy() - y_o)
+    scale = max(1.0, np.abs(y_o).max())
+    assert err.max() <= 1e-2 * scale and err.mean() <= 1e-4 * scale
