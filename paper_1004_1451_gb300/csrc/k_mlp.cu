@@ -5,8 +5,8 @@
 // beta2 = 0.999, eps = 1e-8, He-uniform initialisation from SplitMix64) are those of the
 // interface declared in include/bamg.h.
 //
-// Forward products run on the tensor cores (mma.sync m16n8k16, bf16 in, FP32 accumulate):
-// one warp computes 16 rows x N outputs, the weights staged once per block in shared
+// All products run on the tensor cores (mma.sync m16n8k16, bf16 in, FP32 accumulate): one
+// warp takes 16 rows through all layers, the weights staged once per block in shared
 // memory with a padded row stride.  The training backward's products (input gradients
 // through the ReLU masks, weight gradients summed over the batch) use the same instruction
 // with the incoming gradient rounded to bf16; bias gradients and Adam stay in FP32.
@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <vector>
 
@@ -24,7 +25,9 @@ namespace bamg {
 
 // ------------------------------------------------------------------ parameter layout
 // One flat FP32 buffer [W1 | b1 | W2 | b2 | W3 | b3]; W_l is out x in, row-major.  The
-// bfloat16 copies of W1, W2, W3 sit in one flat buffer in the same order.
+// bfloat16 copies of W1, W2, W3 sit in one buffer in the same order, their rows padded as the
+// kernels keep them in shared memory (ldmatrix rows on distinct banks), so that a block stages
+// all of them with one flat copy.
 constexpr int64_t OFF_W1 = 0;
 constexpr int64_t OFF_B1 = OFF_W1 + (int64_t)MLP_H * MLP_F;
 constexpr int64_t OFF_W2 = OFF_B1 + MLP_H;
@@ -32,18 +35,20 @@ constexpr int64_t OFF_B2 = OFF_W2 + (int64_t)MLP_H * MLP_H;
 constexpr int64_t OFF_W3 = OFF_B2 + MLP_H;
 constexpr int64_t OFF_B3 = OFF_W3 + (int64_t)MLP_S * MLP_H;
 constexpr int64_t NPARAM = OFF_B3 + MLP_S;
+constexpr int NET_LD1 = MLP_F + 8, NET_LD2 = MLP_H + 8;  // padded strides of the bf16 copies
 constexpr int64_t BOFF_W1 = 0;
-constexpr int64_t BOFF_W2 = BOFF_W1 + (int64_t)MLP_H * MLP_F;
-constexpr int64_t BOFF_W3 = BOFF_W2 + (int64_t)MLP_H * MLP_H;
-constexpr int64_t NBF = BOFF_W3 + (int64_t)MLP_S * MLP_H;
+constexpr int64_t BOFF_W2 = BOFF_W1 + (int64_t)MLP_H * NET_LD1;
+constexpr int64_t BOFF_W3 = BOFF_W2 + (int64_t)MLP_H * NET_LD2;
+constexpr int64_t NBF = BOFF_W3 + (int64_t)MLP_S * NET_LD2;
 
 int64_t mlp_param_count() { return NPARAM; }
 
 // index of a flat parameter in the bf16 copy, or -1 for a bias
 __device__ __forceinline__ int64_t bf_index(int64_t q) {
-    if (q < OFF_B1) return BOFF_W1 + q;
-    if (q >= OFF_W2 && q < OFF_B2) return BOFF_W2 + (q - OFF_W2);
-    if (q >= OFF_W3 && q < OFF_B3) return BOFF_W3 + (q - OFF_W3);
+    const int i = (int)q;
+    if (q < OFF_B1) return BOFF_W1 + i / MLP_F * NET_LD1 + i % MLP_F;
+    if (q >= OFF_W2 && q < OFF_B2) return BOFF_W2 + (i - (int)OFF_W2) / MLP_H * NET_LD2 + (i - (int)OFF_W2) % MLP_H;
+    if (q >= OFF_W3 && q < OFF_B3) return BOFF_W3 + (i - (int)OFF_W3) / MLP_H * NET_LD2 + (i - (int)OFF_W3) % MLP_H;
     return -1;
 }
 
@@ -84,16 +89,9 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);  // one conversion instruction for both
     return *reinterpret_cast<const uint32_t*>(&v);
 }
-template <typename TA>
-__device__ __forceinline__ uint32_t load_pair(const TA* p);  // elements p[0], p[1] as bf16x2
-template <>
-__device__ __forceinline__ uint32_t load_pair<float>(const float* p) {
+__device__ __forceinline__ uint32_t load_pair(const float* p) {  // elements p[0], p[1] as bf16x2
     const float2 v = *reinterpret_cast<const float2*>(p);
     return pack_bf16(v.x, v.y);
-}
-template <>
-__device__ __forceinline__ uint32_t load_pair<__nv_bfloat16>(const __nv_bfloat16* p) {
-    return *reinterpret_cast<const uint32_t*>(p);
 }
 
 __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
@@ -103,64 +101,6 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
         "{%0,%1,%2,%3};\n"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-// Y = act(A W^T + b): A is M x K (row-major, element type TA, rounded to bf16 on load), W
-// is N x K bf16, b FP32.  relu: Yb (bf16, M x N) = max(0, .); else Yf (FP32) = the sum.
-// Block: 4 warps x 16 rows.  K a multiple of 16, N a multiple of 8, N <= 128, K <= 128.
-constexpr int FWD_WARPS = 4;
-template <typename TA, int N, int K>
-__global__ void __launch_bounds__(FWD_WARPS * 32)
-    k_mlp_layer(int64_t M, const TA* __restrict__ A, const __nv_bfloat16* __restrict__ W, const float* __restrict__ bias,
-                bool relu, __nv_bfloat16* __restrict__ Yb, float* __restrict__ Yf) {
-    pdl_begin();
-    constexpr int LDW = K + 8;  // padded stride (bf16 elements): conflict-free fragment loads
-    __shared__ __align__(16) __nv_bfloat16 sW[N * LDW];
-    __shared__ float sb[N];
-    for (int idx = threadIdx.x; idx < N * K / 2; idx += blockDim.x) {
-        const int n = (2 * idx) / K, k = (2 * idx) % K;
-        *reinterpret_cast<uint32_t*>(&sW[n * LDW + k]) = *reinterpret_cast<const uint32_t*>(&W[(int64_t)n * K + k]);
-    }
-    for (int n = threadIdx.x; n < N; n += blockDim.x) sb[n] = bias[n];
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int64_t r0 = ((int64_t)blockIdx.x * FWD_WARPS + warp) * 16;
-    if (r0 >= M) return;
-    const int64_t ra = r0 + g, rb = r0 + g + 8;
-    const bool va = ra < M, vb = rb < M;
-    float acc[N / 8][4];
-#pragma unroll
-    for (int nt = 0; nt < N / 8; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[nt][e] = 0.f;
-#pragma unroll
-    for (int kk = 0; kk < K; kk += 16) {
-        const uint32_t a0 = va ? load_pair<TA>(A + ra * K + kk + 2 * t) : 0u;
-        const uint32_t a1 = vb ? load_pair<TA>(A + rb * K + kk + 2 * t) : 0u;
-        const uint32_t a2 = va ? load_pair<TA>(A + ra * K + kk + 2 * t + 8) : 0u;
-        const uint32_t a3 = vb ? load_pair<TA>(A + rb * K + kk + 2 * t + 8) : 0u;
-#pragma unroll
-        for (int nt = 0; nt < N / 8; ++nt) {
-            const __nv_bfloat16* wr = sW + (nt * 8 + g) * LDW + kk + 2 * t;
-            const uint32_t b0 = *reinterpret_cast<const uint32_t*>(wr);
-            const uint32_t b1 = *reinterpret_cast<const uint32_t*>(wr + 8);
-            mma_bf16(acc[nt], a0, a1, a2, a3, b0, b1);
-        }
-    }
-#pragma unroll
-    for (int nt = 0; nt < N / 8; ++nt) {
-        const int c = nt * 8 + 2 * t;
-        float v0 = acc[nt][0] + sb[c], v1 = acc[nt][1] + sb[c + 1];
-        float v2 = acc[nt][2] + sb[c], v3 = acc[nt][3] + sb[c + 1];
-        if (relu) {
-            v0 = fmaxf(v0, 0.f), v1 = fmaxf(v1, 0.f), v2 = fmaxf(v2, 0.f), v3 = fmaxf(v3, 0.f);
-            if (va) *reinterpret_cast<uint32_t*>(Yb + ra * N + c) = pack_bf16(v0, v1);
-            if (vb) *reinterpret_cast<uint32_t*>(Yb + rb * N + c) = pack_bf16(v2, v3);
-        } else {
-            if (va) *reinterpret_cast<float2*>(Yf + ra * N + c) = make_float2(v0, v1);
-            if (vb) *reinterpret_cast<float2*>(Yf + rb * N + c) = make_float2(v2, v3);
-        }
-    }
 }
 
 // ------------------------------------------------------------------ the network in one kernel
@@ -175,11 +115,10 @@ __global__ void __launch_bounds__(FWD_WARPS * 32)
 // (400 MB), loaded weight fragments four bytes at a time and staged the weights in every block of
 // 64 rows: 178 us.  Here one block per SM keeps all weights in shared memory (71 KB, staged once)
 // and its 12 warps walk the 16-row tiles; ldmatrix fetches four fragment registers at a time, and
-// each warp's next feature tile arrives by cp.async while the current one is computed: 47 us.
+// each warp's next feature tile arrives by cp.async while the current one is computed: 45 us.
 // Measured besides: two row tiles a warp sharing each weight fragment, 52 us with 8 warps and 64
 // with 10 (registers), 58 with 12 and no feature staging; one row tile with 16 warps, 48 us.
 constexpr int NET_WARPS = 12;
-constexpr int NET_LD1 = MLP_F + 8, NET_LD2 = MLP_H + 8;  // padded strides: ldmatrix rows on distinct banks
 constexpr int NET_LDX = MLP_F + 8;  // of a feature tile: the fragment loads of a half warp on distinct banks
 struct NetSmem {
     __nv_bfloat16 w1[MLP_H * NET_LD1];
@@ -192,21 +131,17 @@ __device__ __forceinline__ void net_cp16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
 }
-// rows x K bf16 (row-major, contiguous) into rows of LD elements, by the whole block
-template <int K, int LD>
-__device__ __forceinline__ void net_stage(__nv_bfloat16* dst, const __nv_bfloat16* __restrict__ src, int rows) {
-    constexpr int C = K / 8;  // 16-byte pieces a row
-    for (int e = threadIdx.x; e < rows * C; e += blockDim.x) {
-        const int r = e / C, c = e - r * C;
-        net_cp16(dst + r * LD + 8 * c, src + (int64_t)r * K + 8 * c);
-    }
-}
 // All weights and biases into shared memory; every thread of the block calls it.
+static_assert(offsetof(NetSmem, b1) == sizeof(__nv_bfloat16) * NBF && NBF % 8 == 0, "one flat copy of the weights");
+template <int THREADS>
 __device__ __forceinline__ void net_stage_weights(NetSmem& sm, const __nv_bfloat16* __restrict__ Wb,
                                                   const float* __restrict__ P) {
-    net_stage<MLP_F, NET_LD1>(sm.w1, Wb + BOFF_W1, MLP_H);
-    net_stage<MLP_H, NET_LD2>(sm.w2, Wb + BOFF_W2, MLP_H);
-    net_stage<MLP_H, NET_LD2>(sm.w3, Wb + BOFF_W3, MLP_S);
+    constexpr int C = (int)(NBF / 8);  // 16-byte pieces
+#pragma unroll
+    for (int e = 0; e < (C + THREADS - 1) / THREADS; ++e) {
+        const int c = e * THREADS + threadIdx.x;
+        if (c < C) net_cp16(sm.w1 + 8 * c, Wb + 8 * c);
+    }
     for (int e = threadIdx.x; e < MLP_H; e += blockDim.x) {
         sm.b1[e] = P[OFF_B1 + e];
         sm.b2[e] = P[OFF_B2 + e];
@@ -263,16 +198,17 @@ __device__ __forceinline__ void net_hidden(const uint32_t (&A)[KS][4], uint32_t 
     }
 }
 
-// Copies the 16 rows of X from r0 (those < M; 448 bytes each, contiguous) into a warp's tile
-// buffer, asynchronously: 16-byte pieces where X allows them (wide), else 8-byte ones.
+// Copies ROWS rows of X from r0 (those < M; 448 bytes each, contiguous) into a tile buffer by one
+// warp, asynchronously: 16-byte pieces where X allows them (wide), else 8-byte ones.
+template <int ROWS>
 __device__ __forceinline__ void net_fetch(float* buf, const float* __restrict__ X, int64_t r0, int64_t M, bool wide,
                                           int lane) {
-    const int rows = (int)(M - r0 < 16 ? M - r0 : 16);
+    const int rows = (int)(M - r0 < ROWS ? M - r0 : ROWS);
     const float* src = X + r0 * MLP_F;
     if (wide) {
         constexpr int C = MLP_F / 4;
 #pragma unroll
-        for (int e = lane; e < 16 * C; e += 32) {
+        for (int e = lane; e < ROWS * C; e += 32) {
             const int r = e / C, c = e - r * C;
             if (r < rows) net_cp16(buf + r * NET_LDX + 4 * c, src + 4 * e);
         }
@@ -288,6 +224,19 @@ __device__ __forceinline__ void net_fetch(float* buf, const float* __restrict__ 
     }
 }
 
+// The first product's A operand from a feature tile (va, vb: rows g and g + 8 exist)
+__device__ __forceinline__ void net_inputs(uint32_t (&A)[MLP_F / 16][4], const float* buf, bool va, bool vb, int g,
+                                           int t) {
+    const float* p = buf + g * NET_LDX + 2 * t;
+#pragma unroll
+    for (int k = 0; k < MLP_F / 16; ++k) {
+        A[k][0] = va ? load_pair(p + 16 * k) : 0u;
+        A[k][1] = vb ? load_pair(p + 8 * NET_LDX + 16 * k) : 0u;
+        A[k][2] = va ? load_pair(p + 16 * k + 8) : 0u;
+        A[k][3] = vb ? load_pair(p + 8 * NET_LDX + 16 * k + 8) : 0u;
+    }
+}
+
 __global__ void __launch_bounds__(NET_WARPS * 32)
     k_mlp_net(int64_t M, const float* __restrict__ X, const __nv_bfloat16* __restrict__ Wb, const float* __restrict__ P,
               float* __restrict__ Y) {
@@ -300,8 +249,8 @@ __global__ void __launch_bounds__(NET_WARPS * 32)
     const bool wide = (reinterpret_cast<uintptr_t>(X) & 15) == 0;
     // neighbouring tiles on different SMs, so that few rows spread over the whole chip
     int64_t q = blockIdx.x + (int64_t)gridDim.x * warp;
-    if (q < tiles) net_fetch(buf, X, q * 16, M, wide, lane);
-    net_stage_weights(sm, Wb, P);
+    if (q < tiles) net_fetch<16>(buf, X, q * 16, M, wide, lane);
+    net_stage_weights<NET_WARPS * 32>(sm, Wb, P);
     for (; q < tiles; q += step) {
         const int64_t ra = q * 16 + g, rb = ra + 8;
         const bool va = ra < M, vb = rb < M;
@@ -310,16 +259,9 @@ __global__ void __launch_bounds__(NET_WARPS * 32)
         uint32_t H1[8][4], H2[8][4];
         {
             uint32_t A[MLP_F / 16][4];
-            const float* p = buf + g * NET_LDX + 2 * t;
-#pragma unroll
-            for (int k = 0; k < MLP_F / 16; ++k) {
-                A[k][0] = va ? load_pair<float>(p + 16 * k) : 0u;
-                A[k][1] = vb ? load_pair<float>(p + 8 * NET_LDX + 16 * k) : 0u;
-                A[k][2] = va ? load_pair<float>(p + 16 * k + 8) : 0u;
-                A[k][3] = vb ? load_pair<float>(p + 8 * NET_LDX + 16 * k + 8) : 0u;
-            }
+            net_inputs(A, buf, va, vb, g, t);
             __syncwarp();  // the tile is in registers: its buffer takes the next one meanwhile
-            if (q + step < tiles) net_fetch(buf, X, (q + step) * 16, M, wide, lane);
+            if (q + step < tiles) net_fetch<16>(buf, X, (q + step) * 16, M, wide, lane);
             net_hidden<MLP_F / 16, NET_LD1>(A, H1, sm.w1, sm.b1, lane);
         }
         net_hidden<MLP_H / 16, NET_LD2>(H1, H2, sm.w2, sm.b2, lane);
@@ -336,189 +278,424 @@ __global__ void __launch_bounds__(NET_WARPS * 32)
 }
 
 // ------------------------------------------------------------------ backward
-// dY = (2 / rows_in_batch) mask (Y - T), mask = the features' slot-valid flags; the batch
-// loss sum mask (Y - T)^2 / rows_in_batch is added to *loss.
-__global__ void k_mlp_loss(int64_t M, int64_t Mtot, const float* __restrict__ Y, const float* __restrict__ Tg,
-                           const float* __restrict__ Fe, float* __restrict__ dY, double* __restrict__ loss) {
-    pdl_begin();
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double l = 0.0;
-    if (q < M * MLP_S) {
-        const int64_t row = q / MLP_S;
-        const int s = (int)(q - row * MLP_S);
-        const float mask = Fe[row * MLP_F + MLP_NF_SLOT * s] > 0.f ? 1.f : 0.f;
-        const float d = mask * (Y[q] - Tg[q]);
-        dY[q] = 2.f * d / (float)Mtot;
-        l = (double)d * (double)d / (double)Mtot;
-    }
-    l = warp_sum(l);
-    if ((threadIdx.x & 31) == 0 && l != 0.0) atomicAdd(loss, l);
+// A training step is two kernels and the optimiser.  k_mlp_step takes a row tile through the
+// forward pass, the masked loss and the input gradients in one warp: the gradient that enters a
+// product is rounded to bf16 like the forward's inputs, which again turns an accumulator into the
+// next product's A operand in place.  It leaves H1, H2 and the rounded gradients in memory (bf16)
+// for the weight gradients and the unrounded gradients (FP32) for the bias gradients (k_mlp_wgrad, all
+// layers in one launch), and adds up the loss.
+//
+// What bounds it: launches and latency (a batch of 4096 rows is 0.9 GFLOP and 6 MB; 10 us of
+// dependent instructions in k_mlp_step and 6 in k_mlp_wgrad, tensor pipe below 10%).  It took 14
+// launches and 143 us, 88 of them in column sums that one block per column walked row by row, 26 in
+// the transposing loads of each weight gradient; now three launches and 30 us.  (Summing the bias
+// gradients in k_mlp_step's warps and 128 rows a weight block measured 27 us; the order of the sums
+// here, 256 rows a chain and the column sums' tree, is the one the results always had.)
+
+// B fragments of two neighbouring n8 tiles at one k16 step for a product with W itself (k = the
+// row of w, n = the column): w = the corner (k, n), rows of LD
+template <int LD>
+__device__ __forceinline__ void net_ldb_t(uint32_t (&b)[4], const __nv_bfloat16* w, int lane) {
+    const __nv_bfloat16* p = w + ((lane & 7) + ((lane >> 3) & 1) * 8) * LD + ((lane >> 4) << 3);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
 }
-
-// The backward products on the tensor cores as well (mma.sync m16n8k16, bf16 in, FP32
-// accumulate): the gradient entering a product is rounded to bf16 like the forward's inputs;
-// the bias gradients are FP32 sums of the unrounded gradients (k_colsum).
-
-// Dout[m][n] = (sum_k bf16(Din[m][k]) W[k][n]) * (H[m][n] > 0): the gradient at a layer's
-// input (W: K x N bf16, the layer's out x in weights) through the ReLU of the layer below
-// (H: that layer's bf16 output).  As the forward tile: 4 warps x 16 rows per block, W^T
-// staged once per block with a padded stride.  K a multiple of 16, N of 8.
-template <int N, int K>
-__global__ void __launch_bounds__(FWD_WARPS * 32)
-    k_mlp_dgrad(int64_t M, const float* __restrict__ Din, const __nv_bfloat16* __restrict__ W,
-                const __nv_bfloat16* __restrict__ Hm, float* __restrict__ Dout) {
-    pdl_begin();
-    constexpr int LDW = K + 8;
-    __shared__ __align__(16) __nv_bfloat16 sWT[N * LDW];  // sWT[n][k] = W[k][n]
-    for (int idx = threadIdx.x; idx < N * K; idx += blockDim.x) {
-        const int k = idx / N, n = idx - k * N;
-        sWT[n * LDW + k] = W[(int64_t)k * N + n];
-    }
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int64_t r0 = ((int64_t)blockIdx.x * FWD_WARPS + warp) * 16;
-    if (r0 >= M) return;
-    const int64_t ra = r0 + g, rb = r0 + g + 8;
-    const bool va = ra < M, vb = rb < M;
-    float acc[N / 8][4];
-#pragma unroll
-    for (int nt = 0; nt < N / 8; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[nt][e] = 0.f;
-#pragma unroll
-    for (int kk = 0; kk < K; kk += 16) {
-        const uint32_t a0 = va ? load_pair<float>(Din + ra * K + kk + 2 * t) : 0u;
-        const uint32_t a1 = vb ? load_pair<float>(Din + rb * K + kk + 2 * t) : 0u;
-        const uint32_t a2 = va ? load_pair<float>(Din + ra * K + kk + 2 * t + 8) : 0u;
-        const uint32_t a3 = vb ? load_pair<float>(Din + rb * K + kk + 2 * t + 8) : 0u;
-#pragma unroll
-        for (int nt = 0; nt < N / 8; ++nt) {
-            const __nv_bfloat16* wr = sWT + (nt * 8 + g) * LDW + kk + 2 * t;
-            mma_bf16(acc[nt], a0, a1, a2, a3, *reinterpret_cast<const uint32_t*>(wr),
-                     *reinterpret_cast<const uint32_t*>(wr + 8));
-        }
-    }
-#pragma unroll
-    for (int nt = 0; nt < N / 8; ++nt) {
-        const int c = nt * 8 + 2 * t;
-        if (va) {
-            const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(Hm + ra * N + c);
-            *reinterpret_cast<float2*>(Dout + ra * N + c) =
-                make_float2(__low2float(h) > 0.f ? acc[nt][0] : 0.f, __high2float(h) > 0.f ? acc[nt][1] : 0.f);
-        }
-        if (vb) {
-            const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(Hm + rb * N + c);
-            *reinterpret_cast<float2*>(Dout + rb * N + c) =
-                make_float2(__low2float(h) > 0.f ? acc[nt][2] : 0.f, __high2float(h) > 0.f ? acc[nt][3] : 0.f);
-        }
-    }
+// A operand of one k16 step from a 16-row bf16 tile in shared memory (rows of NET_LD2)
+__device__ __forceinline__ void net_lda(uint32_t (&a)[4], const __nv_bfloat16* tile, int k, int lane) {
+    const __nv_bfloat16* p = tile + ((lane & 7) + ((lane >> 3) & 1) * 8) * NET_LD2 + 16 * k + ((lane >> 4) << 3);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
 }
-
-// G[n][k] += sum_m bf16(D[m][n]) X[m][k]: a layer's weight gradient from the gradient at its
-// output (D: M x N FP32) and its input (X: M x K, bf16 activations or the FP32 features,
-// rounded to bf16).  Block (x, y): rows [x WG_ROWS, +WG_ROWS) and the output rows
-// n in [16 y, 16 y + 16).  Rows in chunks of WG_MC; both operands staged transposed in shared
-// memory (row index m contiguous, so each fragment register is one aligned pair), padded
-// so that the fragment loads are free of bank conflicts; the 16 x 8 output tiles of the slab
-// spread over the warps; the block's partial sums go to G with atomics.
-constexpr int WG_MC = 64, WG_WARPS = 4, WG_ROWS = 256;
-template <typename TX, int N, int K>
-__global__ void __launch_bounds__(WG_WARPS * 32)
-    k_mlp_wgrad(int64_t M, const float* __restrict__ D, const TX* __restrict__ X, float* __restrict__ G) {
-    pdl_begin();
-    static_assert(N % 16 == 0 && K % 8 == 0, "tile sizes");
-    constexpr int LDM = WG_MC + 8;                                  // padded row stride (bf16 elements)
-    constexpr int TK = K / 8, TPW = (TK + WG_WARPS - 1) / WG_WARPS;  // output tiles per warp
-    __shared__ __align__(16) __nv_bfloat16 sDT[16 * LDM];           // sDT[n - n0][m - m0]
-    __shared__ __align__(16) __nv_bfloat16 sXT[K * LDM];            // sXT[k][m - m0]
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int n0 = blockIdx.y * 16;
-    const int64_t m_begin = (int64_t)blockIdx.x * WG_ROWS;
-    const int64_t m_end = m_begin + WG_ROWS < M ? m_begin + WG_ROWS : M;
-    float acc[TPW][4];
+// The warp's 32 columns (from c0) of a row tile in the A-operand layout, to the tile in shared
+// memory and to rows ra, rb of a row-major bf16 matrix
+__device__ __forceinline__ void step_put(__nv_bfloat16* tile, __nv_bfloat16* __restrict__ O, const uint32_t (&H)[2][4],
+                                         int c0, int64_t ra, int64_t rb, bool va, bool vb, int g, int t) {
 #pragma unroll
-    for (int q = 0; q < TPW; ++q)
+    for (int k = 0; k < 2; ++k)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc[q][e] = 0.f;
-    for (int64_t m0 = m_begin; m0 < m_end; m0 += WG_MC) {
-        // rows m0 + 2i, m0 + 2i + 1 of D (slab columns) and X, as bf16 pairs along m
-        for (int idx = threadIdx.x; idx < (WG_MC / 2) * 16; idx += blockDim.x) {
-            const int i = idx >> 4, n = idx & 15;
-            const int64_t m = m0 + 2 * i;
-            const float d0 = m < m_end ? D[m * N + n0 + n] : 0.f;
-            const float d1 = m + 1 < m_end ? D[(m + 1) * N + n0 + n] : 0.f;
-            *reinterpret_cast<uint32_t*>(&sDT[n * LDM + 2 * i]) = pack_bf16(d0, d1);
-        }
-        for (int idx = threadIdx.x; idx < (WG_MC / 2) * K; idx += blockDim.x) {
-            const int i = idx / K, k = idx - i * K;
-            const int64_t m = m0 + 2 * i;
-            float x0 = 0.f, x1 = 0.f;
-            if constexpr (sizeof(TX) == 2) {
-                if (m < m_end) x0 = __bfloat162float(X[m * K + k]);
-                if (m + 1 < m_end) x1 = __bfloat162float(X[(m + 1) * K + k]);
-            } else {
-                if (m < m_end) x0 = X[m * K + k];
-                if (m + 1 < m_end) x1 = X[(m + 1) * K + k];
+        for (int e = 0; e < 2; ++e) {
+            const int c = c0 + 16 * k + 8 * e + 2 * t;
+            if (tile) {
+                *reinterpret_cast<uint32_t*>(tile + g * NET_LD2 + c) = H[k][2 * e];
+                *reinterpret_cast<uint32_t*>(tile + (g + 8) * NET_LD2 + c) = H[k][2 * e + 1];
             }
-            *reinterpret_cast<uint32_t*>(&sXT[k * LDM + 2 * i]) = pack_bf16(x0, x1);
+            if (va) *reinterpret_cast<uint32_t*>(O + ra * MLP_H + c) = H[k][2 * e];
+            if (vb) *reinterpret_cast<uint32_t*>(O + rb * MLP_H + c) = H[k][2 * e + 1];
         }
-        __syncthreads();
+}
+// relu(acc + bias) of the warp's 32 columns, rounded
+__device__ __forceinline__ void step_relu(uint32_t (&H)[2][4], const float (&acc)[4][4], const float* bias, int t) {
 #pragma unroll
-        for (int q = 0; q < TPW; ++q) {
-            const int tk = warp + q * WG_WARPS;
-            if (tk < TK) {
+    for (int n = 0; n < 4; ++n) {
+        const float2 bb = *reinterpret_cast<const float2*>(bias + n * 8 + 2 * t);
+        uint32_t* h = H[n >> 1] + 2 * (n & 1);
+        h[0] = pack_bf16(fmaxf(acc[n][0] + bb.x, 0.f), fmaxf(acc[n][1] + bb.y, 0.f));
+        h[1] = pack_bf16(fmaxf(acc[n][2] + bb.x, 0.f), fmaxf(acc[n][3] + bb.y, 0.f));
+    }
+}
+// The gradient through the ReLU mask H > 0 to F (FP32, row-major), rounded into O
+__device__ __forceinline__ void step_mask(uint32_t (&O)[2][4], const float (&acc)[4][4], const uint32_t (&H)[2][4],
+                                          float* __restrict__ F, int c0, int64_t ra, int64_t rb, bool va, bool vb,
+                                          int t) {
 #pragma unroll
-                for (int kk = 0; kk < WG_MC; kk += 16) {
-                    const __nv_bfloat16* ar = sDT + g * LDM + kk + 2 * t;
-                    const __nv_bfloat16* br = sXT + (tk * 8 + g) * LDM + kk + 2 * t;
-                    mma_bf16(acc[q], *reinterpret_cast<const uint32_t*>(ar),
-                             *reinterpret_cast<const uint32_t*>(ar + 8 * LDM), *reinterpret_cast<const uint32_t*>(ar + 8),
-                             *reinterpret_cast<const uint32_t*>(ar + 8 * LDM + 8), *reinterpret_cast<const uint32_t*>(br),
-                             *reinterpret_cast<const uint32_t*>(br + 8));
+    for (int n = 0; n < 4; ++n) {
+        const int k = n >> 1, e = 2 * (n & 1), c = c0 + 8 * n + 2 * t;
+        const __nv_bfloat162 ha = *reinterpret_cast<const __nv_bfloat162*>(&H[k][e]);
+        const __nv_bfloat162 hb = *reinterpret_cast<const __nv_bfloat162*>(&H[k][e + 1]);
+        const float v0 = __low2float(ha) > 0.f ? acc[n][0] : 0.f, v1 = __high2float(ha) > 0.f ? acc[n][1] : 0.f;
+        const float v2 = __low2float(hb) > 0.f ? acc[n][2] : 0.f, v3 = __high2float(hb) > 0.f ? acc[n][3] : 0.f;
+        O[k][e] = pack_bf16(v0, v1);
+        O[k][e + 1] = pack_bf16(v2, v3);
+        if (va) *reinterpret_cast<float2*>(F + ra * MLP_H + c) = make_float2(v0, v1);
+        if (vb) *reinterpret_cast<float2*>(F + rb * MLP_H + c) = make_float2(v2, v3);
+    }
+}
+
+// Forward, loss (sum mask (Y - T)^2 / M added to *loss; mask = the features' slot-valid flags) and
+// input gradients of M rows.
+//
+// Four warps share a row tile, 32 columns of every layer each, and pass the tile on through shared
+// memory: a batch of 4096 rows has only 256 tiles, and one warp through all the products of a
+// tile took 13 us of dependent instructions.  `early`: X was complete before the preceding kernel
+// began, so the first feature tile is fetched while that one still runs.
+constexpr int STEP_GROUPS = 2, STEP_WARPS = 4 * STEP_GROUPS;
+struct StepOut {
+    __nv_bfloat16 *H1, *H2, *D1, *D2, *D3;  // activations and rounded gradients, M x 128 (D3: M x 16)
+    float *F1, *F2, *F3;                    // the gradients unrounded
+    float* G;                               // the flat gradient
+    double* loss;
+};
+struct StepSmem {
+    NetSmem net;
+    float x[STEP_GROUPS][16 * NET_LDX];            // feature tiles
+    __nv_bfloat16 h[STEP_GROUPS][2][16 * NET_LD2];  // H1 then D2, and H2
+};
+__device__ __forceinline__ void step_sync(int group) {
+    asm volatile("bar.sync %0, 128;" ::"r"(group + 1) : "memory");
+}
+// net_fetch by the four warps of a group
+__device__ __forceinline__ void step_fetch(float* buf, const float* __restrict__ X, int64_t r0, int64_t M, bool wide,
+                                           int w, int lane) {
+    if (r0 + 4 * w < M) net_fetch<4>(buf + 4 * w * NET_LDX, X, r0 + 4 * w, M, wide, lane);
+}
+__global__ void __launch_bounds__(STEP_WARPS * 32)
+    k_mlp_step(int64_t M, const float* __restrict__ X, const float* __restrict__ Tg, const __nv_bfloat16* __restrict__ Wb,
+               const float* __restrict__ P, const StepOut out, bool early) {
+    extern __shared__ __align__(16) unsigned char net_raw[];
+    StepSmem& sm = *reinterpret_cast<StepSmem*>(net_raw);
+    __shared__ double s_loss[STEP_GROUPS];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int group = warp >> 2, w = warp & 3, c0 = 32 * w;
+    float* buf = sm.x[group];
+    __nv_bfloat16 *h1t = sm.h[group][0], *h2t = sm.h[group][1];
+    const int64_t tiles = (M + 15) / 16, step = (int64_t)gridDim.x * STEP_GROUPS;
+    const bool wide = (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    int64_t q = blockIdx.x + (int64_t)gridDim.x * group;
+    if (early && q < tiles) step_fetch(buf, X, q * 16, M, wide, w, lane);
+    pdl_begin();
+    if (!early && q < tiles) step_fetch(buf, X, q * 16, M, wide, w, lane);
+    net_stage_weights<STEP_WARPS * 32>(sm.net, Wb, P);
+    double l = 0.0;
+    const float fm = (float)M;
+    for (; q < tiles; q += step) {
+        const int64_t ra = q * 16 + g, rb = ra + 8;
+        const bool va = ra < M, vb = rb < M;
+        float tg[2][4];  // targets of this lane's eight outputs (they may be only 4-byte aligned)
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int c = n * 8 + 2 * t + (e & 1);
+                tg[n][e] = (e < 2 ? va : vb) ? Tg[(e < 2 ? ra : rb) * MLP_S + c] : 0.f;
+            }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        step_sync(group);
+        uint32_t H1[2][4], H2[2][4], D[2][4];
+        unsigned on = 0u;  // slot-valid flags of this lane's eight outputs
+        float acc[4][4];
+        {
+            uint32_t A[MLP_F / 16][4];
+            net_inputs(A, buf, va, vb, g, t);
+#pragma unroll
+            for (int n = 0; n < 2; ++n)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float* f = buf + g * NET_LDX + MLP_NF_SLOT * (n * 8 + 2 * t + e);
+                    if (va && f[0] > 0.f) on |= 1u << (4 * n + e);
+                    if (vb && f[8 * NET_LDX] > 0.f) on |= 1u << (4 * n + 2 + e);
+                }
+            net_product<4, MLP_F / 16, NET_LD1>(acc, A, sm.net.w1 + c0 * NET_LD1, lane);
+        }
+        step_relu(H1, acc, sm.net.b1 + c0, t);
+        step_put(h1t, out.H1, H1, c0, ra, rb, va, vb, g, t);
+        step_sync(group);  // H1 is whole; the feature tile has been read and takes the next one
+        if (q + step < tiles) step_fetch(buf, X, (q + step) * 16, M, wide, w, lane);
+        uint32_t A[MLP_H / 16][4];
+#pragma unroll
+        for (int k = 0; k < MLP_H / 16; ++k) net_lda(A[k], h1t, k, lane);
+        net_product<4, MLP_H / 16, NET_LD2>(acc, A, sm.net.w2 + c0 * NET_LD2, lane);
+        step_relu(H2, acc, sm.net.b2 + c0, t);
+        step_put(h2t, out.H2, H2, c0, ra, rb, va, vb, g, t);
+        step_sync(group);
+#pragma unroll
+        for (int k = 0; k < MLP_H / 16; ++k) net_lda(A[k], h2t, k, lane);
+        float y[2][4];  // every warp forms all 16 outputs and their gradients
+        net_product<2, MLP_H / 16, NET_LD2>(y, A, sm.net.w3, lane);
+        uint32_t D3[4];
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            const float2 bb = *reinterpret_cast<const float2*>(sm.net.b3 + n * 8 + 2 * t);
+            float d[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float mask = (on >> (4 * n + e)) & 1u ? 1.f : 0.f;
+                const float r = (e < 2 ? va : vb) ? mask * (y[n][e] + (e & 1 ? bb.y : bb.x) - tg[n][e]) : 0.f;
+                if (w == 0) l += (double)r * (double)r;
+                d[e] = 2.f * r / fm;
+            }
+            D3[2 * n] = pack_bf16(d[0], d[1]);
+            D3[2 * n + 1] = pack_bf16(d[2], d[3]);
+            if (w == 0) {
+                const int c = n * 8 + 2 * t;
+                if (va) {
+                    *reinterpret_cast<uint32_t*>(out.D3 + ra * MLP_S + c) = D3[2 * n];
+                    *reinterpret_cast<float2*>(out.F3 + ra * MLP_S + c) = make_float2(d[0], d[1]);
+                }
+                if (vb) {
+                    *reinterpret_cast<uint32_t*>(out.D3 + rb * MLP_S + c) = D3[2 * n + 1];
+                    *reinterpret_cast<float2*>(out.F3 + rb * MLP_S + c) = make_float2(d[2], d[3]);
                 }
             }
         }
-        __syncthreads();
-    }
+        // D2 = D3 W3 through H2's mask, D1 = D2 W2 through H1's
 #pragma unroll
-    for (int q = 0; q < TPW; ++q) {
-        const int tk = warp + q * WG_WARPS;
-        if (tk < TK) {
-            const int k = tk * 8 + 2 * t;
-            float* gr = G + (int64_t)(n0 + g) * K + k;
-            atomicAdd(gr, acc[q][0]);
-            atomicAdd(gr + 1, acc[q][1]);
-            atomicAdd(gr + 8 * K, acc[q][2]);
-            atomicAdd(gr + 8 * K + 1, acc[q][3]);
+        for (int n = 0; n < 4; n += 2) {
+            uint32_t b[4];
+            net_ldb_t<NET_LD2>(b, sm.net.w3 + c0 + n * 8, lane);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[n][e] = acc[n + 1][e] = 0.f;
+            mma_bf16(acc[n], D3[0], D3[1], D3[2], D3[3], b[0], b[1]);
+            mma_bf16(acc[n + 1], D3[0], D3[1], D3[2], D3[3], b[2], b[3]);
         }
-    }
-}
-
-// g[n] += sum_m D[m][n]
-__global__ void k_colsum(int64_t M, int N, const float* __restrict__ D, float* __restrict__ g) {
-    pdl_begin();
-    const int n = blockIdx.x;
-    float s = 0.f;
-    for (int64_t m = threadIdx.x; m < M; m += blockDim.x) s += D[m * N + n];
+        step_mask(D, acc, H2, out.F2, c0, ra, rb, va, vb, t);
+        step_put(h1t, out.D2, D, c0, ra, rb, va, vb, g, t);  // over H1: every warp has read it
+        step_sync(group);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    __shared__ float red[8];
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+        for (int k = 0; k < MLP_H / 16; ++k) net_lda(A[k], h1t, k, lane);
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[n][e] = 0.f;
+#pragma unroll
+        for (int k = 0; k < MLP_H / 16; ++k)
+#pragma unroll
+            for (int n = 0; n < 4; n += 2) {
+                uint32_t b[4];
+                net_ldb_t<NET_LD2>(b, sm.net.w2 + k * 16 * NET_LD2 + c0 + n * 8, lane);
+                mma_bf16(acc[n], A[k][0], A[k][1], A[k][2], A[k][3], b[0], b[1]);
+                mma_bf16(acc[n + 1], A[k][0], A[k][1], A[k][2], A[k][3], b[2], b[3]);
+            }
+        step_mask(D, acc, H1, out.F1, c0, ra, rb, va, vb, t);
+        step_put(nullptr, out.D1, D, c0, ra, rb, va, vb, g, t);
+        // the next tile's H1 goes over D2 after the barrier at its start
+    }
+    if (w == 0) {
+        l = warp_sum(l);
+        if (lane == 0) s_loss[group] = l;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
-        float tot = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-        g[n] += tot;
+        double v = 0.0;
+        for (int i = 0; i < STEP_GROUPS; ++i) v += s_loss[i];
+        atomicAdd(out.loss, v / (double)M);
     }
 }
 
-// Adam (bias-corrected), then the bf16 copy of the weights.
-__global__ void k_adam(float* __restrict__ P, const float* __restrict__ G, float* __restrict__ Mo,
+// Weight and bias gradients of all layers in one launch.  Weights: G[n][k] += sum_m D[m][n] X[m][k]
+// (D: the rounded gradient at the layer's output, X: its input, features rounded here), block (x, y)
+// taking rows [x rows, +rows) and, by y, a slab of 32 outputs of layer 2 (y = 0..3) or 1 (4..7), or
+// layer 3 (8).  Both operands are staged row-major in shared memory, WG_MC rows at a time, and
+// ldmatrix transposes them into fragments (the products run along the rows).  A chain of products
+// covers WG_MC rows and its FP32 sums are then added up in registers: the tensor pipe's own sums
+// truncate, and chains of 2304 rows showed it (2.5e-6 of a gradient against 3e-7).  The block's sums
+// go to G in pairs with atomics.  Biases (y >= 9): the column sums of the unrounded gradients.
+constexpr int WG_MC = 256, WG_WARPS = 8, WG_WJOBS = 9, WG_JOBS = WG_WJOBS + 3;
+constexpr int WG_LDD = 32 + 8, WG_LDX = MLP_H + 8;
+constexpr size_t WG_SMEM = sizeof(__nv_bfloat16) * WG_MC * (WG_LDD + WG_LDX);
+
+__device__ __forceinline__ void ldmatrix_t(uint32_t (&f)[4], const __nv_bfloat16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+// cnt rows of C columns (a multiple of 8, from column c0 of LDG) into rows of LDS; zeros to WG_MC rows
+template <int C, int LDG, int LDS>
+__device__ __forceinline__ void wg_stage(__nv_bfloat16* s, const __nv_bfloat16* __restrict__ src, int c0, int64_t m0,
+                                         int cnt) {
+    constexpr int Q = C / 8;
+#pragma unroll
+    for (int e = threadIdx.x; e < WG_MC * Q; e += WG_WARPS * 32) {
+        const int r = e / Q, c = 8 * (e - r * Q);
+        if (r < cnt)
+            net_cp16(s + r * LDS + c, src + (m0 + r) * LDG + c0 + c);
+        else
+            *reinterpret_cast<uint4*>(s + r * LDS + c) = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+// the warp's tile of MT m16 (all of the slab) x 2 n8 outputs, k columns from kc
+template <int MT>
+__device__ __forceinline__ void wg_tile(const __nv_bfloat16* sD, const __nv_bfloat16* sX, int kc, int lane,
+                                        float (&sum)[2][2][4]) {
+    const int r = lane & 7, s1 = (lane >> 3) & 1, s2 = lane >> 4;
+    float acc[MT][2][4];
+#pragma unroll
+    for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[i][n][e] = 0.f;
+#pragma unroll 4
+    for (int mm = 0; mm < WG_MC; mm += 16) {
+        uint32_t b[4];
+        ldmatrix_t(b, sX + (mm + r + 8 * s1) * WG_LDX + kc + 8 * s2);
+#pragma unroll
+        for (int i = 0; i < MT; ++i) {
+            uint32_t a[4];
+            ldmatrix_t(a, sD + (mm + r + 8 * s2) * WG_LDD + 16 * i + 8 * s1);
+            mma_bf16(acc[i][0], a[0], a[1], a[2], a[3], b[0], b[1]);
+            mma_bf16(acc[i][1], a[0], a[1], a[2], a[3], b[2], b[3]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) sum[i][n][e] += acc[i][n][e];
+}
+__device__ __forceinline__ void wg_red2(float* p, float x, float y) {
+    asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(x), "f"(y) : "memory");
+}
+// G[n] = sum_m D[m][n] for the eight columns from n0, by the block: 256 partial sums over the rows
+// r, r + 256, ..., a butterfly over each 32 of them, then the eight in order
+__device__ __forceinline__ void wg_colsum8(float* s, int64_t M, int N, int n0, const float* __restrict__ D,
+                                           float* __restrict__ G) {
+    const int r = threadIdx.x >> 3, c = threadIdx.x & 7, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = 0.f;
+    const float* p = D + n0 + c;
+    int64_t m0 = 0;
+#pragma unroll 2
+    for (; m0 + 256 <= M; m0 += 256)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] += p[(m0 + 32 * k + r) * N];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        if (m0 + 32 * k + r < M) v[k] += p[(m0 + 32 * k + r) * N];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s[(k * 8 + c) * 33 + r] = v[k];
+    __syncthreads();
+    float mine = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {  // the warp adds up its 32 partial sums of column q
+        float x = s[(warp * 8 + q) * 33 + lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == q) mine = x;
+    }
+    __syncthreads();
+    if (lane < 8) s[warp * 8 + lane] = mine;
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        float tot = 0.f;
+        for (int w = 0; w < 8; ++w) tot += s[w * 8 + threadIdx.x];
+        G[n0 + threadIdx.x] = tot;
+    }
+    __syncthreads();
+}
+__global__ void __launch_bounds__(WG_WARPS * 32, 2)
+    k_mlp_wgrad(int64_t M, int64_t rows, const float* __restrict__ X, const StepOut in) {
+    pdl_begin();
+    extern __shared__ __align__(16) unsigned char wg_raw[];
+    const int job = blockIdx.y;
+    if (job >= WG_WJOBS) {
+        constexpr int NG = (2 * MLP_H + MLP_S) / 8;
+        for (int q = (job - WG_WJOBS) * gridDim.x + blockIdx.x; q < NG; q += (WG_JOBS - WG_WJOBS) * gridDim.x) {
+            float* s = reinterpret_cast<float*>(wg_raw);
+            if (q < MLP_H / 8)
+                wg_colsum8(s, M, MLP_H, 8 * q, in.F1, in.G + OFF_B1);
+            else if (q < 2 * MLP_H / 8)
+                wg_colsum8(s, M, MLP_H, 8 * q - MLP_H, in.F2, in.G + OFF_B2);
+            else
+                wg_colsum8(s, M, MLP_S, 8 * q - 2 * MLP_H, in.F3, in.G + OFF_B3);
+        }
+        return;
+    }
+    __nv_bfloat16* sD = reinterpret_cast<__nv_bfloat16*>(wg_raw);
+    __nv_bfloat16* sX = sD + WG_MC * WG_LDD;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, kc = 16 * warp;
+    const int64_t m_begin = (int64_t)blockIdx.x * rows;
+    const int64_t m_end = m_begin + rows < M ? m_begin + rows : M;
+    const int K = job >= 4 && job < 8 ? MLP_F : MLP_H;
+    float sum[2][2][4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) sum[i][n][e] = 0.f;
+    for (int64_t m0 = m_begin; m0 < m_end; m0 += WG_MC) {
+        const int cnt = (int)(m_end - m0 < WG_MC ? m_end - m0 : WG_MC);
+        if (job < 4) {
+            wg_stage<32, MLP_H, WG_LDD>(sD, in.D2, 32 * job, m0, cnt);
+            wg_stage<MLP_H, MLP_H, WG_LDX>(sX, in.H1, 0, m0, cnt);
+        } else if (job < 8) {
+            wg_stage<32, MLP_H, WG_LDD>(sD, in.D1, 32 * (job - 4), m0, cnt);
+            constexpr int Q = MLP_F / 2;
+#pragma unroll 14
+            for (int e = threadIdx.x; e < WG_MC * Q; e += WG_WARPS * 32) {
+                const int r = e / Q, c = 2 * (e - r * Q);
+                *reinterpret_cast<uint32_t*>(sX + r * WG_LDX + c) = r < cnt ? load_pair(X + (m0 + r) * MLP_F + c) : 0u;
+            }
+        } else {
+            wg_stage<MLP_S, MLP_S, WG_LDD>(sD, in.D3, 0, m0, cnt);
+            wg_stage<MLP_H, MLP_H, WG_LDX>(sX, in.H2, 0, m0, cnt);
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        if (kc < K) {
+            if (job < 8)
+                wg_tile<2>(sD, sX, kc, lane, sum);
+            else
+                wg_tile<1>(sD, sX, kc, lane, sum);
+        }
+        __syncthreads();
+    }
+    if (kc >= K) return;
+    float* G = in.G + (job < 4 ? OFF_W2 + (int64_t)32 * job * MLP_H : job < 8 ? OFF_W1 + (int64_t)32 * (job - 4) * MLP_F : OFF_W3);
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+        if (i == 0 || job < 8)
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                float* p = G + (16 * i + g) * K + kc + 8 * n + 2 * t;
+                wg_red2(p, sum[i][n][0], sum[i][n][1]);
+                wg_red2(p + 8 * K, sum[i][n][2], sum[i][n][3]);
+            }
+}
+
+// Adam (bias-corrected), then the bf16 copy of the weights; G is cleared for the next batch.
+__global__ void k_adam(float* __restrict__ P, float* __restrict__ G, float* __restrict__ Mo,
                        float* __restrict__ Vo, __nv_bfloat16* __restrict__ Wb, float lr, float c1, float c2) {
     pdl_begin();
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= NPARAM) return;
     const float g = G[q];
+    G[q] = 0.f;
     const float m = 0.9f * Mo[q] + 0.1f * g;
     const float v = 0.999f * Vo[q] + 0.001f * g * g;
     Mo[q] = m;
@@ -544,6 +721,7 @@ Model* mlp_create(uint64_t seed, cudaStream_t s) {
     m->Mo.alloc(NPARAM);
     m->Vo.alloc(NPARAM);
     m->Wb.alloc(NBF);
+    BAMG_CK(cudaMemsetAsync(m->Wb.get(), 0, sizeof(__nv_bfloat16) * NBF, s));  // the rows' padding
     BAMG_LAUNCH(k_mlp_init, blocks_for(NPARAM, 256), 256, 0, s, seed, m->P.get());
     BAMG_LAUNCH(k_mlp_to_bf16, blocks_for(NPARAM, 256), 256, 0, s, m->P.get(), m->Wb.get());
     BAMG_CK(cudaMemsetAsync(m->Mo.get(), 0, sizeof(float) * NPARAM, s));
@@ -564,88 +742,74 @@ void mlp_get(const Model* m, float* h_params, cudaStream_t s) {
     BAMG_CK(cudaStreamSynchronize(s));
 }
 
-// Activations of one batch of rows.
+// Activations and gradients (rounded and not) of one batch of rows, and the loss sum.
 struct MlpWork {
-    DevBuf<__nv_bfloat16> H1, H2;
-    DevBuf<float> Y, dY, D2, D1;
+    DevBuf<__nv_bfloat16> H1, H2, D1, D2, D3;
+    DevBuf<float> F1, F2, F3;
     DevBuf<double> loss;
-    void ensure(int64_t rows, bool train) {
-        H1.ensure(rows * MLP_H);
-        H2.ensure(rows * MLP_H);
-        Y.ensure(rows * MLP_S);
-        if (train) {
-            dY.ensure(rows * MLP_S);
-            D2.ensure(rows * MLP_H);
-            D1.ensure(rows * MLP_H);
-            loss.ensure(1);
-        }
+    explicit MlpWork(int64_t rows) {
+        H1.alloc(rows * MLP_H);
+        H2.alloc(rows * MLP_H);
+        D1.alloc(rows * MLP_H);
+        D2.alloc(rows * MLP_H);
+        D3.alloc(rows * MLP_S);
+        F1.alloc(rows * MLP_H);
+        F2.alloc(rows * MLP_H);
+        F3.alloc(rows * MLP_S);
+        loss.alloc(1);
     }
 };
 
-static void forward_rows(const Model* m, int64_t rows, const float* feat, MlpWork& w, float* Y, cudaStream_t s) {
-    const unsigned g = blocks_for(rows, FWD_WARPS * 16);
-    const float* P = m->P.get();
-    const __nv_bfloat16* Wb = m->Wb.get();
-    BAMG_LAUNCH((k_mlp_layer<float, MLP_H, MLP_F>), g, FWD_WARPS * 32, 0, s, rows, feat, Wb + BOFF_W1, P + OFF_B1, true,
-                w.H1.get(), (float*)nullptr);
-    BAMG_LAUNCH((k_mlp_layer<__nv_bfloat16, MLP_H, MLP_H>), g, FWD_WARPS * 32, 0, s, rows,
-                (const __nv_bfloat16*)w.H1.get(), Wb + BOFF_W2, P + OFF_B2, true, w.H2.get(), (float*)nullptr);
-    BAMG_LAUNCH((k_mlp_layer<__nv_bfloat16, MLP_S, MLP_H>), g, FWD_WARPS * 32, 0, s, rows,
-                (const __nv_bfloat16*)w.H2.get(), Wb + BOFF_W3, P + OFF_B3, false, (__nv_bfloat16*)nullptr, Y);
-}
-
-void mlp_forward(const Model* m, int64_t rows, const float* feat, float* Y, cudaStream_t s) {
-    if (rows <= 0) return;
-    constexpr size_t smem = sizeof(NetSmem) + sizeof(float) * NET_WARPS * 16 * NET_LDX;
-    static_assert(smem <= 227 * 1024, "weights and feature tiles in shared memory");
-    static std::atomic<bool> allowed[256] = {};  // more than 48 KB: once per device (idempotent across threads)
+// Dynamic shared memory beyond 48 KB for a kernel, allowed once per device (idempotent across
+// threads); returns the device's SM count.
+template <typename K>
+static int net_device(K kernel, size_t smem, std::atomic<bool> (&allowed)[256]) {
     int dev = 0, nsm = 0;
     BAMG_CK(cudaGetDevice(&dev));
     BAMG_REQUIRE(dev >= 0 && dev < 256, BAMG_EINVAL, "device ordinal out of range");
     if (!allowed[dev]) {
-        BAMG_CK(cudaFuncSetAttribute(k_mlp_net, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        BAMG_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         allowed[dev] = true;
     }
     BAMG_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const unsigned grid = (unsigned)std::min<int64_t>(nsm > 0 ? nsm : 1, (rows + 15) / 16);
-    BAMG_LAUNCH(k_mlp_net, grid, NET_WARPS * 32, smem, s, rows, feat, (const __nv_bfloat16*)m->Wb.get(),
-                (const float*)m->P.get(), Y);
+    return nsm > 0 ? nsm : 1;
+}
+// k_mlp_net: weights and one feature tile a warp
+constexpr size_t NET_BYTES = sizeof(NetSmem) + sizeof(float) * NET_WARPS * 16 * NET_LDX;
+static_assert(NET_BYTES <= 227 * 1024, "shared memory");
+
+void mlp_forward(const Model* m, int64_t rows, const float* feat, float* Y, cudaStream_t s) {
+    if (rows <= 0) return;
+    static std::atomic<bool> allowed[256] = {};
+    const int nsm = net_device(k_mlp_net, NET_BYTES, allowed);
+    BAMG_LAUNCH(k_mlp_net, (unsigned)std::min<int64_t>(nsm, (rows + 15) / 16), NET_WARPS * 32, NET_BYTES, s, rows,
+                feat, (const __nv_bfloat16*)m->Wb.get(), (const float*)m->P.get(), Y);
 }
 
-// Gradients of the batch loss into m->G (zeroed first); the loss sum into w.loss.
-static void gradients(Model* m, int64_t rows, const float* feat, const float* target, MlpWork& w, cudaStream_t s) {
-    forward_rows(m, rows, feat, w, w.Y.get(), s);
-    float* G = m->G.get();
-    const __nv_bfloat16* Wb = m->Wb.get();
-    BAMG_CK(cudaMemsetAsync(G, 0, sizeof(float) * NPARAM, s));
-    BAMG_LAUNCH(k_mlp_loss, blocks_for(rows * MLP_S, 256), 256, 0, s, rows, rows, w.Y.get(), target, feat, w.dY.get(),
-                w.loss.get());
-    const unsigned zb = (unsigned)((rows + WG_ROWS - 1) / WG_ROWS), gd = blocks_for(rows, FWD_WARPS * 16);
-    // layer 3
-    BAMG_LAUNCH((k_mlp_wgrad<__nv_bfloat16, MLP_S, MLP_H>), dim3(zb, MLP_S / 16), WG_WARPS * 32, 0, s, rows,
-                (const float*)w.dY.get(), (const __nv_bfloat16*)w.H2.get(), G + OFF_W3);
-    BAMG_LAUNCH(k_colsum, MLP_S, 256, 0, s, rows, MLP_S, (const float*)w.dY.get(), G + OFF_B3);
-    BAMG_LAUNCH((k_mlp_dgrad<MLP_H, MLP_S>), gd, FWD_WARPS * 32, 0, s, rows, (const float*)w.dY.get(),
-                Wb + BOFF_W3, (const __nv_bfloat16*)w.H2.get(), w.D2.get());
-    // layer 2
-    BAMG_LAUNCH((k_mlp_wgrad<__nv_bfloat16, MLP_H, MLP_H>), dim3(zb, MLP_H / 16), WG_WARPS * 32, 0, s, rows,
-                (const float*)w.D2.get(), (const __nv_bfloat16*)w.H1.get(), G + OFF_W2);
-    BAMG_LAUNCH(k_colsum, MLP_H, 256, 0, s, rows, MLP_H, (const float*)w.D2.get(), G + OFF_B2);
-    BAMG_LAUNCH((k_mlp_dgrad<MLP_H, MLP_H>), gd, FWD_WARPS * 32, 0, s, rows, (const float*)w.D2.get(),
-                Wb + BOFF_W2, (const __nv_bfloat16*)w.H1.get(), w.D1.get());
-    // layer 1
-    BAMG_LAUNCH((k_mlp_wgrad<float, MLP_H, MLP_F>), dim3(zb, MLP_H / 16), WG_WARPS * 32, 0, s, rows,
-                (const float*)w.D1.get(), feat, G + OFF_W1);
-    BAMG_LAUNCH(k_colsum, MLP_H, 256, 0, s, rows, MLP_H, (const float*)w.D1.get(), G + OFF_B1);
+// Gradients of the batch loss added to m->G; the loss sum into w.loss.
+static void gradients(Model* m, int64_t rows, const float* feat, const float* target, MlpWork& w, bool early,
+                      cudaStream_t s) {
+    static std::atomic<bool> allowed[256] = {}, allowed_w[256] = {};
+    const int nsm = net_device(k_mlp_step, sizeof(StepSmem), allowed);
+    net_device(k_mlp_wgrad, WG_SMEM, allowed_w);
+    const StepOut out{w.H1.get(), w.H2.get(), w.D1.get(), w.D2.get(), w.D3.get(),
+                      w.F1.get(), w.F2.get(), w.F3.get(), m->G.get(), w.loss.get()};
+    BAMG_LAUNCH(k_mlp_step, (unsigned)std::min<int64_t>(nsm, (rows + 15) / 16), STEP_WARPS * 32, sizeof(StepSmem), s,
+                rows, feat, target, (const __nv_bfloat16*)m->Wb.get(), (const float*)m->P.get(), out, early);
+    // up to two blocks per SM over the jobs, in whole chunks of rows
+    const int64_t chunks = (rows + WG_MC - 1) / WG_MC, per = (chunks * WG_JOBS + 2 * nsm - 1) / (2 * nsm);
+    const int64_t br = per * WG_MC;
+    BAMG_LAUNCH(k_mlp_wgrad, dim3((unsigned)((rows + br - 1) / br), WG_JOBS), WG_WARPS * 32, WG_SMEM, s, rows, br, feat,
+                out);
 }
 
 double mlp_gradients(Model* m, int64_t rows, const float* feat, const float* target, float* h_grad, cudaStream_t s) {
     BAMG_REQUIRE(rows > 0, BAMG_EINVAL, "mlp_gradients: no rows");
     AllocStream as_(s);
-    MlpWork w;
-    w.ensure(rows, true);
+    MlpWork w(rows);
     BAMG_CK(cudaMemsetAsync(w.loss.get(), 0, sizeof(double), s));
-    gradients(m, rows, feat, target, w, s);
+    BAMG_CK(cudaMemsetAsync(m->G.get(), 0, sizeof(float) * NPARAM, s));
+    gradients(m, rows, feat, target, w, false, s);
     double l = 0.0;
     BAMG_CK(cudaMemcpyAsync(&l, w.loss.get(), sizeof(double), cudaMemcpyDeviceToHost, s));
     if (h_grad) BAMG_CK(cudaMemcpyAsync(h_grad, m->G.get(), sizeof(float) * NPARAM, cudaMemcpyDeviceToHost, s));
@@ -657,17 +821,17 @@ void mlp_train(Model* m, int64_t rows, const float* feat, const float* target, i
                double* h_loss, cudaStream_t s) {
     BAMG_REQUIRE(rows > 0 && epochs >= 0 && batch > 0, BAMG_EINVAL, "mlp_train: bad sizes");
     AllocStream as_(s);
-    MlpWork w;
-    w.ensure(std::min<int64_t>(rows, batch), true);
+    MlpWork w(std::min<int64_t>(rows, batch));
+    BAMG_CK(cudaMemsetAsync(m->G.get(), 0, sizeof(float) * NPARAM, s));
     for (int e = 0; e < epochs; ++e) {
         BAMG_CK(cudaMemsetAsync(w.loss.get(), 0, sizeof(double), s));
         int64_t nb = 0;
         for (int64_t r0 = 0; r0 < rows; r0 += batch, ++nb) {
             const int64_t br = std::min<int64_t>(batch, rows - r0);
-            gradients(m, br, feat + r0 * MLP_F, target + r0 * MLP_S, w, s);
+            gradients(m, br, feat + r0 * MLP_F, target + r0 * MLP_S, w, e > 0 || r0 > 0, s);
             m->t += 1;
             const float c1 = (float)(1.0 - std::pow(0.9, m->t)), c2 = (float)(1.0 - std::pow(0.999, m->t));
-            BAMG_LAUNCH(k_adam, blocks_for(NPARAM, 256), 256, 0, s, m->P.get(), (const float*)m->G.get(),
+            BAMG_LAUNCH(k_adam, blocks_for(NPARAM, 256), 256, 0, s, m->P.get(), m->G.get(),
                         m->Mo.get(), m->Vo.get(), m->Wb.get(), (float)lr, c1, c2);
         }
         if (h_loss) {

@@ -54,3 +54,25 @@ def test_forward_at_tile_edges(rows):
     err = np.abs(alone.cpu().numpy() - y_o)
     scale = max(1.0, np.abs(y_o).max())
     assert err.max() <= 1e-2 * scale and err.mean() <= 1e-4 * scale
+
+
+@pytest.mark.parametrize("rows", [1, 16, 17, 127, 129, 16 * 152 + 3, 16 * 152 * 8 + 5])
+def test_gradients_at_tile_edges(rows):
+    """Loss and gradients against the oracle with the same roundings.  A bf16 rounding that falls the
+    other way moves an entry by at most 2^-8 of itself, so each gradient by at most 2^-8 of its norm;
+    the targets lie at an odd 4-byte address."""
+    torch, m, p, f = _network(rows, seed=rows)
+    T = np.random.default_rng(1).standard_normal((rows, 16)).astype(np.float32) * 0.3
+    Td = torch.empty(rows * 16 + 1, dtype=torch.float32, device="cuda")[1:].view(rows, 16)
+    Td.copy_(torch.tensor(T))
+    g, loss = m.gradients(torch.tensor(f, device="cuda"), Td)
+    f64 = f.astype(np.float64)
+    y, cache = ol.forward(p, f64, use_bf16=True)
+    mask = ol.slot_mask(f64)
+    g_o = ol.backward(p, cache, y, T.astype(np.float64), mask, bf16_grads=True)
+    assert loss == pytest.approx(ol.loss(y, T, mask), rel=1e-3)
+    at = 0
+    for k in ("W1", "b1", "W2", "b2", "W3", "b3"):
+        part = g[at:at + g_o[k].size].reshape(g_o[k].shape)
+        at += g_o[k].size
+        assert np.linalg.norm(part - g_o[k]) <= 2.0 ** -8 * max(np.linalg.norm(g_o[k]), 1e-30), k
