@@ -1325,6 +1325,16 @@ int arn_tile_rows(int n) {
 }
 int arn_tiles(int n) { return (int)blocks_for(n, arn_tile_rows(n)); }
 
+// warp_sum of x in lanes 0..15 and of y in lanes 16..31, by the same tree as warp_sum: the first
+// exchange leaves each half of the warp with one of the two
+__device__ __forceinline__ double warp_sum2(double x, double y, int lane) {
+    const bool up = (lane & 16) != 0;
+    double keep = up ? y : x;
+    keep += __shfl_xor_sync(0xffffffffu, up ? x : y, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) keep += __shfl_xor_sync(0xffffffffu, keep, o);
+    return keep;
+}
 __device__ __forceinline__ double arn_colsum(const double* __restrict__ P, int nb, int stride, int q, int lane) {
     double s = 0.0;
     for (int b = lane; b < nb; b += 32) s += P[(int64_t)b * stride + q];
@@ -1344,36 +1354,68 @@ __device__ __forceinline__ void arn_last_block_sums(const double* P, int nb, int
     if (!s_last) return;
     __threadfence();
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int q = wid; q < ncol; q += nw) {
-        double s = 0.0;
-        for (int b = lane; b < nb; b += 32) s += __ldcg(P + (int64_t)b * stride + q);
-        s = warp_sum(s);
-        if (lane == 0) tot[q] = s;
+    for (int q = 2 * wid; q < ncol; q += 2 * nw) {
+        const double* p = P + q;
+        double x = 0.0, y = 0.0;
+        if (q + 1 < ncol) {
+#pragma unroll 4
+            for (int b = lane; b < nb; b += 32) {
+                x += __ldcg(p + (int64_t)b * stride);
+                y += __ldcg(p + (int64_t)b * stride + 1);
+            }
+        } else {
+#pragma unroll 8
+            for (int b = lane; b < nb; b += 32) x += __ldcg(p + (int64_t)b * stride);
+        }
+        x = warp_sum2(x, y, lane);
+        if ((lane & 15) == 0 && q + (lane >> 4) < ncol) tot[q + (lane >> 4)] = x;
     }
     if (threadIdx.x == 0) *cnt = 0u;
 }
-// per-tile dots of the tile's rows of w with V[0..j] (self = 0) or with itself; the block
-// has just written w, so these reads hit the caches.  Each writing lane fences after its last
-// partial (arn_last_block_sums reads them from another block).
+// per-tile dots of the tile's rows of w (wt: at the tile's first row) with V[0..j] (self = 0) or with
+// itself.  A warp takes two columns at a time: their sums share the exchanges, and GB300's FP64
+// pipe (a warp's operation every 16 cycles) does half the additions of the butterflies.  Each
+// writing lane fences after its last partial (arn_last_block_sums reads them from another block).
 __device__ __forceinline__ void arn_tile_dots(const double* __restrict__ V, int n, int j, int r0, int cnt,
-                                              const double* w, int self, double* __restrict__ Pout, int stride) {
+                                              const double* wt, int self, double* __restrict__ Pout, int stride) {
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const int nv = self ? 1 : j + 1;
-    const double* wt = w + r0;
-    for (int q = wid; q < nv; q += nw) {
-        const double* vq = self ? wt : V + (int64_t)q * n + r0;
-        double acc = 0.0;
-#pragma unroll 4
-        for (int e = lane; e < cnt; e += 32) acc += vq[e] * wt[e];
-        acc = warp_sum(acc);
-        if (lane == 0) Pout[(int64_t)blockIdx.x * stride + q] = acc;
+    for (int q = 2 * wid; q < nv; q += 2 * nw) {
+        const double* va = self ? wt : V + (int64_t)q * n + r0;
+        double x = 0.0, y = 0.0;
+        if (q + 1 < nv) {
+            const double* vb = va + n;
+#pragma unroll 8
+            for (int e = lane; e < cnt; e += 32) {
+                const double we = wt[e];
+                x += va[e] * we;
+                y += vb[e] * we;
+            }
+        } else {
+#pragma unroll 8
+            for (int e = lane; e < cnt; e += 32) x += va[e] * wt[e];
+        }
+        x = warp_sum2(x, y, lane);
+        if ((lane & 15) == 0 && q + (lane >> 4) < nv) Pout[(int64_t)blockIdx.x * stride + q + (lane >> 4)] = x;
     }
-    if (lane == 0 && wid < nv) __threadfence();  // once, after the warp's last partial
+    if ((lane & 15) == 0 && 2 * wid < nv) __threadfence();  // once, after the warp's last partials
 }
+
+// The Arnoldi kernels' blocks.  What bounds them is GB300's FP64 pipe (75% busy in the update of 13
+// columns of 2^18 rows, ncu) once enough loads are in flight: tiles of more than 256 rows get 16
+// warps, two blocks an SM, so that the at most 256 tiles of such a level run side by side; with 8 warps
+// and four loads each in flight the part of an Arnoldi step outside the V-cycle took 142 us on 2^18
+// rows (26 steps), now 91.  Tiles of 256 rows keep 8 warps: 16 were 0.6% slower on a 64 x 64 solve and
+// no faster on 65,536 rows (51 -> 44 us a step either way).
+constexpr int ARN_THREADS = 512;
+// the tile's rows of w are kept in shared memory for the dots while they fit
+constexpr int ARN_SMEM_ROWS = 4096;
+static int arn_threads(int tile) { return tile > ARN_MIN_TILE ? ARN_THREADS : ARN_MIN_TILE; }
+static size_t arn_smem(int tile) { return tile <= ARN_SMEM_ROWS ? sizeof(double) * tile : 0; }
 
 // w = V[j+1] = B z_j (FP64) and its per-tile dots with V[0..j]
 template <typename TX>
-__global__ void __launch_bounds__(256) k_arn_spmv_dots(int n, int tile, const int32_t* __restrict__ rp,
+__global__ void __launch_bounds__(ARN_THREADS, 2) k_arn_spmv_dots(int n, int tile, const int32_t* __restrict__ rp,
                                                        const int32_t* __restrict__ ci, const double* __restrict__ bv,
                                                        const TX* __restrict__ z, const int* __restrict__ dj,
                                                        double* __restrict__ V, double* __restrict__ Pout, int stride,
@@ -1382,12 +1424,16 @@ __global__ void __launch_bounds__(256) k_arn_spmv_dots(int n, int tile, const in
     const int j = *dj;
     const int r0 = blockIdx.x * tile, cnt = min(tile, n - r0);
     double* w = V + (int64_t)(j + 1) * n;
+    extern __shared__ double s_w[];
+    const bool keep = tile <= ARN_SMEM_ROWS;
     for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
         const int i = r0 + e;
-        w[i] = row_sum<double>(rp[i], rp[i + 1], ci, bv, [&](int c) { return (double)z[c]; });
+        const double wi = row_sum<double>(rp[i], rp[i + 1], ci, bv, [&](int c) { return (double)z[c]; });
+        w[i] = wi;
+        if (keep) s_w[e] = wi;
     }
     __syncthreads();
-    arn_tile_dots(V, n, j, r0, cnt, w, 0, Pout, stride);
+    arn_tile_dots(V, n, j, r0, cnt, keep ? s_w : w + r0, 0, Pout, stride);
     if (ticket) arn_last_block_sums(Pout, gridDim.x, stride, j + 1, ticket, tot);
 }
 
@@ -1395,7 +1441,7 @@ __global__ void __launch_bounds__(256) k_arn_spmv_dots(int n, int tile, const in
 // the preceding kernel's last block formed; w -= V[0..j] h; then the per-tile dots of the new
 // w with V[0..j] (next_self = 0) or with itself (next_self = 1), with ticket summed by this
 // kernel's last block into tot
-__global__ void __launch_bounds__(256) k_arn_update_dots(int n, int tile, const int* __restrict__ dj,
+__global__ void __launch_bounds__(ARN_THREADS, 2) k_arn_update_dots(int n, int tile, const int* __restrict__ dj,
                                                          double* __restrict__ V, const double* __restrict__ Pin,
                                                          int nb, double* __restrict__ hout, double* __restrict__ Pout,
                                                          int stride, int next_self, unsigned* __restrict__ ticket,
@@ -1418,15 +1464,34 @@ __global__ void __launch_bounds__(256) k_arn_update_dots(int n, int tile, const 
     __syncthreads();
     const int r0 = blockIdx.x * tile, cnt = min(tile, n - r0);
     double* w = V + (int64_t)(j + 1) * n;
-    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
-        const int i = r0 + e;
-        double sacc = w[i];
+    extern __shared__ double s_w[];
+    const bool keep = tile <= ARN_SMEM_ROWS;
+    int e = threadIdx.x;
+    for (; e + (int)blockDim.x < cnt; e += 2 * blockDim.x) {  // two rows at a time
+        const double* v = V + r0 + e;
+        double x = w[r0 + e], y = w[r0 + e + blockDim.x];
 #pragma unroll 8
-        for (int q = 0; q <= j; ++q) sacc -= V[(int64_t)q * n + i] * sh[q];
-        w[i] = sacc;
+        for (int q = 0; q <= j; ++q, v += n) {
+            x -= v[0] * sh[q];
+            y -= v[blockDim.x] * sh[q];
+        }
+        w[r0 + e] = x;
+        w[r0 + e + blockDim.x] = y;
+        if (keep) {
+            s_w[e] = x;
+            s_w[e + blockDim.x] = y;
+        }
+    }
+    if (e < cnt) {
+        const double* v = V + r0 + e;
+        double x = w[r0 + e];
+#pragma unroll 16
+        for (int q = 0; q <= j; ++q, v += n) x -= v[0] * sh[q];
+        w[r0 + e] = x;
+        if (keep) s_w[e] = x;
     }
     __syncthreads();
-    arn_tile_dots(V, n, j, r0, cnt, w, next_self, Pout, stride);
+    arn_tile_dots(V, n, j, r0, cnt, keep ? s_w : w + r0, next_self, Pout, stride);
     if (ticket) arn_last_block_sums(Pout, gridDim.x, stride, next_self ? 1 : j + 1, ticket, tot);
 }
 
@@ -1554,11 +1619,14 @@ void arnoldi_step_graphable(int n, const MatView<double>& B, double* V, T* Z, T*
     double* Pb = partial + (size_t)nt * stride;
     // each kernel's last block sums the per-tile partials for the next (ticket = dj + 1)
     unsigned* ticket = reinterpret_cast<unsigned*>(dj + 1);
-    BAMG_LAUNCH_PDL(k_arn_spmv_dots<T>, nt, 256, 0, s, n, tile, B.rp, B.ci, B.v, (const T*)zout, (const int*)dj, V,
+    BAMG_LAUNCH_PDL(k_arn_spmv_dots<T>, nt, arn_threads(tile), arn_smem(tile), s, n, tile, B.rp, B.ci, B.v,
+                    (const T*)zout, (const int*)dj, V,
                     Pa, stride, ticket, st + L.h1);
-    BAMG_LAUNCH_PDL(k_arn_update_dots, nt, 256, 0, s, n, tile, (const int*)dj, V, (const double*)Pa, nt, st + L.h1,
+    BAMG_LAUNCH_PDL(k_arn_update_dots, nt, arn_threads(tile), arn_smem(tile), s, n, tile, (const int*)dj, V,
+                    (const double*)Pa, nt, st + L.h1,
                     Pb, stride, 0, ticket, st + L.h2);
-    BAMG_LAUNCH_PDL(k_arn_update_dots, nt, 256, 0, s, n, tile, (const int*)dj, V, (const double*)Pb, nt, st + L.h2,
+    BAMG_LAUNCH_PDL(k_arn_update_dots, nt, arn_threads(tile), arn_smem(tile), s, n, tile, (const int*)dj, V,
+                    (const double*)Pb, nt, st + L.h2,
                     Pa, stride, 1, ticket, st + L.nrm2);
     BAMG_LAUNCH_PDL(k_givens_end, 1, 64, 0, s, dj, st, m, ctl, cond);
     if (!cond) BAMG_CK(cudaMemcpyAsync(h_est, st + L.est, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1599,7 +1667,7 @@ __global__ void __launch_bounds__(256) k_parn_store_dots(int n, int tile, const 
     double* w = V + (int64_t)(j + 1) * n;
     for (int e = threadIdx.x; e < cnt; e += blockDim.x) w[r0 + e] = (double)z[r0 + e];
     __syncthreads();
-    arn_tile_dots(V, n, j, r0, cnt, w, 0, Pout, stride);
+    arn_tile_dots(V, n, j, r0, cnt, w + r0, 0, Pout, stride);
 }
 
 // H[0..j, j] = h1 + h2 (the two Gram-Schmidt passes), H[j+1, j] = ||w||; column-major, ld ldh
@@ -1728,9 +1796,11 @@ void parnoldi_step(int n, const MatView<double>& B, double* V, T* vin, T* zout, 
     double* Pa = partial;
     double* Pb = partial + (size_t)nt * stride;
     BAMG_LAUNCH_PDL(k_parn_store_dots<T>, nt, 256, 0, s, n, tile, (const T*)zout, (const int*)dj, V, Pa, stride);
-    BAMG_LAUNCH_PDL(k_arn_update_dots, nt, 256, 0, s, n, tile, (const int*)dj, V, (const double*)Pa, nt, st + L.h1,
+    BAMG_LAUNCH_PDL(k_arn_update_dots, nt, arn_threads(tile), arn_smem(tile), s, n, tile, (const int*)dj, V,
+                    (const double*)Pa, nt, st + L.h1,
                     Pb, stride, 0, (unsigned*)nullptr, (double*)nullptr);
-    BAMG_LAUNCH_PDL(k_arn_update_dots, nt, 256, 0, s, n, tile, (const int*)dj, V, (const double*)Pb, nt, st + L.h2,
+    BAMG_LAUNCH_PDL(k_arn_update_dots, nt, arn_threads(tile), arn_smem(tile), s, n, tile, (const int*)dj, V,
+                    (const double*)Pb, nt, st + L.h2,
                     Pa, stride, 1, (unsigned*)nullptr, (double*)nullptr);
     BAMG_LAUNCH_PDL(k_givens_scale_j, g, 256, 0, s, n, V, (const int*)dj, st, m, (const double*)Pa, nt, stride);
     BAMG_LAUNCH_PDL(k_parn_hess, 1, 64, 0, s, (const double*)st, m, (const int*)dj, H, ldh);

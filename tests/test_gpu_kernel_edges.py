@@ -76,3 +76,42 @@ def test_gradients_at_tile_edges(rows):
         part = g[at:at + g_o[k].size].reshape(g_o[k].shape)
         at += g_o[k].size
         assert np.linalg.norm(part - g_o[k]) <= 2.0 ** -8 * max(np.linalg.norm(g_o[k]), 1e-30), k
+
+
+def _walk(nx, ny):
+    """A grid walk's CSR arrays on the GPU (uniform 1/degree), without the host's sort."""
+    import torch
+
+    off = torch.tensor([-nx, -1, 1, nx], device="cuda")
+    i = torch.arange(nx * ny, device="cuda")
+    x, y = i % nx, i // nx
+    ok = torch.stack([y > 0, x > 0, x < nx - 1, y < ny - 1], 1)
+    deg = ok.sum(1)
+    col = (i[:, None] + off)[ok]
+    ptr = torch.zeros(nx * ny + 1, dtype=torch.int64, device="cuda")
+    ptr[1:] = deg.cumsum(0)
+    return ptr.int(), col.int(), 1.0 / deg[col].double()
+
+
+@pytest.mark.parametrize("nx,ny", [(40, 40), (257, 255), (261, 259), (1030, 1021)])
+def test_arnoldi_tiles_match_persistent_cycle(nx, ny):
+    """The step kernels against the one-launch cycle, which adds in the same order with other
+    thread counts: row tiles of 256, 512 and beyond what shared memory keeps (4096 rows), ragged
+    last tiles, odd and even column counts.  Same iterates bit for bit."""
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+
+    A = _walk(nx, ny)
+    xs = []
+    for persistent in (0, 1):
+        s = bamg.Solver(*A, r=6, levels=20, grid=(nx, ny), precision="mixed", max_it=7, mle_restart=0,
+                        persistent=persistent)
+        x = torch.empty(nx * ny, dtype=torch.float64, device="cuda")
+        try:
+            s.solve(1e-15, out=x)
+        except bamg.BamgError:
+            pass
+        xs.append(x)
+        s.close()
+    assert torch.equal(xs[0], xs[1]) and bool(torch.isfinite(xs[0]).all())
