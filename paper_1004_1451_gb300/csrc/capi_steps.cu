@@ -132,11 +132,11 @@ int bamg_interp_ls(int dtype, const bamg_mat* B, const uint8_t* cf, const int32_
                      "bad interp_ls args");
         int e;
         if (dtype == BAMG_F64)
-            e = interp_ls<double>(B->n, B->row_ptr, B->col, (const double*)B->val, cf, cidx, (const double*)X, ncols,
+            e = interp_ls<double>(B->n, B->nnz, B->row_ptr, B->col, (const double*)B->val, cf, cidx, (const double*)X, ncols,
                                   ld, d_w, z, mmax, c,
                                   ridge, pcol, (double*)pval, pcnt, s);
         else if (dtype == BAMG_F32)
-            e = interp_ls<float>(B->n, B->row_ptr, B->col, (const float*)B->val, cf, cidx, (const float*)X, ncols, ld,
+            e = interp_ls<float>(B->n, B->nnz, B->row_ptr, B->col, (const float*)B->val, cf, cidx, (const float*)X, ncols, ld,
                                  d_w, z, mmax, c,
                                  ridge, pcol, (float*)pval, pcnt, s);
         else
@@ -190,7 +190,7 @@ static void features_step(const bamg_mat* B, const uint8_t* cf, const int32_t* c
     ex.target = d_target;
     ex.cand = d_cand;
     ex.greedy = d_target != nullptr;
-    const int e = interp_ls<T>(Bv.n, Bv.rp, Bv.ci, Bv.v, cf, cidx, (const T*)X, ncols, ld, d_w, z, mmax, c, ridge,
+    const int e = interp_ls<T>(Bv.n, Bv.nnz, Bv.rp, Bv.ci, Bv.v, cf, cidx, (const T*)X, ncols, ld, d_w, z, mmax, c, ridge,
                                pcol.get(), pval.get(), pcnt.get(), s, nullptr, ex);
     BAMG_REQUIRE(e == 0, BAMG_EOVERFLOW, "neighbourhood search: a fine point needs more than 2048 recorded states");
     BAMG_CK(cudaStreamSynchronize(s));
@@ -204,7 +204,7 @@ static void learned_step(const bamg_mat* B, const uint8_t* cf, const int32_t* ci
     const MatView<T> Bv = view<T>(B);
     TmpBuf<int> err(1, s);
     BAMG_CK(cudaMemsetAsync(err.get(), 0, sizeof(int), s));
-    interp_learned<T>(Bv.n, Bv.rp, Bv.ci, Bv.v, cf, cidx, (const T*)X, ncols, ld, d_w, z, mmax, c, ridge, m->impl,
+    interp_learned<T>(Bv.n, Bv.nnz, Bv.rp, Bv.ci, Bv.v, cf, cidx, (const T*)X, ncols, ld, d_w, z, mmax, c, ridge, m->impl,
                       refit != 0, pcol, (T*)pval, pcnt, s, err.get());
     int h = 0;
     BAMG_CK(cudaMemcpyAsync(&h, err.get(), sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -4,6 +4,7 @@
 // B_{l+1} = Q B P, T_{l+1} = Q T P (Section 1 step 3, Algorithm 3).
 #include <cfloat>
 
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 
@@ -280,27 +281,27 @@ constexpr int MMAX = 16;
 constexpr int CMAX = 4;
 constexpr int KMAX = 32;
 
-// Solves the SPD system A x = b of order m <= CMAX by Cholesky; false if not SPD.
-template <typename T>
-__device__ __forceinline__ bool chol_solve(T (&A)[CMAX][CMAX], const T (&b)[CMAX], int m, T (&x)[CMAX]) {
-    T L[CMAX][CMAX];
-    T y[CMAX];
+// Solves the SPD system A x = b of order m <= CM by Cholesky; false if not SPD.
+template <typename T, int CM>
+__device__ __forceinline__ bool chol_solve(T (&A)[CM][CM], const T (&b)[CM], int m, T (&x)[CM]) {
+    T L[CM][CM];
+    T y[CM];
 #pragma unroll
-    for (int j = 0; j < CMAX; ++j) {
+    for (int j = 0; j < CM; ++j) {
         if (j < m) {
             T s = A[j][j];
 #pragma unroll
-            for (int k = 0; k < CMAX; ++k)
+            for (int k = 0; k < CM; ++k)
                 if (k < j) s -= L[j][k] * L[j][k];
             if (!(s > T(0))) return false;
             const T d = sqrt(s);
             L[j][j] = d;
 #pragma unroll
-            for (int i = 0; i < CMAX; ++i) {
+            for (int i = 0; i < CM; ++i) {
                 if (i > j && i < m) {
                     T t = A[i][j];
 #pragma unroll
-                    for (int k = 0; k < CMAX; ++k)
+                    for (int k = 0; k < CM; ++k)
                         if (k < j) t -= L[i][k] * L[j][k];
                     L[i][j] = t / d;
                 }
@@ -308,21 +309,21 @@ __device__ __forceinline__ bool chol_solve(T (&A)[CMAX][CMAX], const T (&b)[CMAX
         }
     }
 #pragma unroll
-    for (int j = 0; j < CMAX; ++j) {
+    for (int j = 0; j < CM; ++j) {
         if (j < m) {
             T t = b[j];
 #pragma unroll
-            for (int k = 0; k < CMAX; ++k)
+            for (int k = 0; k < CM; ++k)
                 if (k < j) t -= L[j][k] * y[k];
             y[j] = t / L[j][j];
         }
     }
 #pragma unroll
-    for (int j = CMAX - 1; j >= 0; --j) {
+    for (int j = CM - 1; j >= 0; --j) {
         if (j < m) {
             T t = y[j];
 #pragma unroll
-            for (int k = 0; k < CMAX; ++k)
+            for (int k = 0; k < CM; ++k)
                 if (k > j && k < m) t -= L[k][j] * x[k];
             x[j] = t / L[j][j];
         }
@@ -401,7 +402,11 @@ __device__ void learned_features(int i, int lane, int node, int ncand, int depth
 // ties) joins J.
 // Visited set of a neighbourhood search: open addressing over 2 CAP slots (load <= 1/2),
 // keys are node indices, -1 = empty.
-__device__ __forceinline__ unsigned vis_hash(int v, int nslots) { return ((unsigned)v * 2654435761u) & (nslots - 1); }
+// (the product's top bits: its low bits repeat for states whose indices differ by a multiple of
+// nslots, as neighbours in adjacent rows of a grid 512 wide do)
+__device__ __forceinline__ unsigned vis_hash(int v, int nslots) {
+    return ((unsigned)v * 2654435761u) >> (__clz(nslots) + 1);
+}
 __device__ __forceinline__ bool vis_contains(const int* hs, int nslots, int v) {
     for (unsigned h = vis_hash(v, nslots);; h = (h + 1) & (nslots - 1)) {
         const int k = hs[h];
@@ -619,7 +624,7 @@ __device__ bool ls_point(int i, const int32_t* __restrict__ rp, const int32_t* _
 #pragma unroll
             for (int a = 0; a < CMAX; ++a)
                 if (a <= t) A[a][a] += delta;
-            if (chol_solve<T>(A, rhs, t + 1, pl)) {
+            if (chol_solve<T, CMAX>(A, rhs, t + 1, pl)) {
                 T acc = T(0);
                 for (int k = 0; k < ncols; ++k) {
                     T r = xi[k] - pl[t] * xs[k];
@@ -749,8 +754,386 @@ __global__ void __launch_bounds__(WARPS * 32, (WARPS > 1 && sizeof(T) == 4) ? 8 
     }
 }
 
+// ---------------------------------------------------------------- two points a warp
+// The fit without optional outputs, in two kernels: the neighbourhood searches, then the greedy
+// fits.  Each half of a warp takes one point, 16 lanes for the at most 16 candidates.  Same candidates
+// and the same arithmetic per candidate as ls_point, so the same rows bit for bit.
+//
+// What bounds them: instruction issue and the chain of dependent loads (every operand sits in L1 or
+// L2).  One warp a point with half its lanes idle in the fit took 2240 warp instructions a fine point
+// (631 us for 2^18 points of a triangulation, 16 columns).  Here
+//  - the search's batches need no order within a depth (candidates are ranked by depth and coarse
+//    index, and a search cut short by the list's capacity goes to the second pass), so an entry is
+//    new if it wins its slot of the visited table: one compare-and-swap instead of a lookup, a match
+//    over the warp and an insertion, and 4, 8 or 16 lanes walk a row instead of a search for the row
+//    of each entry;
+//  - at the last depth only coarse entries are taken down (the old list, filled by fine ones, sent
+//    points of long-row levels to the second pass);
+//  - coarse entries are listed as they are found, so a rank is a count within its depth;
+//  - a lane keeps its candidate's test-vector row in registers (NC columns, 16-byte loads where X
+//    allows them) instead of reading it again in each of the fit's five passes;
+//  - the search, which waits for loads, runs with few registers and many warps, apart from the fit.
+// Measured on those 2^18 points: one kernel 576 us; apart, search 307 and fit 172; with the visited
+// table hashed by the product's top bits search 154 (ncu); the call 725 -> 370 us.  FP64, 16 columns,
+// 93,300 points: 1591 -> 923 us.
+constexpr int LSP_WARPS = 4;
+// One search by GL lanes: CAP nodes recorded (beyond, the second pass) for the frontiers, and as
+// many coarse nodes with their coarse indices, depth by depth.
+template <int GL>
+struct LsSearch {
+    static constexpr int CAP = 8 * GL;
+    int vis[CAP], hash[2 * CAP];
+    int cnode[CAP], ccol[CAP];
+};
+
+// whether v is new: it wins (or finds) its slot of the visited table
+template <int HS>
+__device__ __forceinline__ bool lsp_claim(int* hs, int v) {
+    for (unsigned h = vis_hash(v, HS);; h = (h + 1) & (HS - 1)) {
+        int k = *(volatile int*)&hs[h];
+        if (k == -1) {
+            k = atomicCAS(&hs[h], -1, v);
+            if (k == -1) return true;
+        }
+        if (k == v) return false;
+    }
+}
+
+// Neighbourhood search (Eq. (3.5), with the extension to depth 3) of point i (i < 0: none) by GL lanes
+// (half a warp or a whole one): candidates (nodes, in rank order) into cand; their count, or -1 when
+// the list overflowed.  1 << gs lanes walk a row, U entries each at a time.  Every lane of the warp
+// calls it.
+template <int GL, int U>
+__device__ __forceinline__ int lsp_search(int i, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                                          const uint8_t* __restrict__ cf, const int32_t* __restrict__ cidx, int z,
+                                          int mmax, int gs, LsSearch<GL>& sh, int32_t* __restrict__ cand) {
+    constexpr int CAP = LsSearch<GL>::CAP;
+    const int lane = threadIdx.x & 31, sub = lane & (GL - 1), hb = lane & ~(GL - 1);
+    const unsigned lt = ((1u << sub) - 1u) << hb, half = (GL == 32 ? 0xffffffffu : 0xffffu) << hb;
+    {
+        int4* h4 = reinterpret_cast<int4*>(sh.hash);
+#pragma unroll
+        for (int e = 0; e < 2 * CAP / 4 / GL; ++e) h4[GL * e + sub] = make_int4(-1, -1, -1, -1);
+    }
+    __syncwarp();
+    if (sub == 0 && i >= 0) {
+        sh.vis[0] = i;
+        sh.hash[vis_hash(i, 2 * CAP)] = i;
+    }
+    __syncwarp();
+    int nvis = 1, nclaim = 1, fs = 0, fe = 1;
+    int nc = 0, c1 = 0, c2 = 0;  // nc coarse nodes, c1 at depth 1, c2 up to depth 2
+    bool run = i >= 0, ovf = false;
+    const int rows = GL >> gs, width = 1 << gs;
+#pragma unroll 1
+    for (int d = 1; d <= 3; ++d) {
+        // beyond z only while no coarse point has been reached; no deeper once mmax are known
+        run = run && !((d > z && nc > 0) || nc >= mmax);
+        if (!__any_sync(0xffffffffu, run)) break;
+        // the last depth, or the list is full: only coarse nodes count from here on
+        bool fonly = d == 3 || (d >= z && nc > 0);
+#pragma unroll 1
+        for (int f0 = fs; __any_sync(0xffffffffu, run && f0 < fe); f0 += rows) {
+            const int f = f0 + (sub >> gs);
+            int p = 0, pe = 0;
+            if (run && f < fe) {
+                const int u = sh.vis[f];
+                p = rp[u] + (sub & (width - 1));
+                pe = rp[u + 1];
+            }
+#pragma unroll 1
+            for (; __any_sync(0xffffffffu, p < pe); p += U * width) {
+                int v[U];
+                bool c[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) v[u] = p + u * width < pe ? ci[p + u * width] : -1;
+#pragma unroll
+                for (int u = 0; u < U; ++u) c[u] = v[u] >= 0 && cf[v[u]] != 0;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const bool want = run && v[u] >= 0 && (!fonly || c[u]);
+                    if (U > 1 && !__any_sync(0xffffffffu, want)) continue;
+                    const bool isnew = want && lsp_claim<2 * CAP>(sh.hash, v[u]);
+                    const bool vc = isnew && c[u];
+                    const unsigned bal = __ballot_sync(0xffffffffu, isnew) & half;
+                    const unsigned balc = __ballot_sync(0xffffffffu, vc) & half;
+                    fonly = fonly || nvis + __popc(bal) > CAP;
+                    nclaim += __popc(bal);
+                    // the coarse list is full, or the table would be with the next batch
+                    if (nc + __popc(balc) > CAP || nclaim > 2 * CAP - 1 - GL) {
+                        ovf = true;
+                        run = false;
+                        pe = 0;
+                    } else {
+                        if (isnew && !fonly) sh.vis[nvis + __popc(bal & lt)] = v[u];
+                        if (vc) {
+                            const int q = nc + __popc(balc & lt);
+                            sh.cnode[q] = v[u];
+                            sh.ccol[q] = cidx[v[u]];
+                        }
+                        if (!fonly) nvis += __popc(bal);
+                        nc += __popc(balc);
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+        if (fonly && run) {  // a truncated depth is exact only if the search ends here
+            if (d < 3 && nc < mmax && !(d >= z && nc > 0)) ovf = true;
+            run = false;
+        }
+        if (d == 1) c1 = nc;
+        if (d <= 2) c2 = nc;
+        fs = fe;
+        fe = nvis;
+    }
+    if (i < 0 || ovf) nc = 0;
+    // rank by (depth, coarse index): the list holds depth 1, then 2, then 3
+#pragma unroll 1
+    for (int q = sub; __any_sync(0xffffffffu, q < nc); q += GL) {
+        if (q < nc) {
+            const int a = q < c1 ? 0 : q < c2 ? c1 : c2, b = q < c1 ? c1 : q < c2 ? c2 : nc;
+            const int kq = sh.ccol[q];
+            int rank = a;
+            for (int e = a; e < b && rank < mmax; ++e) rank += sh.ccol[e] < kq;
+            if (rank < mmax) cand[rank] = sh.cnode[q];
+        }
+    }
+    return ovf ? -1 : (nc < mmax ? nc : mmax);
+}
+
+// cand: mmax nodes a point; ncand: their count, -1 for a coarse point or one left to the second pass.
+template <int GL, int U>
+__global__ void __launch_bounds__(LSP_WARPS * 32, 10)
+    k_ls_search(int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci, const uint8_t* __restrict__ cf,
+                const int32_t* __restrict__ cidx, int z, int mmax, int gs, int32_t* __restrict__ cand,
+                int32_t* __restrict__ ncand, int* __restrict__ ovf_list, int* __restrict__ ovf_count) {
+    pdl_begin();
+    constexpr int PW = 32 / GL;  // points a warp
+    __shared__ alignas(16) LsSearch<GL> s_point[LSP_WARPS][PW];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane & (GL - 1), h = lane / GL;
+    LsSearch<GL>& sh = s_point[wid][h];
+    const int64_t work = ((int64_t)n + PW - 1) / PW, stride = (int64_t)gridDim.x * LSP_WARPS;
+#pragma unroll 1
+    for (int64_t q = (int64_t)blockIdx.x * LSP_WARPS + wid; q < work; q += stride) {
+        const int64_t i = PW * q + h;
+        const bool fine = i < n && cf[i] == 0;
+        int m = -1;
+        if (__any_sync(0xffffffffu, fine)) {
+            m = lsp_search<GL, U>(fine ? (int)i : -1, rp, ci, cf, cidx, z, mmax, gs, sh, cand + i * mmax);
+            if (m < 0 && sub == 0) ovf_list[atomicAdd(ovf_count, 1)] = (int)i;  // the second pass redoes it
+        }
+        if (sub == 0 && i < n) ncand[i] = fine ? m : -1;
+        __syncwarp();  // the shared memory takes the next points
+    }
+}
+
+template <typename T, int CM>
+struct LsFit {
+    alignas(16) T xi[KMAX];
+    alignas(16) T xj[CM][KMAX];
+};
+// blocks an SM: as many as leave the registers a candidate's row needs
+constexpr int lsp_blocks(int size, int nc) {
+    return size == 4 ? (nc <= 8 ? 6 : nc <= 16 ? 5 : 4) : (nc <= 8 ? 4 : nc <= 16 ? 3 : 2);
+}
+template <typename T, int NC, int CM>
+__global__ void __launch_bounds__(LSP_WARPS * 32, lsp_blocks(sizeof(T), NC))
+    k_ls_pair(int n, const uint8_t* __restrict__ cf, const int32_t* __restrict__ cidx, const int32_t* __restrict__ cand,
+              const int32_t* __restrict__ ncands, const T* __restrict__ X, int ncols, int ld,
+              const double* __restrict__ w, int mmax, int c, double ridge, bool vec, int32_t* __restrict__ pcol,
+              T* __restrict__ pval, int32_t* __restrict__ pcnt) {
+    pdl_begin();
+    constexpr int W = V16<T>::W;
+    __shared__ LsFit<T, CM> s_half[LSP_WARPS][2];
+    __shared__ alignas(16) T s_w[KMAX];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane & 15, hb = lane & 16;
+    if (threadIdx.x < KMAX) s_w[threadIdx.x] = threadIdx.x < ncols ? (T)w[threadIdx.x] : T(0);
+    __syncthreads();
+    LsFit<T, CM>& sh = s_half[wid][hb >> 4];
+    const T INF = (T)INFINITY;
+    const int64_t pairs = ((int64_t)n + 1) / 2, stride = (int64_t)gridDim.x * LSP_WARPS;
+#pragma unroll 1
+    for (int64_t q = (int64_t)blockIdx.x * LSP_WARPS + wid; q < pairs; q += stride) {
+        const int64_t i64 = 2 * q + (hb >> 4);
+        const int ncand = i64 < n ? ncands[i64] : -1;
+        const bool fine = ncand >= 0;
+        if (i64 < n && !fine && cf[i64]) {  // a coarse point's unit row
+            if (sub < c) {
+                pcol[i64 * c + sub] = sub == 0 ? cidx[i64] : -1;
+                pval[i64 * c + sub] = sub == 0 ? T(1) : T(0);
+            }
+            if (sub == 0) pcnt[i64] = 1;
+        }
+        if (!__any_sync(0xffffffffu, fine)) continue;
+        const int node = sub < ncand ? cand[i64 * mmax + sub] : -1;
+        const int ccol = node >= 0 ? cidx[node] : 0;
+        T xs[NC];
+        if (node >= 0) {
+            const T* x = X + (int64_t)node * ld;
+            if (vec) {
+#pragma unroll
+                for (int k = 0; k < NC; k += W)
+                    if (k < ncols) {
+                        V16<T>::load(x + k, xs + k);
+#pragma unroll
+                        for (int e = 1; e < W; ++e)
+                            if (k + e >= ncols) xs[k + e] = T(0);
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < W; ++e) xs[k + e] = T(0);
+                    }
+            } else {
+#pragma unroll
+                for (int k = 0; k < NC; ++k) xs[k] = k < ncols ? x[k] : T(0);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < NC; ++k) xs[k] = T(0);
+        }
+        for (int k = sub; k < NC; k += 16) sh.xi[k] = fine && k < ncols ? X[i64 * ld + k] : T(0);
+        __syncwarp();
+        T gss = T(0), bs = T(0);
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            const T wk = s_w[k], v = xs[k];
+            gss += wk * v * v;
+            bs += wk * v * sh.xi[k];
+        }
+        // greedy least squares (Algorithm 2)
+        T gsj[CM], GJJ[CM][CM], bJ[CM], pbest[CM];
+        int J[CM];
+#pragma unroll
+        for (int a = 0; a < CM; ++a) {
+            gsj[a] = bJ[a] = pbest[a] = T(0);
+            J[a] = 0x7fffffff;
+#pragma unroll
+            for (int b = 0; b < CM; ++b) GJJ[a][b] = T(0);
+        }
+        bool used = false, go = fine;
+        int nJ = 0;
+#pragma unroll
+        for (int t = 0; t < CM; ++t) {
+            if (t >= c) break;
+            T L = INF;
+            T pl[CM];
+#pragma unroll
+            for (int a = 0; a < CM; ++a) pl[a] = T(0);
+            if (go && node >= 0 && !used) {
+                T A[CM][CM], rhs[CM];
+                T tr = gss;
+#pragma unroll
+                for (int a = 0; a < CM; ++a) {
+#pragma unroll
+                    for (int b = 0; b < CM; ++b) A[a][b] = (a < t && b < t) ? GJJ[a][b] : T(0);
+                    rhs[a] = a < t ? bJ[a] : T(0);
+                    if (a < t) tr += GJJ[a][a];
+                }
+#pragma unroll
+                for (int a = 0; a < CM; ++a) {
+                    if (a < t) {
+                        A[a][t] = gsj[a];
+                        A[t][a] = gsj[a];
+                    }
+                }
+                A[t][t] = gss;
+                rhs[t] = bs;
+                const T delta = (T)ridge * tr / (T)(t + 1);
+#pragma unroll
+                for (int a = 0; a < CM; ++a)
+                    if (a <= t) A[a][a] += delta;
+                if (chol_solve<T, CM>(A, rhs, t + 1, pl)) {
+                    T acc = T(0);
+#pragma unroll
+                    for (int k = 0; k < NC; ++k) {
+                        T r = sh.xi[k] - pl[t] * xs[k];
+#pragma unroll
+                        for (int a = 0; a < CM; ++a)
+                            if (a < t) r -= pl[a] * sh.xj[a][k];
+                        acc += s_w[k] * r * r;
+                    }
+                    L = (acc == acc) ? acc : INF;
+                }
+            }
+            T bestL = L;
+            int bestLane = lane;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) {
+                const T oL = __shfl_xor_sync(0xffffffffu, bestL, o);
+                const int oLane = __shfl_xor_sync(0xffffffffu, bestLane, o);
+                if (oL < bestL || (oL == bestL && oLane < bestLane)) {
+                    bestL = oL;
+                    bestLane = oLane;
+                }
+            }
+            go = go && bestL < INF;
+            if (!__any_sync(0xffffffffu, go)) break;
+            const T w_gss = __shfl_sync(0xffffffffu, gss, bestLane);
+            const T w_bs = __shfl_sync(0xffffffffu, bs, bestLane);
+            const int w_c = __shfl_sync(0xffffffffu, ccol, bestLane);
+            T w_g[CM], w_p[CM];
+#pragma unroll
+            for (int a = 0; a < CM; ++a) {
+                w_g[a] = __shfl_sync(0xffffffffu, gsj[a], bestLane);
+                w_p[a] = __shfl_sync(0xffffffffu, pl[a], bestLane);
+            }
+            if (go) {
+#pragma unroll
+                for (int a = 0; a < CM; ++a) {
+                    if (a < t) {
+                        GJJ[t][a] = w_g[a];
+                        GJJ[a][t] = w_g[a];
+                    }
+                    pbest[a] = a <= t ? w_p[a] : T(0);
+                }
+                GJJ[t][t] = w_gss;
+                bJ[t] = w_bs;
+                J[t] = w_c;
+                nJ = t + 1;
+                if (lane == bestLane) {  // the winner's row, from its registers
+                    used = true;
+#pragma unroll
+                    for (int k = 0; k < NC; k += W) V16<T>::store(&sh.xj[t][k], xs + k);
+                }
+            }
+            __syncwarp();
+            if (t + 1 < CM && t + 1 < c) {
+                T g = T(0);
+#pragma unroll
+                for (int k = 0; k < NC; ++k) g += s_w[k] * xs[k] * sh.xj[t][k];
+                gsj[t] = g;
+            }
+        }
+        if (fine && sub == 0) {
+            T vals[CM];
+#pragma unroll
+            for (int a = 0; a < CM; ++a) vals[a] = pbest[a];
+#pragma unroll
+            for (int a = 1; a < CM; ++a)  // by coarse index; empty slots (index 0x7fffffff) last
+#pragma unroll
+                for (int b = a; b > 0; --b)
+                    if (J[b - 1] > J[b]) {
+                        const int tc = J[b];
+                        J[b] = J[b - 1];
+                        J[b - 1] = tc;
+                        const T tv = vals[b];
+                        vals[b] = vals[b - 1];
+                        vals[b - 1] = tv;
+                    }
+#pragma unroll
+            for (int a = 0; a < CM; ++a)
+                if (a < c) {
+                    pcol[i64 * c + a] = a < nJ ? J[a] : -1;
+                    pval[i64 * c + a] = a < nJ ? vals[a] : T(0);
+                }
+            pcnt[i64] = nJ;
+        }
+        __syncwarp();  // the halves' shared memory takes the next pair
+    }
+}
+
 template <typename T>
-int interp_ls(int n, const int32_t* rp, const int32_t* ci, const T* bv, const uint8_t* cf, const int32_t* cidx,
+int interp_ls(int n, int nnz, const int32_t* rp, const int32_t* ci, const T* bv, const uint8_t* cf, const int32_t* cidx,
               const T* X, int ncols, int ld, const double* d_w, int z, int mmax, int c, double ridge, int32_t* pcol,
               T* pval, int32_t* pcnt, cudaStream_t s, int* d_err, const LsOut& ex) {
     BAMG_REQUIRE(ncols >= 1 && ncols <= KMAX, BAMG_EINVAL, "interp_ls: 1 <= ncols <= 32");
@@ -760,30 +1143,62 @@ int interp_ls(int n, const int32_t* rp, const int32_t* ci, const T* bv, const ui
     if (n == 0) return 0;
     // two passes: the common case with a small visited list and 4 warps per block, then the
     // (rare) points whose search overflowed it, with a large list and one warp per block
-    TmpBuf<int> olist(n, s), ocount(1, s), err(1, s);
-    BAMG_CK(cudaMemsetAsync(ocount.get(), 0, sizeof(int), s));
-    int* e = d_err ? d_err : err.get();  // with d_err the caller reads the overflow flag later
-    if (!d_err) BAMG_CK(cudaMemsetAsync(err.get(), 0, sizeof(int), s));
-    // the optional outputs are compiled into a separate instance (they cost registers)
     const bool extra = ex.feat || ex.target || ex.cand || !ex.greedy;
+    // one allocation: the overflow count and flag, the listed points, and the searches' results
+    TmpBuf<int32_t> work(2 + (size_t)n * (extra ? 1 : 2 + mmax), s);
+    int *ocount = work.get(), *err = work.get() + 1, *olist = work.get() + 2;
+    int32_t *ncand = work.get() + 2 + n, *cand = ncand + n;
+    BAMG_CK(cudaMemsetAsync(ocount, 0, 2 * sizeof(int), s));
+    int* e = d_err ? d_err : err;  // with d_err the caller reads the overflow flag later
+    // the optional outputs are compiled into a separate instance (they cost registers)
     if (extra) {
         BAMG_LAUNCH((k_ls_fit<T, VIS_CAP, LS_WARPS, true>), blocks_for(n, LS_WARPS), LS_WARPS * 32, 0, s, n, rp, ci, bv,
                     cf, cidx, X, ncols, ld, d_w, z, mmax, c, ridge, pcol, pval, pcnt, (const int*)nullptr,
-                    (const int*)nullptr, olist.get(), ocount.get(), e, ex);
+                    (const int*)nullptr, olist, ocount, e, ex);
         BAMG_LAUNCH((k_ls_fit<T, VIS_CAP2, 1, true>), LS2_BLOCKS, 32, 0, s, n, rp, ci, bv, cf, cidx, X, ncols, ld, d_w,
-                    z, mmax, c, ridge, pcol, pval, pcnt, (const int*)olist.get(), (const int*)ocount.get(),
+                    z, mmax, c, ridge, pcol, pval, pcnt, (const int*)olist, (const int*)ocount,
                     (int*)nullptr, (int*)nullptr, e, ex);
     } else {
-        BAMG_LAUNCH((k_ls_fit<T, VIS_CAP, LS_WARPS, false>), blocks_for(n, LS_WARPS), LS_WARPS * 32, 0, s, n, rp, ci,
-                    bv, cf, cidx, X, ncols, ld, d_w, z, mmax, c, ridge, pcol, pval, pcnt, (const int*)nullptr,
-                    (const int*)nullptr, olist.get(), ocount.get(), e, ex);
+        int dev = 0, nsm = 0;
+        BAMG_CK(cudaGetDevice(&dev));
+        BAMG_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+        // enough blocks for two rounds of the resident ones; beyond, the warps walk the pairs
+        auto search = [&](auto kern, int per_block, int gs) {
+            const unsigned g = (unsigned)std::min<int64_t>(((int64_t)n + per_block - 1) / per_block, (int64_t)nsm * 20);
+            BAMG_LAUNCH(kern, g, LSP_WARPS * 32, 0, s, n, rp, ci, cf, cidx, z, mmax, gs, cand, ncand,
+                        olist, ocount);
+        };
+        // short rows: half a warp a point, the lanes that take an average row in one step; long rows (or
+        // too few points to fill the chip with halves): a warp a point, four rows of up to 32 entries at
+        // a time.  On a triangulation's coarse levels (rows of 19 to 36 entries, 6015 to 464 points) the
+        // fit of a rebuild took 119 to 247 us with halves, 70 to 110 with warps, 64 to 86 before.
+        if ((int64_t)nnz > 10 * (int64_t)n || n <= nsm * 32)
+            search(k_ls_search<32, 4>, LSP_WARPS, 3);
+        else
+            search(k_ls_search<16, 1>, 2 * LSP_WARPS, (int64_t)nnz <= 4 * (int64_t)n ? 2 : 3);
+        const unsigned grid =
+            (unsigned)std::min<int64_t>(((int64_t)n + 2 * LSP_WARPS - 1) / (2 * LSP_WARPS), (int64_t)nsm * 12);
+        constexpr int W = V16<T>::W;
+        const bool vec = ld % W == 0 && ((uintptr_t)X & 15) == 0;
+        auto go = [&](auto kern) {
+            BAMG_LAUNCH(kern, grid, LSP_WARPS * 32, 0, s, n, cf, cidx, (const int32_t*)cand,
+                        (const int32_t*)ncand, X, ncols, ld, d_w, mmax, c, ridge, vec, pcol, pval, pcnt);
+        };
+        if (c <= 2) {
+            if (ncols <= 8) go(k_ls_pair<T, 8, 2>);
+            else if (ncols <= 16) go(k_ls_pair<T, 16, 2>);
+            else if (ncols <= 24) go(k_ls_pair<T, 24, 2>);
+            else go(k_ls_pair<T, 32, 2>);
+        } else {
+            go(k_ls_pair<T, 32, 4>);
+        }
         BAMG_LAUNCH((k_ls_fit<T, VIS_CAP2, 1, false>), LS2_BLOCKS, 32, 0, s, n, rp, ci, bv, cf, cidx, X, ncols, ld,
-                    d_w, z, mmax, c, ridge, pcol, pval, pcnt, (const int*)olist.get(), (const int*)ocount.get(),
+                    d_w, z, mmax, c, ridge, pcol, pval, pcnt, (const int*)olist, (const int*)ocount,
                     (int*)nullptr, (int*)nullptr, e, ex);
     }
     if (d_err) return 0;
     int h = 0;
-    BAMG_CK(cudaMemcpyAsync(&h, err.get(), sizeof(int), cudaMemcpyDeviceToHost, s));
+    BAMG_CK(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     BAMG_CK(cudaStreamSynchronize(s));
     return h ? BAMG_EOVERFLOW : 0;
 }
@@ -850,7 +1265,7 @@ __global__ void k_learned_select(int n, const uint8_t* __restrict__ cf, const in
         }
         const T delta = (T)ridge * tr / (T)nJ;
         for (int a = 0; a < nJ; ++a) A[a][a] += delta;
-        if (chol_solve<T>(A, rhs, nJ, sol))
+        if (chol_solve<T, CMAX>(A, rhs, nJ, sol))
 #pragma unroll
             for (int a = 0; a < CMAX; ++a) p[a] = a < nJ ? sol[a] : T(0);
     }
@@ -875,7 +1290,7 @@ __global__ void k_learned_select(int n, const uint8_t* __restrict__ cf, const in
 }
 
 template <typename T>
-int interp_learned(int n, const int32_t* rp, const int32_t* ci, const T* bv, const uint8_t* cf, const int32_t* cidx,
+int interp_learned(int n, int nnz, const int32_t* rp, const int32_t* ci, const T* bv, const uint8_t* cf, const int32_t* cidx,
                    const T* X, int ncols, int ld, const double* d_w, int z, int mmax, int c, double ridge,
                    const Model* model, bool refit, int32_t* pcol, T* pval, int32_t* pcnt, cudaStream_t s, int* d_err) {
     BAMG_REQUIRE(model != nullptr, BAMG_EINVAL, "learned interpolation without a model");
@@ -887,7 +1302,7 @@ int interp_learned(int n, const int32_t* rp, const int32_t* ci, const T* bv, con
     ex.feat = feat.get();
     ex.cand = cand.get();
     ex.greedy = false;
-    const int e = interp_ls<T>(n, rp, ci, bv, cf, cidx, X, ncols, ld, d_w, z, mmax, c, ridge, pcol, pval, pcnt, s,
+    const int e = interp_ls<T>(n, nnz, rp, ci, bv, cf, cidx, X, ncols, ld, d_w, z, mmax, c, ridge, pcol, pval, pcnt, s,
                                d_err, ex);
     if (e) return e;
     mlp_forward(model, n, feat.get(), Y.get(), s);
@@ -1516,10 +1931,10 @@ void csr_to_dense(int n, const int32_t* rp, const int32_t* ci, const T* v, doubl
 }
 
 #define INST(T)                                                                                                     \
-    template int interp_ls<T>(int, const int32_t*, const int32_t*, const T*, const uint8_t*, const int32_t*,       \
+    template int interp_ls<T>(int, int, const int32_t*, const int32_t*, const T*, const uint8_t*, const int32_t*,       \
                               const T*, int, int, const double*, int, int, int, double, int32_t*, T*, int32_t*,     \
                               cudaStream_t, int*, const LsOut&);                                                    \
-    template int interp_learned<T>(int, const int32_t*, const int32_t*, const T*, const uint8_t*, const int32_t*,  \
+    template int interp_learned<T>(int, int, const int32_t*, const int32_t*, const T*, const uint8_t*, const int32_t*,  \
                                    const T*, int, int, const double*, int, int, int, double, const Model*, bool,    \
                                    int32_t*, T*, int32_t*, cudaStream_t, int*);                                     \
     template void build_restriction<T>(const EllView<T>&, int, DevBuf<int32_t>&, DevBuf<int32_t>&, DevBuf<T>&,      \

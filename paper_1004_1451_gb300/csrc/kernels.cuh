@@ -106,14 +106,14 @@ void coarsen_grid(int nx, int ny, uint8_t* cf, int32_t* cidx, cudaStream_t s);
 void coarse_to_fine(int n, const uint8_t* cf, const int32_t* cidx, int32_t* c2f, cudaStream_t s);
 // Returns an error flag (BAMG_EOVERFLOW if a neighbourhood search overflowed).
 template <typename T>
-int interp_ls(int n, const int32_t* rp, const int32_t* ci, const T* bv, const uint8_t* cf, const int32_t* cidx,
+int interp_ls(int n, int nnz, const int32_t* rp, const int32_t* ci, const T* bv, const uint8_t* cf, const int32_t* cidx,
               const T* X, int ncols, int ld, const double* d_w, int z, int mmax, int c, double ridge, int32_t* pcol,
               T* pval, int32_t* pcnt, cudaStream_t s, int* d_err = nullptr, const LsOut& ex = LsOut());
 // Learned interpolation of one level: candidates and features (the LS kernel's search),
 // the MLP, then per fine point the c slots of largest |y| with weights y or, with refit,
 // the Eq. (3.6) minimiser over them.  Coarse rows are unit rows.
 template <typename T>
-int interp_learned(int n, const int32_t* rp, const int32_t* ci, const T* bv, const uint8_t* cf, const int32_t* cidx,
+int interp_learned(int n, int nnz, const int32_t* rp, const int32_t* ci, const T* bv, const uint8_t* cf, const int32_t* cidx,
                    const T* X, int ncols, int ld, const double* d_w, int z, int mmax, int c, double ridge,
                    const Model* model, bool refit, int32_t* pcol, T* pval, int32_t* pcnt, cudaStream_t s,
                    int* d_err = nullptr);

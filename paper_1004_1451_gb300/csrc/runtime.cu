@@ -317,7 +317,7 @@ struct Solver : SolverBase {
         c.pval.alloc((size_t)c.n * o.caliber);
         c.pcnt.alloc(c.n);
         if (o.interp == BAMG_INTERP_LEARNED) {
-            interp_learned<T>(c.n, c.rp.get(), c.ci.get(), c.bv.get(), c.cf.get(), c.cidx.get(), c.X.get(), ld, ld,
+            interp_learned<T>(c.n, c.nnz, c.rp.get(), c.ci.get(), c.bv.get(), c.cf.get(), c.cidx.get(), c.X.get(), ld, ld,
                               c.w.get(), o.z, o.mmax, o.caliber, ridge(), o.model->impl, o.learned_refit != 0,
                               c.pcol.get(), c.pval.get(), c.pcnt.get(), s, ls_err.get());
         } else {
@@ -329,7 +329,7 @@ struct Solver : SolverBase {
                 }
                 rec_rows += c.n;
             }
-            interp_ls<T>(c.n, c.rp.get(), c.ci.get(), c.bv.get(), c.cf.get(), c.cidx.get(), c.X.get(), ld, ld,
+            interp_ls<T>(c.n, c.nnz, c.rp.get(), c.ci.get(), c.bv.get(), c.cf.get(), c.cidx.get(), c.X.get(), ld, ld,
                          c.w.get(), o.z, o.mmax, o.caliber, ridge(), c.pcol.get(), c.pval.get(), c.pcnt.get(), s,
                          ls_err.get(), ex);
         }

@@ -105,7 +105,7 @@ def test_arnoldi_tiles_match_persistent_cycle(nx, ny):
     A = _walk(nx, ny)
     xs = []
     for persistent in (0, 1):
-        s = bamg.Solver(*A, r=6, levels=20, grid=(nx, ny), precision="mixed", max_it=7, mle_restart=0,
+        s = bamg.Solver(*A, r=10, levels=20, grid=(nx, ny), precision="mixed", max_it=7, mle_restart=0,
                         persistent=persistent)
         x = torch.empty(nx * ny, dtype=torch.float64, device="cuda")
         try:
@@ -115,3 +115,68 @@ def test_arnoldi_tiles_match_persistent_cycle(nx, ny):
         xs.append(x)
         s.close()
     assert torch.equal(xs[0], xs[1]) and bool(torch.isfinite(xs[0]).all())
+
+
+def _level(kind, n, ncols, ld, dtype, offset, seed):
+    """B (pattern with unit diagonal), a C/F split and test vectors whose rows start `offset` elements
+    into their storage."""
+    import scipy.sparse as sp
+    import torch
+
+    rng = np.random.default_rng(seed)
+    if kind == "grid":  # five entries a row, neighbours a multiple of 512 apart
+        nx = 512
+        i = np.arange(n)
+        pairs = [(i[:-1], i[1:]), (i[:-nx], i[nx:])] if n > nx else [(i[:-1], i[1:])]
+    elif kind == "ring":  # about 12 entries a row
+        i = np.arange(n)
+        pairs = [(i, (i + rng.integers(1, 40, n)) % n) for _ in range(6)]
+    else:  # hubs: a few rows of hundreds of entries, so that searches overflow the first list
+        i = np.arange(n)
+        pairs = [(i, rng.integers(0, n, n)) for _ in range(2)] + [(np.full(300, h), rng.integers(0, n, 300)) for h in range(4)]
+    a, b = (np.concatenate([p[k] for p in pairs]) for k in (0, 1))
+    A = sp.coo_matrix((np.ones(a.size), (a, b)), shape=(n, n))
+    A = sp.csr_matrix(A + A.T + sp.identity(n))
+    A.data[:] = -0.1
+    A.setdiag(1.0)
+    A.sort_indices()
+    cf = rng.random(n) < 0.3
+    cf[0] = True
+    cidx = np.where(cf, np.cumsum(cf) - 1, -1)
+    td = torch.float64 if dtype == "fp64" else torch.float32
+    X = torch.empty(n * ld + offset, dtype=td, device="cuda")[offset:].view(n, ld)
+    X.copy_(torch.tensor(rng.random((n, ld)) + 0.5))
+    X[:, ncols:] = float("nan")  # columns beyond ncols are not read into a result
+    B = tuple(torch.tensor(v, device="cuda") for v in (A.indptr.astype(np.int32), A.indices.astype(np.int32)))
+    B += (torch.tensor(A.data, dtype=td, device="cuda"),)
+    w = torch.tensor(np.concatenate([rng.random(ncols), np.zeros(32 - ncols)]), device="cuda")
+    return B, torch.tensor(cf.astype(np.uint8), device="cuda"), torch.tensor(cidx.astype(np.int32), device="cuda"), X, w
+
+
+@pytest.mark.parametrize("kind,n", [("grid", 1), ("grid", 1023), ("grid", 9001), ("ring", 2001), ("hubs", 1500),
+                                    ("hubs", 7000)])
+@pytest.mark.parametrize("ncols,ld,offset,c,z,mmax,dtype", [
+    (1, 4, 0, 1, 1, 16, "fp32"), (8, 8, 0, 2, 2, 16, "fp32"), (9, 12, 0, 2, 2, 5, "fp32"), (16, 17, 0, 2, 2, 16, "fp32"),
+    (20, 20, 1, 2, 2, 16, "fp32"), (24, 24, 0, 2, 3, 16, "fp32"), (31, 32, 0, 2, 2, 16, "fp32"), (12, 12, 0, 4, 2, 16, "fp32"),
+    (10, 10, 0, 2, 2, 16, "fp64"), (17, 18, 0, 3, 1, 16, "fp64"), (5, 5, 1, 2, 3, 1, "fp64")])
+def test_interpolation_rows_equal_the_recording_path(kind, n, ncols, ld, offset, c, z, mmax, dtype):
+    """interp_ls (searches and fits in two kernels, two points a warp) against interp_features, whose
+    kernel takes a point a warp and also writes its rows by candidate: the same rows bit for bit, over
+    short and long rows, lists that overflow, odd sizes, alignments and column counts."""
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+
+    B, cf, cidx, X, w = _level(kind, n, ncols, ld, dtype, offset, seed=n + ncols)
+    pcol, pval, pcnt = bamg.interp_ls(B, cf, cidx, X, ncols, w, z=z, mmax=mmax, c=c, ridge=1e-4)
+    _, tgt, cand = bamg.interp_features(B, cf, cidx, X, ncols, w, z=z, mmax=mmax, c=c, ridge=1e-4, targets=True)
+    pcol, pval, pcnt, tgt, cand = (t.cpu().numpy() for t in (pcol, pval, pcnt, tgt, cand))
+    cidx_h, cf_h = cidx.cpu().numpy(), cf.cpu().numpy().astype(bool)
+    assert (pcnt[cf_h] == 1).all() and (pcol[cf_h, 0] == cidx_h[cf_h]).all() and (pval[cf_h, 0] == 1).all()
+    for i in np.flatnonzero(~cf_h):
+        slots = np.flatnonzero(tgt[i])
+        assert len(slots) == pcnt[i] and (pcol[i, pcnt[i]:] == -1).all() and (pval[i, pcnt[i]:] == 0).all()
+        cols = cidx_h[cand[i, slots]]
+        order = np.argsort(cols)
+        assert np.array_equal(cols[order], pcol[i, :pcnt[i]])
+        assert np.array_equal(tgt[i, slots][order], pval[i, :pcnt[i]].astype(np.float32))
