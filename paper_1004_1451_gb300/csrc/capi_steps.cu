@@ -154,25 +154,9 @@ static void galerkin_step(const bamg_mat* Bm, const void* T_val, int nc, const i
                           int64_t cap, int64_t* h_nnz, cudaStream_t s) {
     MatView<T> B = view<T>(Bm);
     EllView<T> P{B.n, c, pcol, (const T*)pval, pcnt};
-    cudaStream_t prev = alloc_stream();
-    alloc_stream() = s;
-    struct Restore {
-        cudaStream_t p;
-        ~Restore() { alloc_stream() = p; }
-    } restore_{prev};
-    DevBuf<int32_t> qrp, qci;
-    DevBuf<T> qv;
-    build_restriction<T>(P, nc, qrp, qci, qv, s);
-    GalerkinOut<T> go;
-    galerkin<T>(B, (const T*)T_val, qrp.get(), qci.get(), qv.get(), P, nc, go, s);
-    if (h_nnz) *h_nnz = go.nnz;
-    if (cap < go.nnz) throw Error(BAMG_ESIZE, "galerkin: output capacity too small");
-    BAMG_REQUIRE(out_rp && out_ci && out_bv, BAMG_EINVAL, "null output");
-    BAMG_CK(cudaMemcpyAsync(out_rp, go.rp.get(), sizeof(int32_t) * (nc + 1), cudaMemcpyDeviceToDevice, s));
-    BAMG_CK(cudaMemcpyAsync(out_ci, go.ci.get(), sizeof(int32_t) * go.nnz, cudaMemcpyDeviceToDevice, s));
-    BAMG_CK(cudaMemcpyAsync(out_bv, go.bv.get(), sizeof(T) * go.nnz, cudaMemcpyDeviceToDevice, s));
-    if (out_tv) BAMG_CK(cudaMemcpyAsync(out_tv, go.tv.get(), sizeof(T) * go.nnz, cudaMemcpyDeviceToDevice, s));
-    BAMG_CK(cudaStreamSynchronize(s));
+    const int64_t nnz = galerkin_into<T>(B, (const T*)T_val, P, nc, out_rp, out_ci, (T*)out_bv, (T*)out_tv, cap, s);
+    if (h_nnz) *h_nnz = nnz;
+    if (cap < nnz) throw Error(BAMG_ESIZE, "galerkin: output capacity too small");
 }
 }  // namespace bamg
 

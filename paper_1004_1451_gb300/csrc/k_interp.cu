@@ -1384,19 +1384,24 @@ __global__ void k_q_sort(int nc, const int32_t* __restrict__ qrp, int32_t* __res
     for (int p = a; p < b; ++p) qv[p] = inv(pcnt[qci[p]]);
 }
 
+// Q's row pointers and (unsorted) entries; cnt and cursor: nc ints of scratch each, adjacent
+static void restriction_pattern(int n, int c, const int32_t* pcol, const int32_t* pcnt, int nc, int32_t* cnt,
+                                int32_t* qrp, int32_t* qci, cudaStream_t s) {
+    BAMG_CK(cudaMemsetAsync(cnt, 0, 2 * sizeof(int32_t) * nc, s));
+    BAMG_LAUNCH(k_q_count, blocks_for(n, 256), 256, 0, s, n, c, pcol, pcnt, cnt);
+    exclusive_scan(cnt, qrp, nc, s);
+    BAMG_LAUNCH(k_q_fill, blocks_for(n, 256), 256, 0, s, n, c, pcol, pcnt, (const int32_t*)qrp, cnt + nc, qci);
+}
+
 template <typename T>
 void build_restriction(const EllView<T>& P, int nc, DevBuf<int32_t>& qrp, DevBuf<int32_t>& qci, DevBuf<T>& qv,
                        cudaStream_t s) {
-    TmpBuf<int32_t> cnt(nc, s), cursor(nc, s);
-    BAMG_CK(cudaMemsetAsync(cnt.get(), 0, sizeof(int32_t) * nc, s));
-    BAMG_CK(cudaMemsetAsync(cursor.get(), 0, sizeof(int32_t) * nc, s));
-    BAMG_LAUNCH(k_q_count, blocks_for(P.n, 256), 256, 0, s, P.n, P.c, P.pcol, P.pcnt, cnt.get());
+    TmpBuf<int32_t> cnt(2 * (size_t)nc, s);
     qrp.alloc(nc + 1);
-    exclusive_scan(cnt.get(), qrp.get(), nc, s);
     const size_t nq = (size_t)P.n * P.c;  // bound: every row of P has at most c entries
     qci.alloc(nq > 0 ? nq : 1);
     qv.alloc(nq > 0 ? nq : 1);
-    BAMG_LAUNCH(k_q_fill, blocks_for(P.n, 256), 256, 0, s, P.n, P.c, P.pcol, P.pcnt, qrp.get(), cursor.get(), qci.get());
+    restriction_pattern(P.n, P.c, P.pcol, P.pcnt, nc, cnt.get(), qrp.get(), qci.get(), s);
     BAMG_LAUNCH(k_q_sort<T>, blocks_for(nc, 128), 128, 0, s, nc, qrp.get(), qci.get(), qv.get(), P.pcnt);
 }
 
@@ -1468,14 +1473,16 @@ __global__ void k_gal_compact(int nc, const int32_t* __restrict__ poff, const in
 // Expansion, ordering and summation of one coarse row in one warp, in shared memory: the
 // lanes enumerate the row's (Q entry, B entry) pairs in order, each writing the products of
 // its pair at their position in the definition order (a warp prefix sum over the pairs'
-// product counts).  The products are then taken in chunks of 32 in that order: the lanes
-// of a chunk that share a J are summed by the lowest one, in lane order, onto J's running
-// sum (a slot in order of first appearance, found through a small open-addressing table),
-// so every J sums its products in definition order; the slots are finally ranked by J.
-// Rows are handled by a first kernel with room for
-// GAL_CAP_S products per warp (most rows); longer rows go to a list that a second kernel
-// accumulates in a hash table (below), and beyond its capacity through global memory
-// with a quadratic scan.
+// product counts).  Every product then finds its J's slot (in order of first appearance, through
+// a small open-addressing table) and its place among the slot's products, a counting sort lists
+// the products slot by slot, and a lane adds up one slot's products in definition order: half of
+// the warp B's, the other half T's.  The slots are finally ranked by J.
+// What bounds it in FP64 is the pipe (a warp's operation every 16 cycles, however few lanes take part):
+// summing the equal lanes of each chunk of 32 products, first B's and then T's, took 64 additions a
+// row of 115 products with a few lanes in each; a row now takes as many as its longest sum (about 30).
+// Rows are handled by a first kernel with room for GAL_CAP_S products per warp (most rows); longer
+// rows go to a list that a second kernel accumulates in a hash table (below), and beyond its capacity
+// by ranges of J.
 constexpr int GAL_WARPS_S = 4;
 constexpr int GAL_CAP_S = 256;  // a power of two: also the slots of the row's J table
 constexpr int GAL_CAP_LOG = 8;
@@ -1494,19 +1501,20 @@ struct GalArgs {
     const int32_t* pcnt;
     int c;
     const int32_t* poff;
-    int32_t* pJ;  // global product space (rows beyond the shared capacity)
-    T *pvb, *pvt;
     int32_t *ucnt, *uJ;
     T *ubv, *utv;
-    uint8_t* head;
+};
+template <typename T>
+struct GalRow {  // one warp's row: products, then their slots
+    T v[2][GAL_CAP_S];  // B's and T's products
+    int J[GAL_CAP_S], hkey[GAL_CAP_S];
+    unsigned short cnt[GAL_CAP_S], start[GAL_CAP_S];  // of a slot's products
+    unsigned char hval[GAL_CAP_S], slot[GAL_CAP_S], pos[GAL_CAP_S], order[GAL_CAP_S];
 };
 
-// One coarse row I in one warp.  local: sJ/svb/svt (products, then the row's slots), hkey
-// and hval (the J table) in shared memory, GAL_CAP_S entries each (np <= GAL_CAP_S); else
-// the products go to the global product space.
+// One coarse row I of at most GAL_CAP_S products in one warp.
 template <typename T>
-__device__ void gal_row(const GalArgs<T>& a, int I, bool local, int* sJ, T* svb, T* svt, int* hkey,
-                        unsigned char* hval) {
+__device__ void gal_row(const GalArgs<T>& a, int I, GalRow<T>& w) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const int o = a.poff[I], np = a.poff[I + 1] - o;
@@ -1552,121 +1560,94 @@ __device__ void gal_row(const GalArgs<T>& a, int I, bool local, int* sJ, T* svb,
                 const T qt = a.tv ? mul_rn(qq_, a.tv[p]) : (j == i ? qq_ : T(0));
                 for (int sl = 0; sl < cnt; ++sl) {
                     const T pv = a.pval[(int64_t)j * a.c + sl];
-                    const int J = a.pcol[(int64_t)j * a.c + sl];
                     const int e = pos0 + sl;
-                    if (local) {
-                        sJ[e] = J;
-                        svb[e] = mul_rn(qb, pv);
-                        svt[e] = mul_rn(qt, pv);
-                    } else {
-                        a.pJ[o + e] = J;
-                        a.pvb[o + e] = mul_rn(qb, pv);
-                        a.pvt[o + e] = mul_rn(qt, pv);
-                    }
+                    w.J[e] = a.pcol[(int64_t)j * a.c + sl];
+                    w.v[0][e] = mul_rn(qb, pv);
+                    w.v[1][e] = mul_rn(qt, pv);
                 }
             }
             base += __shfl_sync(0xffffffffu, incl, 31);
         }
     }
-    __syncwarp();
-    if (local) {
-        for (int e = lane; e < GAL_CAP_S; e += 32) hkey[e] = 0;  // key J + 1; 0 = free
-        __syncwarp();
-        int U = 0;  // slots so far (U <= e0: each slot took at least one earlier product)
-        for (int e0 = 0; e0 < np; e0 += 32) {
-            const int e = e0 + lane;
-            const int J = e < np ? sJ[e] : -1 - lane;
-            const unsigned grp = __match_any_sync(0xffffffffu, J);
-            const bool leader = e < np && (grp & lt) == 0u;
-            bool claimed = false;
-            unsigned h = 0;
-            T sb = T(0), st = T(0);
-            if (leader) {
-                h = ((unsigned)J * 2654435761u) >> (32 - GAL_CAP_LOG);
-                for (;;) {  // ends: the table has a free entry while U < GAL_CAP_S
-                    const int k = hkey[h];
-                    if (k == J + 1) break;
-                    if (k == 0 && atomicCAS(&hkey[h], 0, J + 1) == 0) {
-                        claimed = true;
-                        break;
-                    }
-                    h = (h + 1) & (GAL_CAP_S - 1);
-                }
-                if (claimed) {
-                    sb = svb[e];
-                    st = svt[e];
-                } else {  // J's slot from an earlier chunk (index < e0)
-                    const int u = hval[h];
-                    sb = add_rn(svb[u], svb[e]);
-                    st = add_rn(svt[u], svt[e]);
-                }
-                for (unsigned m = grp & (grp - 1u); m; m &= m - 1u) {
-                    const int pos = e0 + __ffs(m) - 1;
-                    sb = add_rn(sb, svb[pos]);
-                    st = add_rn(st, svt[pos]);
-                }
-            }
-            const unsigned cb = __ballot_sync(0xffffffffu, claimed);
-            __syncwarp();  // this chunk's products are read before slots overwrite them
-            if (leader) {
-                int u;
-                if (claimed) {
-                    u = U + __popc(cb & lt);  // < e0 + 32: a position already read
-                    hval[h] = (unsigned char)u;
-                    sJ[u] = J;
-                } else {
-                    u = hval[h];
-                }
-                svb[u] = sb;
-                svt[u] = st;
-            }
-            U += __popc(cb);
-            __syncwarp();
-        }
-        for (int u = lane; u < U; u += 32) {  // slot u goes to position rank(J) of the row
-            const int Ju = sJ[u];
-            int rank = 0;
-            for (int v = 0; v < U; ++v) rank += sJ[v] < Ju;
-            a.uJ[o + rank] = (int32_t)Ju;
-            a.ubv[o + rank] = svb[u];
-            a.utv[o + rank] = svt[u];
-        }
-        if (lane == 0) a.ucnt[I] = U;
-        __syncwarp();
-        return;
-    }
-    // products in global memory: quadratic scan
-    for (int e = lane; e < np; e += 32) {
-        const int Je = a.pJ[o + e];
-        bool hd = true;
-        for (int e2 = 0; e2 < e; ++e2)
-            if (a.pJ[o + e2] == Je) {
-                hd = false;
-                break;
-            }
-        a.head[o + e] = hd ? 1 : 0;
-    }
-    __syncwarp();
-    int cntu = 0;
-    for (int e = lane; e < np; e += 32) {
-        if (!a.head[o + e]) continue;
-        ++cntu;
-        const int Je = a.pJ[o + e];
-        int rank = 0;
-        for (int e2 = 0; e2 < np; ++e2) rank += (a.head[o + e2] && a.pJ[o + e2] < Je);
-        T sb = a.pvb[o + e], st = a.pvt[o + e];
-        for (int e2 = e + 1; e2 < np; ++e2)
-            if (a.pJ[o + e2] == Je) {
-                sb = add_rn(sb, a.pvb[o + e2]);
-                st = add_rn(st, a.pvt[o + e2]);
-            }
-        a.uJ[o + rank] = Je;
-        a.ubv[o + rank] = sb;
-        a.utv[o + rank] = st;
-    }
+    {
+        int4* h4 = reinterpret_cast<int4*>(w.hkey);  // key J + 1; 0 = free
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) cntu += __shfl_xor_sync(0xffffffffu, cntu, off);
-    if (lane == 0) a.ucnt[I] = cntu;
+        for (int e = 0; e < GAL_CAP_S / 128; ++e) h4[32 * e + lane] = make_int4(0, 0, 0, 0);
+    }
+    __syncwarp();
+    int U = 0;  // slots so far (U <= e0: each slot took at least one earlier product)
+    for (int e0 = 0; e0 < np; e0 += 32) {
+        const int e = e0 + lane;
+        const int J = e < np ? w.J[e] : -1 - lane;
+        const unsigned grp = __match_any_sync(0xffffffffu, J);
+        const bool leader = e < np && (grp & lt) == 0u;
+        bool claimed = false;
+        unsigned h = 0;
+        if (leader) {
+            h = ((unsigned)J * 2654435761u) >> (32 - GAL_CAP_LOG);
+            for (;;) {  // ends: the table has a free entry while U < GAL_CAP_S
+                const int k = w.hkey[h];
+                if (k == J + 1) break;
+                if (k == 0 && atomicCAS(&w.hkey[h], 0, J + 1) == 0) {
+                    claimed = true;
+                    break;
+                }
+                h = (h + 1) & (GAL_CAP_S - 1);
+            }
+        }
+        const unsigned cb = __ballot_sync(0xffffffffu, claimed);
+        __syncwarp();  // this chunk's J are read before slots overwrite them
+        int u = 0, before = 0;
+        if (leader) {
+            if (claimed) {
+                u = U + __popc(cb & lt);  // < e0 + 32: a position already read
+                w.hval[h] = (unsigned char)u;
+                w.J[u] = J;
+            } else {
+                u = w.hval[h];
+                before = w.cnt[u];
+            }
+            w.cnt[u] = (unsigned short)(before + __popc(grp));
+        }
+        const int src = __ffs(grp) - 1;
+        u = __shfl_sync(0xffffffffu, u, src);
+        before = __shfl_sync(0xffffffffu, before, src);
+        if (e < np) {
+            w.slot[e] = (unsigned char)u;
+            w.pos[e] = (unsigned char)(before + __popc(grp & lt));
+        }
+        U += __popc(cb);
+        __syncwarp();
+    }
+    int run = 0;
+    for (int u0 = 0; u0 < U; u0 += 32) {  // starts of the slots' products
+        const int u = u0 + lane, cnt = u < U ? w.cnt[u] : 0;
+        int incl = cnt;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += v;
+        }
+        if (u < U) w.start[u] = (unsigned short)(run + incl - cnt);
+        run += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    __syncwarp();
+    for (int e = lane; e < np; e += 32) w.order[w.start[w.slot[e]] + w.pos[e]] = (unsigned char)e;
+    __syncwarp();
+    const int h = lane >> 4;  // 0: B's products, 1: T's
+    const T* val = w.v[h];
+    for (int u = lane & 15; u < U; u += 16) {  // slot u goes to position rank(J) of the row
+        const int Ju = w.J[u];
+        const unsigned char* ord = w.order + w.start[u];
+        const int cnt = w.cnt[u];
+        T x = val[ord[0]];
+        for (int k = 1; k < cnt; ++k) x = add_rn(x, val[ord[k]]);
+        int rank = 0;
+        for (int v = 0; v < U; ++v) rank += w.J[v] < Ju;
+        (h ? a.utv : a.ubv)[o + rank] = x;
+        if (h == 0) a.uJ[o + rank] = (int32_t)Ju;
+    }
+    if (lane == 0) a.ucnt[I] = U;
     __syncwarp();
 }
 
@@ -1675,9 +1656,7 @@ template <typename T>
 __global__ void __launch_bounds__(GAL_WARPS_S * 32)
     k_gal_small(const __grid_constant__ GalArgs<T> a, int32_t* __restrict__ list, int* __restrict__ nlist) {
     pdl_begin();
-    __shared__ int sJ[GAL_WARPS_S][GAL_CAP_S], hkey[GAL_WARPS_S][GAL_CAP_S];
-    __shared__ T svb[GAL_WARPS_S][GAL_CAP_S], svt[GAL_WARPS_S][GAL_CAP_S];
-    __shared__ unsigned char hval[GAL_WARPS_S][GAL_CAP_S];
+    __shared__ alignas(16) GalRow<T> s_row[GAL_WARPS_S];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int I = blockIdx.x * GAL_WARPS_S + wid;
     if (I >= a.nc) return;
@@ -1686,7 +1665,7 @@ __global__ void __launch_bounds__(GAL_WARPS_S * 32)
         if (lane == 0) list[atomicAdd(nlist, 1)] = I;
         return;
     }
-    gal_row<T>(a, I, true, sJ[wid], svb[wid], svt[wid], hkey[wid], hval[wid]);
+    gal_row<T>(a, I, s_row[wid]);
 }
 
 // Long rows by accumulation instead of sorting: the products of each batch of 32 (Q, B)
@@ -1694,7 +1673,7 @@ __global__ void __launch_bounds__(GAL_WARPS_S * 32)
 // then find or claim their J in an open-addressing table (GAL_HSLOTS slots), the lanes
 // that share a J in a chunk are summed by the lowest one in lane order, so every J
 // accumulates its products in definition order.  The table's entries are finally sorted
-// by J.  A row with more distinct J than half the table goes to the quadratic scan.
+// by J.  A row with more distinct J than half the table is summed by ranges of J.
 constexpr int GAL_HSLOTS = 2048;
 constexpr int GAL_STAGE = 32 * 4;  // products of one batch of pairs (caliber <= 4)
 
@@ -1791,7 +1770,7 @@ __device__ bool gal_row_hash(const GalArgs<T>& a, int I, int* hkey, T* hvb, T* h
             used += __popc(__ballot_sync(0xffffffffu, claimed));
             __syncwarp();
         }
-        if (used > GAL_HSLOTS / 2) return false;  // too many distinct J: quadratic fallback
+        if (used > GAL_HSLOTS / 2) return false;  // too many distinct J: by ranges of J
     }
     // compact the occupied slots, sort by J, write the row
     int u = 0;
@@ -1835,6 +1814,74 @@ __device__ bool gal_row_hash(const GalArgs<T>& a, int I, int* hkey, T* hvb, T* h
     return true;
 }
 
+// A row of any length: the products with J in [lo, lo + GAL_HSLOTS) are added in definition order
+// into a table indexed by J - lo, lo starting at the row's smallest J not yet done; each range's
+// entries come out in order of J.
+template <typename T>
+__device__ void gal_row_ranges(const GalArgs<T>& a, int I, int* seen, T* tvb, T* tvt) {
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int o = a.poff[I], q0 = a.qrp[I], q1 = a.qrp[I + 1];
+    int done = 0, lo = 0;  // entries written; J below lo are done
+    for (;;) {
+        int mn = 0x7fffffff;  // the smallest J >= lo
+        for (int q = q0; q < q1; ++q) {
+            const int i = a.qci[q];
+            for (int p = a.rp[i] + lane; p < a.rp[i + 1]; p += 32) {
+                const int j = a.ci[p];
+                for (int sl = 0; sl < a.pcnt[j]; ++sl) {
+                    const int J = a.pcol[(int64_t)j * a.c + sl];
+                    if (J >= lo && J < mn) mn = J;
+                }
+            }
+        }
+        mn = __reduce_min_sync(0xffffffffu, mn);
+        if (mn == 0x7fffffff) break;
+        lo = mn;
+        for (int e = lane; e < GAL_HSLOTS; e += 32) {
+            seen[e] = 0;
+            tvb[e] = T(0);
+            tvt[e] = T(0);
+        }
+        __syncwarp();
+        for (int q = q0; q < q1; ++q) {
+            const int i = a.qci[q];
+            const T qq = a.qv[q];
+            for (int p = a.rp[i]; p < a.rp[i + 1] && lane == 0; ++p) {  // (rows this long are rare)
+                const int j = a.ci[p];
+                const T qb = mul_rn(qq, a.bv[p]), qt = a.tv ? mul_rn(qq, a.tv[p]) : (j == i ? qq : T(0));
+                for (int sl = 0; sl < a.pcnt[j]; ++sl) {
+                    const int J = a.pcol[(int64_t)j * a.c + sl];
+                    if (J < lo || J - lo >= GAL_HSLOTS) continue;
+                    const T pv = a.pval[(int64_t)j * a.c + sl];
+                    const T vb = mul_rn(qb, pv), vt = mul_rn(qt, pv);
+                    const bool first = seen[J - lo] == 0;
+                    tvb[J - lo] = first ? vb : add_rn(tvb[J - lo], vb);
+                    tvt[J - lo] = first ? vt : add_rn(tvt[J - lo], vt);
+                    seen[J - lo] = 1;
+                }
+            }
+        }
+        __syncwarp();
+        for (int e0 = 0; e0 < GAL_HSLOTS; e0 += 32) {
+            const int e = e0 + lane;
+            const unsigned bal = __ballot_sync(0xffffffffu, seen[e] != 0);
+            if (seen[e]) {
+                const int at = o + done + __popc(bal & lt);
+                a.uJ[at] = lo + e;
+                a.ubv[at] = tvb[e];
+                a.utv[at] = tvt[e];
+            }
+            done += __popc(bal);
+        }
+        __syncwarp();
+        if (lo > 0x7fffffff - GAL_HSLOTS) break;
+        lo += GAL_HSLOTS;
+    }
+    if (lane == 0) a.ucnt[I] = done;
+    __syncwarp();
+}
+
 // the listed rows, one warp per block, persistent over the list
 template <typename T>
 __global__ void __launch_bounds__(32) k_gal_large(const __grid_constant__ GalArgs<T> a,
@@ -1851,64 +1898,231 @@ __global__ void __launch_bounds__(32) k_gal_large(const __grid_constant__ GalArg
     const int cnt = *nlist;
     for (int k = blockIdx.x; k < cnt; k += gridDim.x) {
         const int I = list[k];
-        if (!gal_row_hash<T>(a, I, hkey, hvb, hvt, sJ, sb_, st_, skeys)) gal_row<T>(a, I, false, nullptr, nullptr, nullptr, nullptr, nullptr);
+        if (!gal_row_hash<T>(a, I, hkey, hvb, hvt, sJ, sb_, st_, skeys)) gal_row_ranges<T>(a, I, hkey, hvb, hvt);
     }
+}
+
+// The number of entries of B_c alone (the sizing call): every row's distinct J, counted by inserting
+// them into a table of GAL_SYM_S slots a warp (a row that fills three quarters of it goes to `list`),
+// or of GAL_SYM_L slots a block; a row that fills that too sets *over.
+constexpr int GAL_SYM_S = 512, GAL_SYM_L = 8192;
+constexpr int GAL_SYM_SUMS = 64;  // partial totals, a sector apart: one address would take every row in turn
+template <int HS, int THREADS>
+__device__ __forceinline__ int gal_distinct(int I, const int32_t* __restrict__ qrp, const int32_t* __restrict__ qci,
+                                            const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                                            const int32_t* __restrict__ pcol, const int32_t* __restrict__ pcnt, int c,
+                                            int t, int* table, volatile int* full) {
+    int mine = 0;  // J this thread claimed
+    const int q1 = qrp[I + 1];
+    constexpr int G = 8, R = THREADS / G;  // eight lanes walk a row of B
+    for (int q = qrp[I] + t / G; q < q1; q += R) {
+        const int i = qci[q], pe = rp[i + 1];
+        for (int p = rp[i] + (t & (G - 1)); p < pe; p += G) {
+            const int j = ci[p], m = pcnt[j];
+            for (int sl = 0; sl < m; ++sl) {
+                const int J = pcol[(int64_t)j * c + sl];
+                unsigned h = ((unsigned)J * 2654435761u) >> (__clz(HS) + 1);
+                for (int probe = 0; probe < HS; ++probe, h = (h + 1) & (HS - 1)) {
+                    int k = ((volatile int*)table)[h];
+                    if (k == -1) {
+                        k = atomicCAS(&table[h], -1, J);
+                        if (k == -1) ++mine;
+                    }
+                    if (k == -1 || k == J) break;
+                    if (probe == HS / 4) *full = 1;  // long probes: the table is filling up
+                }
+                if (*full) return mine;
+            }
+        }
+    }
+    return mine;
+}
+__global__ void __launch_bounds__(GAL_WARPS_S * 32)
+    k_gal_sym(int nc, const int32_t* __restrict__ qrp, const int32_t* __restrict__ qci, const int32_t* __restrict__ rp,
+              const int32_t* __restrict__ ci, const int32_t* __restrict__ pcol, const int32_t* __restrict__ pcnt, int c,
+              int32_t* __restrict__ list, int* __restrict__ nlist, int* __restrict__ total) {
+    pdl_begin();
+    __shared__ alignas(16) int s_table[GAL_WARPS_S][GAL_SYM_S];
+    __shared__ int s_full[GAL_WARPS_S];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int I = blockIdx.x * GAL_WARPS_S + wid;
+    if (I >= nc) return;
+    int4* t4 = reinterpret_cast<int4*>(s_table[wid]);
+#pragma unroll
+    for (int e = 0; e < GAL_SYM_S / 128; ++e) t4[32 * e + lane] = make_int4(-1, -1, -1, -1);
+    if (lane == 0) s_full[wid] = 0;
+    __syncwarp();
+    int m = gal_distinct<GAL_SYM_S, 32>(I, qrp, qci, rp, ci, pcol, pcnt, c, lane, s_table[wid], &s_full[wid]);
+    __syncwarp();
+    m = __reduce_add_sync(0xffffffffu, m);
+    if (lane == 0) {
+        if (s_full[wid])
+            list[atomicAdd(nlist, 1)] = I;
+        else
+            atomicAdd(total + 8 * (blockIdx.x % GAL_SYM_SUMS), m);
+    }
+}
+__global__ void __launch_bounds__(256)
+    k_gal_sym_large(const int32_t* __restrict__ qrp, const int32_t* __restrict__ qci, const int32_t* __restrict__ rp,
+                    const int32_t* __restrict__ ci, const int32_t* __restrict__ pcol, const int32_t* __restrict__ pcnt,
+                    int c, const int32_t* __restrict__ list, const int* __restrict__ nlist, int* __restrict__ total,
+                    int* __restrict__ over) {
+    pdl_begin();
+    __shared__ int s_table[GAL_SYM_L];
+    __shared__ int s_full, s_sum;
+    const int cnt = *nlist;
+    for (int k = blockIdx.x; k < cnt; k += gridDim.x) {
+        __syncthreads();
+        for (int e = threadIdx.x; e < GAL_SYM_L; e += blockDim.x) s_table[e] = -1;
+        if (threadIdx.x == 0) s_full = s_sum = 0;
+        __syncthreads();
+        const int m = gal_distinct<GAL_SYM_L, 256>(list[k], qrp, qci, rp, ci, pcol, pcnt, c, threadIdx.x, s_table, &s_full);
+        atomicAdd(&s_sum, m);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            if (s_full)
+                *over = 1;
+            else
+                atomicAdd(total, s_sum);
+        }
+    }
+}
+
+// 256-byte aligned slices of one temporary
+struct Slices {
+    size_t used = 0;
+    size_t add(size_t bytes) {
+        const size_t at = used;
+        used += (bytes + 255) & ~size_t(255);
+        return at;
+    }
+};
+// The products of B_c and T_c row by row (at the rows' product offsets poff, ucnt entries each).
+template <typename T>
+struct GalProducts {
+    size_t tot;
+    Slices sl;
+    size_t o_np, o_poff, o_ucnt, o_list, o_nlist, o_uJ, o_ubv, o_utv;
+    GalProducts(const MatView<T>& B, int nc, int c) {
+        // bound on the product count: each entry b_ij meets at most c columns of Q and c rows of P
+        const size_t bound = (size_t)B.nnz * c * c;
+        BAMG_REQUIRE(bound < (size_t)INT32_MAX, BAMG_EINVAL, "galerkin: product count may overflow int32");
+        tot = bound > 0 ? bound : 1;
+        o_np = sl.add(sizeof(int32_t) * nc);
+        o_poff = sl.add(sizeof(int32_t) * ((size_t)nc + 1));
+        o_ucnt = sl.add(sizeof(int32_t) * nc);
+        o_list = sl.add(sizeof(int32_t) * nc);
+        o_nlist = sl.add(sizeof(int));
+        o_uJ = sl.add(sizeof(int32_t) * tot);
+        o_ubv = sl.add(sizeof(T) * tot);
+        o_utv = sl.add(sizeof(T) * tot);
+    }
+    GalArgs<T> run(char* w, const MatView<T>& B, const T* T_val, const int32_t* qrp, const int32_t* qci, const T* qv,
+                   const EllView<T>& P, int nc, cudaStream_t s) const {
+        int32_t *np = (int32_t*)(w + o_np), *poff = (int32_t*)(w + o_poff), *list = (int32_t*)(w + o_list);
+        int* nlist = (int*)(w + o_nlist);
+        BAMG_LAUNCH(k_gal_count, blocks_for(nc, GAL_COUNT_WARPS), GAL_COUNT_WARPS * 32, 0, s, nc, qrp, qci, B.rp, B.ci,
+                    P.pcnt, np);
+        exclusive_scan(np, poff, nc, s);
+        const GalArgs<T> ga{nc,     qrp, qci,  qv, B.rp, B.ci, B.v, T_val, P.pcol, P.pval, P.pcnt, P.c, poff,
+                            (int32_t*)(w + o_ucnt), (int32_t*)(w + o_uJ), (T*)(w + o_ubv), (T*)(w + o_utv)};
+        BAMG_CK(cudaMemsetAsync(nlist, 0, sizeof(int), s));
+        BAMG_LAUNCH(k_gal_small<T>, blocks_for(nc, GAL_WARPS_S), GAL_WARPS_S * 32, 0, s, ga, list, nlist);
+        auto large_smem = [](size_t tb) {
+            return (size_t)GAL_HSLOTS * (sizeof(unsigned long long) + 2 * tb + sizeof(int)) +
+                   GAL_STAGE * (2 * tb + sizeof(int));
+        };
+        static std::atomic<bool> attr[256] = {};  // per device; idempotent across host threads
+        int dev = 0;
+        BAMG_CK(cudaGetDevice(&dev));
+        BAMG_REQUIRE(dev >= 0 && dev < 256, BAMG_EINVAL, "device ordinal out of range");
+        if (!attr[dev]) {
+            BAMG_CK(cudaFuncSetAttribute(k_gal_large<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)large_smem(sizeof(T))));
+            attr[dev] = true;
+        }
+        BAMG_LAUNCH(k_gal_large<T>, GAL_BLOCKS_L, 32, large_smem(sizeof(T)), s, ga, (const int32_t*)list,
+                    (const int*)nlist);
+        return ga;
+    }
+};
+template <typename T>
+static void gal_compact(const GalArgs<T>& ga, const int32_t* rp, int32_t* ci, T* bv, T* tv, cudaStream_t s) {
+    BAMG_LAUNCH(k_gal_compact<T>, blocks_for(ga.nc, GAL_COUNT_WARPS), GAL_COUNT_WARPS * 32, 0, s, ga.nc, ga.poff, ga.ucnt,
+                rp, ga.uJ, ga.ubv, ga.utv, ci, bv, tv);
 }
 
 template <typename T>
 void galerkin(const MatView<T>& B, const T* T_val, const int32_t* qrp, const int32_t* qci, const T* qv,
               const EllView<T>& P, int nc, GalerkinOut<T>& out, cudaStream_t s, bool defer) {
-    TmpBuf<int32_t> np(nc, s), poff(nc + 1, s);
-    BAMG_LAUNCH(k_gal_count, blocks_for(nc, GAL_COUNT_WARPS), GAL_COUNT_WARPS * 32, 0, s, nc, qrp, qci, B.rp, B.ci,
-                P.pcnt, np.get());
-    exclusive_scan(np.get(), poff.get(), nc, s);
-    // bound on the product count: each entry b_ij meets at most c columns of Q and c rows of P
-    const size_t bound = (size_t)B.nnz * P.c * P.c;
-    BAMG_REQUIRE(bound < (size_t)INT32_MAX, BAMG_EINVAL, "galerkin: product count may overflow int32");
-    const size_t tot = bound > 0 ? bound : 1;
-    TmpBuf<int32_t> pJ(tot, s), uJ(tot, s), ucnt(nc, s);
-    TmpBuf<T> pvb(tot, s), pvt(tot, s), ubv(tot, s), utv(tot, s);
-    TmpBuf<uint8_t> head(tot, s);
-    GalArgs<T> ga{nc,     qrp,    qci, qv,         B.rp,     B.ci,      B.v,       T_val,      P.pcol,   P.pval,
-                  P.pcnt, P.c,    poff.get(), pJ.get(), pvb.get(), pvt.get(), ucnt.get(), uJ.get(), ubv.get(),
-                  utv.get(), head.get()};
-    TmpBuf<int32_t> list(nc, s);
-    TmpBuf<int> nlist(1, s);
-    BAMG_CK(cudaMemsetAsync(nlist.get(), 0, sizeof(int), s));
-    BAMG_LAUNCH(k_gal_small<T>, blocks_for(nc, GAL_WARPS_S), GAL_WARPS_S * 32, 0, s, ga, list.get(), nlist.get());
-    auto large_smem = [](size_t tb) {
-        return (size_t)GAL_HSLOTS * (sizeof(unsigned long long) + 2 * tb + sizeof(int)) + GAL_STAGE * (2 * tb + sizeof(int));
-    };
-    const size_t smem_l = large_smem(sizeof(T));
-    static std::atomic<bool> attr[256] = {};  // per device; idempotent across host threads
-    int dev = 0;
-    BAMG_CK(cudaGetDevice(&dev));
-    BAMG_REQUIRE(dev >= 0 && dev < 256, BAMG_EINVAL, "device ordinal out of range");
-    if (!attr[dev]) {
-        BAMG_CK(cudaFuncSetAttribute(k_gal_large<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)large_smem(sizeof(float))));
-        BAMG_CK(cudaFuncSetAttribute(k_gal_large<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)large_smem(sizeof(double))));
-        attr[dev] = true;
-    }
-    BAMG_LAUNCH(k_gal_large<T>, GAL_BLOCKS_L, 32, smem_l, s, ga, (const int32_t*)list.get(), (const int*)nlist.get());
+    const GalProducts<T> gp(B, nc, P.c);
+    TmpBuf<char> work(gp.sl.used, s);
+    const GalArgs<T> ga = gp.run(work.get(), B, T_val, qrp, qci, qv, P, nc, s);
     out.rp.alloc(nc + 1);
-    size_t nz = tot;  // with defer: room for the bound, the count still on its way
+    size_t nz = gp.tot;  // with defer: room for the bound, the count still on its way
     // (only while the bound's arrays stay small: large ones cost more to allocate than the wait)
-    if (defer && tot * (sizeof(int32_t) + 2 * sizeof(T)) > ((size_t)64 << 20)) defer = false;
+    if (defer && gp.tot * (sizeof(int32_t) + 2 * sizeof(T)) > ((size_t)64 << 20)) defer = false;
     if (defer) {
-        exclusive_scan_total_begin(ucnt.get(), out.rp.get(), nc, s);
+        exclusive_scan_total_begin(ga.ucnt, out.rp.get(), nc, s);
         out.nnz = -1;
     } else {
-        out.nnz = exclusive_scan_total(ucnt.get(), out.rp.get(), nc, s);
+        out.nnz = exclusive_scan_total(ga.ucnt, out.rp.get(), nc, s);
         nz = out.nnz > 0 ? (size_t)out.nnz : 1;
     }
     out.ci.alloc(nz);
     out.bv.alloc(nz);
     out.tv.alloc(nz);
-    BAMG_LAUNCH(k_gal_compact<T>, blocks_for(nc, GAL_COUNT_WARPS), GAL_COUNT_WARPS * 32, 0, s, nc, poff.get(),
-                ucnt.get(), out.rp.get(), uJ.get(),
-                ubv.get(), utv.get(), out.ci.get(), out.bv.get(), out.tv.get());
+    gal_compact<T>(ga, out.rp.get(), out.ci.get(), out.bv.get(), out.tv.get(), s);
+}
+
+// The products into the caller's arrays (capacity cap; out_tv may be null).  Returns the number of
+// entries; nothing is written when it exceeds cap.  With cap 0 (the sizing call) only the number is
+// formed, from the patterns: it took as long as the products.
+template <typename T>
+int64_t galerkin_into(const MatView<T>& B, const T* T_val, const EllView<T>& P, int nc, int32_t* out_rp,
+                      int32_t* out_ci, T* out_bv, T* out_tv, int64_t cap, cudaStream_t s) {
+    const size_t nq = (size_t)P.n * P.c > 0 ? (size_t)P.n * P.c : 1;
+    if (cap == 0) {
+        Slices sl;
+        const size_t o_cnt = sl.add(2 * sizeof(int32_t) * (size_t)nc), o_qrp = sl.add(sizeof(int32_t) * ((size_t)nc + 1)),
+                     o_qci = sl.add(sizeof(int32_t) * nq), o_list = sl.add(sizeof(int32_t) * (size_t)nc),
+                     o_num = sl.add((8 + 8 * GAL_SYM_SUMS) * sizeof(int));
+        GalProducts<T> bound(B, nc, P.c);  // refuses what the products would refuse
+        TmpBuf<char> work(sl.used, s);
+        int32_t *qrp = (int32_t*)(work.get() + o_qrp), *qci = (int32_t*)(work.get() + o_qci);
+        int32_t* list = (int32_t*)(work.get() + o_list);
+        int* num = (int*)(work.get() + o_num);  // listed rows, overflow, then the partial totals
+        restriction_pattern(P.n, P.c, P.pcol, P.pcnt, nc, (int32_t*)(work.get() + o_cnt), qrp, qci, s);
+        int h[8 + 8 * GAL_SYM_SUMS];
+        BAMG_CK(cudaMemsetAsync(num, 0, sizeof h, s));
+        BAMG_LAUNCH(k_gal_sym, blocks_for(nc, GAL_WARPS_S), GAL_WARPS_S * 32, 0, s, nc, (const int32_t*)qrp,
+                    (const int32_t*)qci, B.rp, B.ci, P.pcol, P.pcnt, P.c, list, num, num + 8);
+        BAMG_LAUNCH(k_gal_sym_large, GAL_BLOCKS_L, 256, 0, s, (const int32_t*)qrp, (const int32_t*)qci, B.rp, B.ci, P.pcol,
+                    P.pcnt, P.c, (const int32_t*)list, (const int*)num, num + 8, num + 1);
+        BAMG_CK(cudaMemcpyAsync(h, num, sizeof h, cudaMemcpyDeviceToHost, s));
+        BAMG_CK(cudaStreamSynchronize(s));
+        int64_t nnz = 0;
+        for (int k = 0; k < GAL_SYM_SUMS; ++k) nnz += h[8 + 8 * k];
+        if (!h[1] && nnz > 0) return nnz;
+    }
+    GalProducts<T> gp(B, nc, P.c);
+    const size_t o_cnt = gp.sl.add(2 * sizeof(int32_t) * (size_t)nc), o_qrp = gp.sl.add(sizeof(int32_t) * ((size_t)nc + 1)),
+                 o_qci = gp.sl.add(sizeof(int32_t) * nq), o_qv = gp.sl.add(sizeof(T) * nq),
+                 o_rp = gp.sl.add(sizeof(int32_t) * ((size_t)nc + 1)), o_tv = gp.sl.add(out_tv ? 0 : sizeof(T) * gp.tot);
+    TmpBuf<char> work(gp.sl.used, s);
+    char* w = work.get();
+    int32_t *qrp = (int32_t*)(w + o_qrp), *qci = (int32_t*)(w + o_qci), *rp = (int32_t*)(w + o_rp);
+    T* qv = (T*)(w + o_qv);
+    restriction_pattern(P.n, P.c, P.pcol, P.pcnt, nc, (int32_t*)(w + o_cnt), qrp, qci, s);
+    BAMG_LAUNCH(k_q_sort<T>, blocks_for(nc, 128), 128, 0, s, nc, (const int32_t*)qrp, qci, qv, P.pcnt);
+    const GalArgs<T> ga = gp.run(w, B, T_val, qrp, qci, qv, P, nc, s);
+    const int64_t nnz = exclusive_scan_total(ga.ucnt, rp, nc, s);
+    if (cap < nnz) return nnz;
+    BAMG_REQUIRE(out_rp && out_ci && out_bv, BAMG_EINVAL, "null output");
+    BAMG_CK(cudaMemcpyAsync(out_rp, rp, sizeof(int32_t) * ((size_t)nc + 1), cudaMemcpyDeviceToDevice, s));
+    gal_compact<T>(ga, rp, out_ci, out_bv, out_tv ? out_tv : (T*)(w + o_tv), s);
+    BAMG_CK(cudaStreamSynchronize(s));
+    return nnz;
 }
 
 template <typename T>
@@ -1941,6 +2155,8 @@ void csr_to_dense(int n, const int32_t* rp, const int32_t* ci, const T* v, doubl
                                        cudaStream_t);                                                               \
     template void galerkin<T>(const MatView<T>&, const T*, const int32_t*, const int32_t*, const T*,                \
                               const EllView<T>&, int, GalerkinOut<T>&, cudaStream_t, bool);                         \
+    template int64_t galerkin_into<T>(const MatView<T>&, const T*, const EllView<T>&, int, int32_t*, int32_t*, T*,  \
+                                      T*, int64_t, cudaStream_t);                                                   \
     template void galerkin_nnz<T>(GalerkinOut<T>&, cudaStream_t);                                                   \
     template void csr_to_dense<T>(int, const int32_t*, const int32_t*, const T*, double*, cudaStream_t);
 INST(float)

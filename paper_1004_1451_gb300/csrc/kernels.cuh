@@ -135,6 +135,9 @@ struct GalerkinOut {
 template <typename T>
 void galerkin(const MatView<T>& B, const T* T_val, const int32_t* qrp, const int32_t* qci, const T* qv,
               const EllView<T>& P, int nc, GalerkinOut<T>& out, cudaStream_t s, bool defer = false);
+template <typename T>  // into the caller's arrays, or with cap 0 the number of entries alone
+int64_t galerkin_into(const MatView<T>& B, const T* T_val, const EllView<T>& P, int nc, int32_t* out_rp,
+                      int32_t* out_ci, T* out_bv, T* out_tv, int64_t cap, cudaStream_t s);
 template <typename T>
 void galerkin_nnz(GalerkinOut<T>& out, cudaStream_t s);
 template <typename T>
