@@ -230,6 +230,12 @@ int bamg_parnoldi(bamg_handle* h, double* x, int flags, double tol, bamg_stats* 
 /* Frees the handle and its device memory.  NULL is allowed. */
 void bamg_free(bamg_handle* h);
 
+/* Device memory: the library allocates from a pool of its own, which keeps up to 512 MiB of unused
+ * memory per device between calls (beyond that it is given back at each synchronisation), and keeps
+ * the private streams of up to 16 freed handles.  This call gives back, on the current device, what no
+ * handle uses; it synchronises the device.  Bookkeeping, no passage of the paper. */
+int bamg_release_memory(void);
+
 /* Message of the calling thread's last failed call ("" if none).  Static storage. */
 const char* bamg_last_error(void);
 

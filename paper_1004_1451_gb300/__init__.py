@@ -15,7 +15,7 @@ from . import _capi as capi
 from ._capi import BamgError  # noqa: F401
 
 __all__ = ["Solver", "Model", "solve_batch", "interp_dataset", "interp_features", "interp_learned", "import_hierarchy", "tv_init", "relax", "relax_noalloc", "tv_weights", "coarsen_grid", "coarsen_cr",
-           "interp_ls", "galerkin", "coarse_eig", "launch_count", "default_opts", "BamgError"]
+           "interp_ls", "galerkin", "coarse_eig", "launch_count", "release_memory", "default_opts", "BamgError"]
 
 
 def _lib():
@@ -50,6 +50,12 @@ def _mat(rp, ci, val):
 def launch_count() -> int:
     """Kernels launched by the library in this process."""
     return int(_lib().bamg_launch_count())
+
+
+def release_memory() -> None:
+    """Gives back the device memory and streams the library keeps for its next calls
+    (bamg_release_memory)."""
+    capi.check(_lib().bamg_release_memory())
 
 
 _OPT_NAMES = [f[0] for f in capi.Opts._fields_]

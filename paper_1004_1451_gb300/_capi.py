@@ -75,6 +75,7 @@ SIGNATURES = {
                               _D, _I, C.POINTER(Stats)]),
     "bamg_last_error": (C.c_char_p, []),
     "bamg_launch_count": (C.c_uint64, []),
+    "bamg_release_memory": (C.c_int, []),
     "bamg_hierarchy_info": (_I, [_P, C.POINTER(_I), _P, _P, C.POINTER(_D)]),
     "bamg_level_export": (_I, [_P, _I, _I, _P, C.c_int64, C.POINTER(C.c_int64)]),
     "bamg_hierarchy_layout": (_I, [_P, _I, C.POINTER(_I), C.POINTER(_I), C.POINTER(_I), C.POINTER(_I)]),

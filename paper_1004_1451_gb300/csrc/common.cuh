@@ -4,8 +4,10 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <map>
 #include <stdexcept>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "../../include/bamg.h"
@@ -81,55 +83,139 @@ inline unsigned blocks_for(int64_t work, int per_block) {
     return (unsigned)(b < 1 ? 1 : b);
 }
 
-// Stream on which DevBuf allocations are ordered (set by the owner of the work: the
-// handle's stream during setup and solve).  Thread-local.
-cudaStream_t& alloc_stream();
-// Sets alloc_stream() for a scope.
-struct AllocStream {
-    cudaStream_t prev;
-    explicit AllocStream(cudaStream_t s) : prev(alloc_stream()) { alloc_stream() = s; }
-    ~AllocStream() { alloc_stream() = prev; }
+// Device memory comes from a pool of the library's own (one per device, made at its first use):
+// cudaMallocAsync's default pool gives every unused byte back to the system at each
+// synchronisation, and mapping a call's temporaries again took 100 to 400 us (two thirds of a
+// galerkin call).  This pool keeps up to MEM_POOL_KEEP unused bytes at a synchronisation and gives the
+// rest back; bamg_release_memory() gives back the rest too.  Blocks are ordered by stream as
+// cudaMallocAsync's are, across threads and streams.
+constexpr uint64_t MEM_POOL_KEEP = uint64_t(512) << 20;
+void pool_alloc(void** p, size_t bytes, cudaStream_t s);
+void pool_trim();  // of the current device
+
+// A solver's small long-lived buffers: slices of chunks from the pool, given out by size and taken
+// back into a free list (at once, for buffers are reused in the order of the solver's streams, which
+// are fenced against one another).  A setup allocates some 200 of them, at 2 us each, and at 30 us with
+// eight host threads in the allocator at a time.  Blocks above MAX_SLICE come from the pool
+// directly.  The chunks are freed with the solver.
+struct DevArena {
+    static constexpr size_t MAX_SLICE = size_t(4) << 20, FIRST_CHUNK = size_t(2) << 20, MAX_CHUNK = size_t(32) << 20;
+    struct Chunk {
+        char* base;
+        size_t cap, top;
+        cudaStream_t s;
+    };
+    std::vector<Chunk> chunks;
+    std::multimap<size_t, char*> free_;
+    std::unordered_map<char*, size_t> size_;
+    void* alloc(size_t bytes, cudaStream_t s) {
+        bytes = (bytes + 255) & ~size_t(255);
+        auto it = free_.lower_bound(bytes);
+        if (it != free_.end() && it->first <= 2 * bytes) {
+            char* p = it->second;
+            free_.erase(it);
+            return p;
+        }
+        if (chunks.empty() || chunks.back().top + bytes > chunks.back().cap) {
+            const size_t next = chunks.empty() ? FIRST_CHUNK : 2 * chunks.back().cap;
+            const size_t cap = next < MAX_CHUNK ? next : MAX_CHUNK;
+            Chunk c{nullptr, cap > bytes ? cap : bytes, 0, s};
+            pool_alloc((void**)&c.base, c.cap, s);
+            chunks.push_back(c);
+        }
+        Chunk& c = chunks.back();
+        char* p = c.base + c.top;
+        c.top += bytes;
+        size_[p] = bytes;
+        return p;
+    }
+    void free(void* p) { free_.emplace(size_.at((char*)p), (char*)p); }
+    DevArena() = default;
+    ~DevArena() {
+        for (Chunk& c : chunks) cudaFreeAsync(c.base, c.s);
+    }
+    DevArena(const DevArena&) = delete;
+    DevArena& operator=(const DevArena&) = delete;
 };
 
-// Owning device buffer from the stream-ordered pool (cudaMallocAsync on alloc_stream()),
-// so building a hierarchy does not synchronise the device for every allocation.
+// Stream on which DevBuf allocations are ordered (set by the owner of the work: the
+// handle's stream during setup and solve), and the arena small ones come from (null: the pool).
+// Thread-local.
+cudaStream_t& alloc_stream();
+DevArena*& dev_arena();
+// Sets both for a scope.
+struct AllocStream {
+    cudaStream_t prev;
+    DevArena* prev_a;
+    explicit AllocStream(cudaStream_t s, DevArena* a = nullptr) : prev(alloc_stream()), prev_a(dev_arena()) {
+        alloc_stream() = s;
+        dev_arena() = a;
+    }
+    ~AllocStream() {
+        alloc_stream() = prev;
+        dev_arena() = prev_a;
+    }
+};
+
+// Owning device buffer from the arena or the pool, ordered on alloc_stream(), so building a
+// hierarchy does not synchronise the device for every allocation.
 // Callers synchronise their streams before the owner is destroyed.
 template <typename T>
 struct DevBuf {
     T* p = nullptr;
     size_t n = 0;
     cudaStream_t s = nullptr;
+    DevArena* a = nullptr;
     DevBuf() = default;
     explicit DevBuf(size_t n_) { alloc(n_); }
     void alloc(size_t n_) {
         release();
         s = alloc_stream();
-        if (n_) BAMG_CK(cudaMallocAsync((void**)&p, n_ * sizeof(T), s));
+        const size_t bytes = n_ * sizeof(T);
+        a = bytes <= DevArena::MAX_SLICE ? dev_arena() : nullptr;
+        if (n_) {
+            if (a)
+                p = static_cast<T*>(a->alloc(bytes, s));
+            else
+                pool_alloc((void**)&p, bytes, s);
+        }
         n = n_;
     }
     void ensure(size_t n_) {
         if (n_ > n) alloc(n_);
     }
     void release() {
-        if (p) cudaFreeAsync(p, s);
+        if (p) {
+            if (a)
+                a->free(p);
+            else
+                cudaFreeAsync(p, s);
+        }
         p = nullptr;
         n = 0;
     }
     ~DevBuf() { release(); }
     DevBuf(const DevBuf&) = delete;
     DevBuf& operator=(const DevBuf&) = delete;
-    DevBuf(DevBuf&& o) noexcept : p(o.p), n(o.n), s(o.s) { o.p = nullptr; o.n = 0; }
+    DevBuf(DevBuf&& o) noexcept : p(o.p), n(o.n), s(o.s), a(o.a) { o.p = nullptr; o.n = 0; }
     DevBuf& operator=(DevBuf&& o) noexcept {
         release();
         p = o.p;
         n = o.n;
         s = o.s;
+        a = o.a;
         o.p = nullptr;
         o.n = 0;
         return *this;
     }
     T* get() const { return p; }
 };
+
+// A block of mapped pinned host memory (PINNED_SLOT bytes), from pages that live as long as the
+// process: a cudaHostAlloc takes 130 us and stops the other threads' allocations.
+constexpr size_t PINNED_SLOT = 256;
+void* pinned_acquire();
+void pinned_release(void* p);
 
 // Stack allocator for the temporaries of one stream: chunks from the stream-ordered pool,
 // handed out in 256-byte aligned slices and taken back when the slices are released (any
@@ -150,7 +236,7 @@ struct StackArena {
     cudaStream_t s;
     std::vector<Chunk> chunks;
     std::vector<Slice> stack;
-    static constexpr size_t MIN_CHUNK = size_t(64) << 20;
+    static constexpr size_t MIN_CHUNK = size_t(16) << 20;
     explicit StackArena(cudaStream_t st) : s(st) {}
     void* push(size_t bytes) {
         bytes = (bytes + 255) & ~size_t(255);
@@ -158,7 +244,7 @@ struct StackArena {
         while (c < chunks.size() && chunks[c].top + bytes > chunks[c].cap) ++c;
         if (c == chunks.size()) {
             Chunk k{nullptr, bytes > MIN_CHUNK ? bytes : MIN_CHUNK, 0};
-            BAMG_CK(cudaMallocAsync((void**)&k.base, k.cap, s));
+            pool_alloc((void**)&k.base, k.cap, s);
             chunks.push_back(k);
         }
         Chunk& k = chunks[c];
@@ -216,7 +302,7 @@ struct TmpBuf {
             a = cur;
             p = static_cast<T*>(a->push(n * sizeof(T)));
         } else {
-            BAMG_CK(cudaMallocAsync((void**)&p, n * sizeof(T), s));
+            pool_alloc((void**)&p, n * sizeof(T), s);
         }
     }
     ~TmpBuf() {

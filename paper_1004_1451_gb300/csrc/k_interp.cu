@@ -171,6 +171,9 @@ __global__ void __launch_bounds__(SCAN_ONE_T) k_scan_one(const int32_t* in, int3
 struct HostWord {
     int32_t* h = nullptr;
     int32_t* d = nullptr;
+    ~HostWord() {  // at the thread's end
+        if (h) pinned_release(h);
+    }
 };
 static HostWord& host_word() {
     thread_local HostWord w[64];
@@ -179,7 +182,7 @@ static HostWord& host_word() {
     BAMG_REQUIRE(dev >= 0 && dev < 64, BAMG_EINVAL, "device ordinal out of range");
     HostWord& hw = w[dev];
     if (!hw.h) {
-        BAMG_CK(cudaHostAlloc((void**)&hw.h, 64, cudaHostAllocMapped | cudaHostAllocPortable));
+        hw.h = static_cast<int32_t*>(pinned_acquire());
         BAMG_CK(cudaHostGetDevicePointer((void**)&hw.d, hw.h, 0));
     }
     return hw;

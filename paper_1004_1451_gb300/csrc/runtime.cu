@@ -44,6 +44,141 @@ cudaStream_t& alloc_stream() {
     static thread_local cudaStream_t st = nullptr;
     return st;
 }
+DevArena*& dev_arena() {
+    static thread_local DevArena* a = nullptr;
+    return a;
+}
+
+// ---------------------------------------------------------------- memory and streams kept
+static int current_device() {
+    int dev = 0;
+    BAMG_CK(cudaGetDevice(&dev));
+    BAMG_REQUIRE(dev >= 0 && dev < 64, BAMG_EINVAL, "device ordinal out of range");
+    return dev;
+}
+static std::atomic<cudaMemPool_t> g_pool[64] = {};
+static cudaMemPool_t mem_pool() {
+    const int dev = current_device();
+    cudaMemPool_t pool = g_pool[dev].load(std::memory_order_acquire);
+    if (pool) return pool;
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    pool = g_pool[dev].load();
+    if (pool) return pool;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    BAMG_CK(cudaMemPoolCreate(&pool, &props));
+    uint64_t keep = MEM_POOL_KEEP;
+    BAMG_CK(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
+    // no search for blocks that other streams happen to have finished with: after eight threads'
+    // streams had used the pool, that search took 12 us an allocation (a cr call 507 us instead of 264)
+    int off = 0;
+    BAMG_CK(cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowOpportunistic, &off));
+    g_pool[dev].store(pool, std::memory_order_release);
+    return pool;
+}
+void pool_alloc(void** p, size_t bytes, cudaStream_t s) { BAMG_CK(cudaMallocFromPoolAsync(p, bytes, mem_pool(), s)); }
+
+// The private streams of solvers that are gone, with their fence events: up to STREAMS_KEPT per
+// device (creating them takes some 50 us a solver).
+struct StreamSet {
+    cudaStream_t ps = nullptr;
+    cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+};
+static void destroy(const StreamSet& k) {
+    if (k.ev_in) cudaEventDestroy(k.ev_in);
+    if (k.ev_out) cudaEventDestroy(k.ev_out);
+    if (k.ps) cudaStreamDestroy(k.ps);
+}
+constexpr size_t STREAMS_KEPT = 16;
+struct KeptStreams {
+    std::mutex mu;
+    std::vector<StreamSet> sets[64];
+};
+static KeptStreams& kept_streams() {
+    static KeptStreams* k = new KeptStreams;  // never destroyed: the driver may be gone by then
+    return *k;
+}
+static StreamSet acquire_streams(int dev) {
+    {
+        KeptStreams& k = kept_streams();
+        std::lock_guard<std::mutex> lock(k.mu);
+        if (!k.sets[dev].empty()) {
+            const StreamSet s = k.sets[dev].back();
+            k.sets[dev].pop_back();
+            return s;
+        }
+    }
+    StreamSet s;
+    try {
+        BAMG_CK(cudaStreamCreateWithFlags(&s.ps, cudaStreamNonBlocking));
+        BAMG_CK(cudaEventCreateWithFlags(&s.ev_in, cudaEventDisableTiming));
+        BAMG_CK(cudaEventCreateWithFlags(&s.ev_out, cudaEventDisableTiming));
+    } catch (...) {
+        destroy(s);
+        throw;
+    }
+    return s;
+}
+// s: synchronised, nothing pending
+static void keep_streams(int dev, const StreamSet& s) {
+    KeptStreams& k = kept_streams();
+    {
+        std::lock_guard<std::mutex> lock(k.mu);
+        if (k.sets[dev].size() < STREAMS_KEPT) {
+            k.sets[dev].push_back(s);
+            return;
+        }
+    }
+    destroy(s);
+}
+// the current device's unused pool memory and kept streams
+void pool_trim() {
+    const int dev = current_device();
+    std::vector<StreamSet> drop;
+    {
+        KeptStreams& k = kept_streams();
+        std::lock_guard<std::mutex> lock(k.mu);
+        drop.swap(k.sets[dev]);
+    }
+    for (const StreamSet& s : drop) destroy(s);
+    cudaMemPool_t pool = g_pool[dev].load();
+    if (pool) {
+        BAMG_CK(cudaDeviceSynchronize());
+        BAMG_CK(cudaMemPoolTrimTo(pool, 0));
+    }
+}
+
+struct PinnedPages {
+    std::mutex mu;
+    std::vector<void*> free_;
+};
+static PinnedPages& pinned_pages() {
+    static PinnedPages* p = new PinnedPages;
+    return *p;
+}
+void* pinned_acquire() {
+    PinnedPages& g = pinned_pages();
+    std::lock_guard<std::mutex> lock(g.mu);
+    if (g.free_.empty()) {
+        constexpr size_t PAGE = 64 * PINNED_SLOT;
+        char* page = nullptr;
+        BAMG_CK(cudaHostAlloc((void**)&page, PAGE, cudaHostAllocMapped | cudaHostAllocPortable));
+        for (size_t o = 0; o < PAGE; o += PINNED_SLOT) g.free_.push_back(page + o);
+    }
+    void* p = g.free_.back();
+    g.free_.pop_back();
+    return p;
+}
+void pinned_release(void* p) {
+    PinnedPages& g = pinned_pages();
+    std::lock_guard<std::mutex> lock(g.mu);
+    g.free_.push_back(p);
+}
+
 StackArena*& tmp_arena() {
     static thread_local StackArena* a = nullptr;
     return a;
@@ -175,22 +310,27 @@ struct PhaseTrace {
 // is destroyed after every device buffer of the derived solver: buffers (re)allocated
 // during a solve (the MLE restart's rebuilt levels) are released on this stream.
 struct PrivateStream {
-    cudaStream_t ps = nullptr;
-    cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+    StreamSet k;
+    int dev = -1;
     ~PrivateStream() {
-        if (ps) cudaStreamSynchronize(ps);
-        if (ev_in) cudaEventDestroy(ev_in);
-        if (ev_out) cudaEventDestroy(ev_out);
-        if (ps) cudaStreamDestroy(ps);
+        if (!k.ps) return;
+        if (cudaStreamSynchronize(k.ps) == cudaSuccess)
+            keep_streams(dev, k);
+        else
+            destroy(k);
     }
 };
 
 struct SolverBase {
     PrivateStream priv;  // first member: destroyed last
+    DevArena darena;     // then the small buffers' memory
+    double* h_pin = nullptr;  // PINNED_SLOT bytes of pinned host memory
     bamg_opts o{};
     cudaStream_t s = nullptr;
     double setup_ms = 0.0;
-    virtual ~SolverBase() {}
+    virtual ~SolverBase() {
+        if (h_pin) pinned_release(h_pin);
+    }
     virtual int nlevels() const = 0;
     virtual void level_size(int l, int64_t* n, int64_t* nnz) const = 0;
     virtual void solve(double* x, int flags, double tol, bamg_stats* st) = 0;
@@ -226,11 +366,10 @@ struct Solver : SolverBase {
     DevBuf<double> V, state, partial, x0, xw, rn;
     DevBuf<T> Z, vin, zout;
     DevBuf<int> dj;
-    double* h_pin = nullptr;
     // one Arnoldi step captured as a CUDA graph, replayed on the private stream
-    cudaStream_t& ps = priv.ps;
-    cudaEvent_t& ev_in = priv.ev_in;
-    cudaEvent_t& ev_out = priv.ev_out;
+    cudaStream_t& ps = priv.k.ps;
+    cudaEvent_t& ev_in = priv.k.ev_in;
+    cudaEvent_t& ev_out = priv.k.ev_out;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     int64_t graph_kernels = 0;  // kernels of one step
@@ -245,7 +384,6 @@ struct Solver : SolverBase {
         if (ps) cudaStreamSynchronize(ps);
         if (gexec) cudaGraphExecDestroy(gexec);
         if (graph) cudaGraphDestroy(graph);
-        if (h_pin) cudaFreeHost(h_pin);
         // the private stream itself is destroyed by SolverBase::priv after the buffers
     }
     int nlevels() const override { return (int)lv.size(); }
@@ -626,7 +764,7 @@ struct Solver : SolverBase {
     void setup(const bamg_csr* A, int r_, int levels, double mle_tol = 0.0, int max_cycles = 0, bool mle_l2 = false,
                int* h_cycles = nullptr, double* h_ratio = nullptr) {
         auto t0 = std::chrono::steady_clock::now();
-        AllocStream as_(s);
+        AllocStream as_(s, &darena);
         if (!arena || arena->s != s) arena = std::make_unique<StackArena>(s);
         ArenaScope ar_(*arena);
         PhaseTrace tr(s);
@@ -677,7 +815,7 @@ struct Solver : SolverBase {
     // longer in use); the captured Arnoldi step is dropped, its pointers being stale.
     void mle_restart(const double* x) {
         BAMG_CK(cudaStreamSynchronize(s));
-        AllocStream as_(s);
+        AllocStream as_(s, &darena);
         const int n = lv[0]->n;
         {
             TmpBuf<double> nrm(2, s), part((size_t)dots_partial_blocks(n) + 64, s);
@@ -703,7 +841,7 @@ struct Solver : SolverBase {
 
     // --------------------------------------------------------------- import
     void import(int nlev, const bamg_level_in* in, const double* h_pinv, const double* h_x_init) {
-        AllocStream as_(s);
+        AllocStream as_(s, &darena);
         lv.clear();
         for (int l = 0; l < nlev; ++l) {
             auto L = std::make_unique<LevelT<T>>();
@@ -778,11 +916,11 @@ struct Solver : SolverBase {
     // power iteration on the residual propagator I - B C (see bamg_vcycle_factor)
     double vcycle_factor(int iters) override {
         check_setup_flags(false);
-        AllocStream as_(s);
+        AllocStream as_(s, &darena);
         const int n = lv[0]->n;
         const MatView<double> B = B64();
         TmpBuf<double> x(n, s), r(n, s), z(n, s), t(n, s), mom(2, s);
-        if (!h_pin) BAMG_CK(cudaMallocHost(&h_pin, 32 * sizeof(double)));
+        if (!h_pin) h_pin = static_cast<double*>(pinned_acquire());
         BAMG_LAUNCH(k_vf_start, blocks_for(n, 256), 256, 0, s, n, x.get());
         spmv_f64(B, x.get(), r.get(), 1.0, s);
         auto normalise = [&]() {  // r <- (r - mean) / ||r - mean||; returns the norm
@@ -814,18 +952,18 @@ struct Solver : SolverBase {
 
     void vcycle_apply(const double* v, double* z) override {
         check_setup_flags(false);
-        AllocStream as_(s);
+        AllocStream as_(s, &darena);
         const int n = lv[0]->n;
         if constexpr (std::is_same<T, double>::value) {
             auto vl = vlevels(v, z);
             vcycle<T>(vl, pinvT.get(), o.omega, o.nu_pre, o.nu_post, s);
         } else {
             vin.ensure(n);
-            TmpBuf<float> zo(n, s);
+            zout.ensure(n);
             launch_convert<double, float>(n, v, vin.get(), s);
-            auto vl = vlevels(vin.get(), zo.get());
+            auto vl = vlevels(vin.get(), zout.get());
             vcycle<T>(vl, pinvT.get(), o.omega, o.nu_pre, o.nu_post, s);
-            launch_convert<float, double>(n, zo.get(), z, s);
+            launch_convert<float, double>(n, zout.get(), z, s);
         }
     }
 
@@ -936,11 +1074,10 @@ struct Solver : SolverBase {
     }
 
     void ensure_private_stream() {
-        if (!h_pin) BAMG_CK(cudaMallocHost(&h_pin, 32 * sizeof(double)));
+        if (!h_pin) h_pin = static_cast<double*>(pinned_acquire());
         if (!ps) {
-            BAMG_CK(cudaStreamCreateWithFlags(&ps, cudaStreamNonBlocking));
-            BAMG_CK(cudaEventCreateWithFlags(&ev_in, cudaEventDisableTiming));
-            BAMG_CK(cudaEventCreateWithFlags(&ev_out, cudaEventDisableTiming));
+            priv.dev = current_device();
+            priv.k = acquire_streams(priv.dev);
         }
     }
     // runs f with s = the private stream, fenced against the caller's stream on both sides
@@ -965,7 +1102,7 @@ struct Solver : SolverBase {
     }
 
     void solve(double* x_user, int flags, double tol, bamg_stats* st) override {
-        AllocStream as_(s);
+        AllocStream as_(s, &darena);
         const int n = lv[0]->n;
         m = std::min(std::max(o.gmres_m, 1), GMRES_MMAX);
         GmresLayout GL(m);
@@ -989,7 +1126,7 @@ struct Solver : SolverBase {
     DevBuf<double> Hh, eta, zero;
     void parnoldi(double* x_user, int flags, double tol, bamg_stats* st) override {
         check_setup_flags(false);
-        AllocStream as_(s);
+        AllocStream as_(s, &darena);
         const int n = lv[0]->n;
         const int mp = std::min(std::max(o.gmres_m, 1), PARN_MMAX);
         GmresLayout GL(mp);
@@ -1622,6 +1759,10 @@ int bamg_solve_batch(int nchains, const bamg_csr* As, const int* r, const int* l
     for (auto& t : pool) t.join();
     g_err = first_msg;
     return first_code;
+}
+
+int bamg_release_memory(void) {
+    return guarded([&] { pool_trim(); });
 }
 
 const char* bamg_last_error(void) { return g_err.c_str(); }

@@ -180,3 +180,41 @@ def test_interpolation_rows_equal_the_recording_path(kind, n, ncols, ld, offset,
         order = np.argsort(cols)
         assert np.array_equal(cols[order], pcol[i, :pcnt[i]])
         assert np.array_equal(tgt[i, slots][order], pval[i, :pcnt[i]].astype(np.float32))
+
+
+def test_kept_memory_is_bounded_and_given_back():
+    """Handles made, used and freed on several threads and streams keep at most the pool's 512 MiB and
+    their streams; release_memory gives it back.  (The first handle loads kernels and pages.)"""
+    import threading
+
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+
+    A = _walk(160, 150)
+    results = {}
+
+    def work(k):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(3):
+                s = bamg.Solver(*A, r=8, levels=20, grid=(160, 150), precision="mixed")
+                x, _ = s.solve(1e-10)
+                s.close()
+            torch.cuda.current_stream().synchronize()
+            results[k] = x
+
+    work(-1)
+    bamg.release_memory()
+    torch.cuda.empty_cache()
+    free0 = torch.cuda.mem_get_info()[0]
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    assert free0 - torch.cuda.mem_get_info()[0] <= (640 << 20)
+    assert all(torch.equal(results[k], results[-1]) for k in range(4))
+    bamg.release_memory()
+    assert free0 - torch.cuda.mem_get_info()[0] <= (64 << 20)
