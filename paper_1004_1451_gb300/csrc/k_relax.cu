@@ -372,8 +372,6 @@ void relax(const MatView<T>& B, const T* T_val, const T* dB, const T* dinvB, con
     const int nvec = (ncols + W - 1) / W;
     if (B.n == 0 || nvec == 0 || nu <= 0) return;
     const int64_t work_items = (int64_t)B.n * nvec;
-    const unsigned grid = (unsigned)std::min<int64_t>(blocks_for(work_items, 256),
-                                                      (int64_t)sm_count() * JAC_BLOCKS_PER_SM);
     const bool short_rows = (int64_t)B.nnz <= 5 * (int64_t)B.n;
     // small levels: one chunk per thread, two blocks per SM (the shorter per-thread work is
     // faster there); large levels: the fixed rule or the tuned shape
@@ -425,7 +423,7 @@ void relax(const MatView<T>& B, const T* T_val, const T* dB, const T* dinvB, con
         src = dst;
         dst = t;
     }
-    if (src != X) BAMG_LAUNCH(k_copy_cols<T>, grid, 256, 0, s, B.n, src, X, ld, col0, nvec);
+    if (src != X) BAMG_LAUNCH(k_copy_cols<T>, blocks_for(work_items, 256), 256, 0, s, B.n, src, X, ld, col0, nvec);
 }
 
 // ---------------------------------------------------------------- column statistics

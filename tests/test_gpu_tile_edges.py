@@ -218,3 +218,33 @@ def test_kept_memory_is_bounded_and_given_back():
     assert all(torch.equal(results[k], results[-1]) for k in range(4))
     bamg.release_memory()
     assert free0 - torch.cuda.mem_get_info()[0] <= (64 << 20)
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "fp64"])
+@pytest.mark.parametrize("nx,ny,ncols", [(150, 100, 10), (700, 301, 16)])
+def test_odd_sweep_counts_write_every_row(dtype, nx, ny, ncols):
+    """An odd number of sweeps ends in the work buffer and is copied back: three sweeps in one call and
+    one sweep three times (each copied back) and two and one give the same bits, on every row."""
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+
+    ptr, col, val = _walk(nx, ny)
+    td = torch.float64 if dtype == "fp64" else torch.float32
+    n = nx * ny
+    # B = I - A with the diagonal last in each row's order of columns put in its place
+    row = torch.repeat_interleave(torch.arange(n, device="cuda"), (ptr[1:] - ptr[:-1]).long())
+    rows = torch.cat([row, torch.arange(n, device="cuda")])
+    cols = torch.cat([col.long(), torch.arange(n, device="cuda")])
+    vals = torch.cat([-val, torch.ones(n, dtype=torch.float64, device="cuda")])
+    order = torch.argsort(rows * n + cols)
+    B = ((ptr + torch.arange(n + 1, device="cuda")).int(), cols[order].int(), vals[order].to(td))
+    X0 = torch.rand(n, ncols, dtype=td, device="cuda")
+    once, thrice, split = X0.clone(), X0.clone(), X0.clone()
+    bamg.relax(B, once, ncols, 0, 0.7, 3)
+    for _ in range(3):
+        bamg.relax(B, thrice, ncols, 0, 0.7, 1)
+    bamg.relax(B, split, ncols, 0, 0.7, 2)
+    assert torch.equal((split != X0).any(1), torch.ones(n, dtype=torch.bool, device="cuda"))
+    bamg.relax(B, split, ncols, 0, 0.7, 1)
+    assert torch.equal(once, split) and torch.equal(once, thrice)
