@@ -45,12 +45,13 @@ static void relax_step(const bamg_mat* Bm, const void* T_val, const double* lam,
     MatView<T> B = view<T>(Bm);
     check_block<T>(X, ncols, ld, col0);
     BAMG_REQUIRE(work && ((uintptr_t)work & 15) == 0, BAMG_EINVAL, "work must be 16-byte aligned");
-    TmpBuf<T> dB(B.n, s), dT(B.n, s), dinv(B.n, s);
-    launch_diag<T>(B, dB.get(), s);
-    launch_reciprocal<T>(B.n, dB.get(), dinv.get(), s);
-    if (T_val) launch_diag_vals<T>(B.n, B.rp, B.ci, (const T*)T_val, dT.get(), s);
-    relax<T>(B, (const T*)T_val, dB.get(), dinv.get(), T_val ? dT.get() : nullptr, lam, ncols, ld, col0, (T)omega, nu,
-             (T*)X, (T*)work, s);
+    const size_t stride = ((size_t)B.n + 63) & ~size_t(63);
+    TmpBuf<T> diags(3 * stride, s);
+    T *dB = diags.get(), *dinv = dB + stride, *dT = T_val ? dinv + stride : nullptr;
+    // FP32: the first sweep forms the diagonals; FP64: a pass of their own
+    const bool first = sizeof(T) == 4;
+    if (!first) launch_diagonals<T>(B.n, B.rp, B.ci, B.v, (const T*)T_val, dB, dT, dinv, s);
+    relax<T>(B, (const T*)T_val, dB, dinv, dT, lam, ncols, ld, col0, (T)omega, nu, (T*)X, (T*)work, s, true, first);
     BAMG_CK(cudaStreamSynchronize(s));
 }
 }  // namespace bamg

@@ -118,12 +118,18 @@ void launch_identity_on_pattern(int n, const int32_t* rp, const int32_t* ci, T* 
 // entries, gathers) overlap with earlier rows' work.  Entries beyond the first JB of a
 // row are read in predicated batches of JB; JB is 5 for matrices with at most five
 // entries per row on average (grid walks, tandem queues), else 6.
+//
+// DIAG: the diagonal arrays are not there yet.  The sweep finds the row's diagonal among the entries
+// it reads anyway, and stores it (1 / b_ii, or b_ii and t_ii for the shifted sweep) for the sweeps
+// after it.  A pass of its own over the matrix and one over the diagonal took 61 us of a four-sweep
+// call of 650 us on 2048 x 2048 states.  FP32 only: every thread of a row divides, which the FP64
+// pipe does not repeat for nothing.
 constexpr int JAC_BLOCKS_PER_SM = 2;
 
-template <typename T, bool SHIFT, int JB, int CPT>
+template <typename T, bool SHIFT, int JB, int CPT, bool DIAG>
 __global__ void __launch_bounds__(256, JAC_BLOCKS_PER_SM)
     k_jacobi(int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci, const T* __restrict__ bv,
-             const T* __restrict__ tv, const T* __restrict__ dB, const T* __restrict__ dinvB, const T* __restrict__ dT,
+             const T* __restrict__ tv, T* __restrict__ dB, T* __restrict__ dinvB, T* __restrict__ dT,
              const double* __restrict__ lam, int ncols, const T* __restrict__ X, T* __restrict__ Y, int ld, int col0,
              int nvec, T omega) {
     pdl_begin();
@@ -167,8 +173,8 @@ __global__ void __launch_bounds__(256, JAC_BLOCKS_PER_SM)
         T xs[CW];
 #pragma unroll
         for (int q = 0; q < CPT; ++q) V16<T>::load(X + row * ld + off + q * W, xs + q * W);
-        const T d0 = SHIFT ? __ldg(dB + row) : __ldg(dinvB + row);
-        const T d1 = has_t ? __ldg(dT + row) : T(1);
+        T d0 = DIAG ? T(0) : SHIFT ? __ldg(dB + row) : __ldg(dinvB + row);
+        T d1 = DIAG && has_t ? T(0) : has_t ? __ldg(dT + row) : T(1);
         // ... while the next row's first entries and the row pointers after it arrive
         const int ncnt = nrow < n ? min(JB, np1 - np0) : 0;
         int njj[JB];
@@ -194,6 +200,10 @@ __global__ void __launch_bounds__(256, JAC_BLOCKS_PER_SM)
                 const int j = __ldg(ci + p);
                 const T b = __ldg(bv + p);
                 const T tq = has_t ? __ldg(tv + p) : T(0);
+                if (DIAG && j == row) {
+                    d0 = b;
+                    if (has_t) d1 = tq;
+                }
 #pragma unroll
                 for (int q = 0; q < CPT; ++q) {
                     T xq[W];
@@ -225,6 +235,10 @@ __global__ void __launch_bounds__(256, JAC_BLOCKS_PER_SM)
 #pragma unroll
             for (int u = 0; u < JB; ++u)
                 if (u < c2) {
+                    if (DIAG && kj[u] == row) {
+                        d0 = kb[u];
+                        if (has_t) d1 = kt[u < NT ? u : 0];
+                    }
 #pragma unroll
                     for (int e = 0; e < CW; ++e) acc[e] += kb[u] * kx[u][e];
                     if (has_t)
@@ -235,12 +249,23 @@ __global__ void __launch_bounds__(256, JAC_BLOCKS_PER_SM)
 #pragma unroll
         for (int u = 0; u < JB; ++u)
             if (u < cnt) {
+                if (DIAG && jj[u] == row) {
+                    d0 = bb[u];
+                    if (has_t) d1 = tt[u < NT ? u : 0];
+                }
 #pragma unroll
                 for (int e = 0; e < CW; ++e) acc[e] += bb[u] * xv[u][e];
                 if (has_t)
 #pragma unroll
                     for (int e = 0; e < CW; ++e) accT[e] += tt[u < NT ? u : 0] * xv[u][e];
             }
+        if (DIAG) {
+            if (!SHIFT) d0 = T(1) / d0;
+            if (ch == 0) {
+                (SHIFT ? dB : dinvB)[row] = d0;
+                if (has_t) dT[row] = d1;
+            }
+        }
         T y[CW];
         if (SHIFT) {
 #pragma unroll
@@ -302,14 +327,24 @@ __global__ void k_copy_cols(int n, const T* __restrict__ src, T* __restrict__ ds
 
 // One sweep of the launch shape (chunks per thread, blocks per SM of the grid): Y from X.
 template <typename T>
-static void jacobi_sweep(const MatView<T>& B, const T* T_val, const T* dB, const T* dinvB, const T* dT,
-                         const double* d_lambda, int ncols, int ld, int col0, T omega, int nvec, bool short_rows,
-                         int cpt, int bps, const T* X, T* Y, cudaStream_t s) {
+static void jacobi_sweep(const MatView<T>& B, const T* T_val, T* dB, T* dinvB, T* dT, const double* d_lambda, int ncols,
+                         int ld, int col0, T omega, int nvec, bool short_rows, int cpt, int bps, bool diag, const T* X,
+                         T* Y, cudaStream_t s) {
     const unsigned grid = (unsigned)std::min<int64_t>(blocks_for((int64_t)B.n * (nvec / cpt), 256),
                                                       (int64_t)sm_count() * bps);
-#define BAMG_JAC(SH, JBV, CP)                                                                                     \
-    BAMG_LAUNCH((k_jacobi<T, SH, JBV, CP>), grid, 256, 0, s, B.n, B.rp, B.ci, B.v, T_val, dB, dinvB, dT, d_lambda, \
-                ncols, X, Y, ld, col0, nvec, omega)
+    auto go = [&](auto kern) {
+        BAMG_LAUNCH(kern, grid, 256, 0, s, B.n, B.rp, B.ci, B.v, T_val, dB, dinvB, dT, d_lambda, ncols, X, Y, ld, col0, nvec,
+                    omega);
+    };
+#define BAMG_JAC(SH, JBV, CP)                          \
+    do {                                              \
+        if constexpr (sizeof(T) == 4)                 \
+            if (diag) {                               \
+                go(k_jacobi<T, SH, JBV, CP, true>);   \
+                break;                                \
+            }                                         \
+        go(k_jacobi<T, SH, JBV, CP, false>);          \
+    } while (0)
     const int variant = (d_lambda ? 4 : 0) + (cpt == 2 ? 2 : 0) + (short_rows ? 0 : 1);
     switch (variant) {
         case 0: BAMG_JAC(false, 5, 1); break;
@@ -366,8 +401,8 @@ int jacobi_tuned_shapes(int* out, int max_rows) {
 }
 
 template <typename T>
-void relax(const MatView<T>& B, const T* T_val, const T* dB, const T* dinvB, const T* dT, const double* d_lambda,
-           int ncols, int ld, int col0, T omega, int nu, T* X, T* work, cudaStream_t s, bool tune) {
+void relax(const MatView<T>& B, const T* T_val, T* dB, T* dinvB, T* dT, const double* d_lambda, int ncols, int ld,
+           int col0, T omega, int nu, T* X, T* work, cudaStream_t s, bool tune, bool diag) {
     constexpr int W = V16<T>::W;
     const int nvec = (ncols + W - 1) / W;
     if (B.n == 0 || nvec == 0 || nu <= 0) return;
@@ -395,11 +430,11 @@ void relax(const MatView<T>& B, const T* T_val, const T* dB, const T* dinvB, con
             float best = 0.f;
             for (const JacShape& c : cand) {
                 jacobi_sweep<T>(B, T_val, dB, dinvB, dT, d_lambda, ncols, ld, col0, omega, nvec, short_rows, c.cpt,
-                                c.bps, X, work, s);  // warm-up
+                                c.bps, diag, X, work, s);  // warm-up
                 BAMG_CK(cudaEventRecord(e0, s));
                 for (int r = 0; r < 3; ++r)
                     jacobi_sweep<T>(B, T_val, dB, dinvB, dT, d_lambda, ncols, ld, col0, omega, nvec, short_rows, c.cpt,
-                                    c.bps, X, work, s);
+                                    c.bps, false, X, work, s);
                 BAMG_CK(cudaEventRecord(e1, s));
                 BAMG_CK(cudaEventSynchronize(e1));
                 float ms = 0.f;
@@ -418,7 +453,7 @@ void relax(const MatView<T>& B, const T* T_val, const T* dB, const T* dinvB, con
     T* dst = work;
     for (int k = 0; k < nu; ++k) {
         jacobi_sweep<T>(B, T_val, dB, dinvB, dT, d_lambda, ncols, ld, col0, omega, nvec, short_rows, shape.cpt,
-                        shape.bps, src, dst, s);
+                        shape.bps, diag && k == 0, src, dst, s);
         T* t = src;
         src = dst;
         dst = t;
@@ -812,8 +847,8 @@ int build_system_matrix(int n, int nnzA, const int32_t* rpA, const int32_t* ciA,
     template void launch_diagonals<T>(int, const int32_t*, const int32_t*, const T*, const T*, T*, T*, T*,         \
                                       cudaStream_t);                                                                \
     template void launch_identity_on_pattern<T>(int, const int32_t*, const int32_t*, T*, cudaStream_t);            \
-    template void relax<T>(const MatView<T>&, const T*, const T*, const T*, const T*, const double*, int, int, int, \
-                           T, int, T*, T*, cudaStream_t, bool);                                                    \
+    template void relax<T>(const MatView<T>&, const T*, T*, T*, T*, const double*, int, int, int, T, int, T*, T*,  \
+                           cudaStream_t, bool, bool);                                                    \
     template void tv_weights<T>(const MatView<T>&, int, int, int, const uint8_t*, double, T*, double*, cudaStream_t); \
     template void rayleigh_update<T>(const MatView<T>&, const T*, const T*, int, int, int, double, double*,         \
                                      uint8_t*, cudaStream_t);                                                      \

@@ -47,8 +47,9 @@ void launch_identity_on_pattern(int n, const int32_t* rp, const int32_t* ci, T* 
 // nu sweeps; T_val/dT/d_lambda may be null (no shift).  work: n*ld scratch.  tune: on large
 // levels, time the launch shapes once per shape key (jacobi_tuned_shapes lists the choices).
 template <typename T>
-void relax(const MatView<T>& B, const T* T_val, const T* dB, const T* dinvB, const T* dT, const double* d_lambda,
-           int ncols, int ld, int col0, T omega, int nu, T* X, T* work, cudaStream_t s, bool tune = true);
+void relax(const MatView<T>& B, const T* T_val, T* dB, T* dinvB, T* dT, const double* d_lambda, int ncols, int ld,
+           int col0, T omega, int nu, T* X, T* work, cudaStream_t s, bool tune = true, bool diag = false);
+// (diag, FP32 only: dB, dinvB and dT are formed by the first sweep)
 // Rows (precision bytes, shift, entry batch, 16-byte chunks per row, log2 n, chunks per
 // thread, blocks per SM) of the tuned sweep shapes, at most max_rows; returns the count.
 int jacobi_tuned_shapes(int* out, int max_rows);

@@ -221,7 +221,7 @@ def test_kept_memory_is_bounded_and_given_back():
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "fp64"])
-@pytest.mark.parametrize("nx,ny,ncols", [(150, 100, 10), (700, 301, 16)])
+@pytest.mark.parametrize("nx,ny,ncols", [(150, 100, 12), (700, 301, 16)])
 def test_odd_sweep_counts_write_every_row(dtype, nx, ny, ncols):
     """An odd number of sweeps ends in the work buffer and is copied back: three sweeps in one call and
     one sweep three times (each copied back) and two and one give the same bits, on every row."""
@@ -248,3 +248,56 @@ def test_odd_sweep_counts_write_every_row(dtype, nx, ny, ncols):
     assert torch.equal((split != X0).any(1), torch.ones(n, dtype=torch.bool, device="cuda"))
     bamg.relax(B, split, ncols, 0, 0.7, 1)
     assert torch.equal(once, split) and torch.equal(once, thrice)
+
+
+@pytest.mark.parametrize("shift", [False, True])
+@pytest.mark.parametrize("rows_entries,n,ncols,nu", [(3, 1, 4, 1), (5, 1000, 10, 2), (5, 400001, 16, 3), (14, 3001, 7, 2),
+                                                     (14, 300000, 8, 1)])
+def test_first_sweep_forms_the_diagonals(shift, rows_entries, n, ncols, nu):
+    """FP32 sweeps whose first one reads the diagonals off the rows, against sweeps one call at a time
+    with the diagonals at hand (relax_noalloc where it fits, else single-sweep calls): same bits, the
+    diagonal among the first entries of a row or beyond them, small levels and tuned ones."""
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+
+    g = torch.Generator(device="cuda").manual_seed(n)
+    m = min(rows_entries, n)
+    i = torch.arange(n, device="cuda")
+    off = torch.arange(m, device="cuda") - (m - 1 if rows_entries == 14 else m // 2)  # the last entry, or the middle
+    col = (i[:, None] + off[None, :]).clamp(0, n - 1)
+    col = torch.where(col == torch.cat([col[:, 1:], col[:, -1:] + n], 1), torch.full_like(col, -1), col)  # unique
+    ok = col >= 0
+    ptr = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    ptr[1:] = ok.sum(1).cumsum(0)
+    val = torch.where(col == i[:, None], 1.0 + torch.rand(n, m, generator=g, device="cuda"),
+                      -0.1 * torch.rand(n, m, generator=g, device="cuda"))[ok]
+    B = (ptr.int(), col[ok].int(), val.contiguous())
+    T = (0.5 + 0.1 * torch.rand(val.numel(), generator=g, device="cuda")) if shift else None
+    lam = (0.01 * torch.rand(ncols, generator=g, device="cuda")).double() if shift else None
+    ld = (ncols + 3) // 4 * 4
+    X = torch.rand(n, ld, generator=g, device="cuda")
+    Y = X.clone()
+    bamg.relax(B, X, ncols, 0, 0.7, nu, T_val=T, lam=lam)
+    if n * (ld + 3) * 4 <= (8 << 20) - 4096:
+        bamg.relax_noalloc(B, Y, ncols, 0, 0.7, nu, T_val=T, lam=lam)
+    else:
+        d = torch.zeros(n, device="cuda")
+        row = torch.repeat_interleave(i, ok.sum(1))
+        at = B[1].long() == row
+        d[row[at]] = val[at]
+        for _ in range(nu):
+            bamg.relax(B, Y, ncols, 0, 0.7, 1, T_val=T, lam=lam)
+        Z = torch.rand(n, ld, generator=g, device="cuda")
+        R = Z.double()
+        v = val.double() if not shift else None
+        bamg.relax(B, Z, ncols, 0, 0.7, 1, T_val=T, lam=lam)
+        for c in range(ncols):  # one sweep in FP64: 14 products and a quotient in FP32, 2^-24 each
+            l = lam[c] if shift else 0.0
+            w = val.double() - l * T.double() if shift else v
+            s = torch.segment_reduce(w * R[:, c][B[1].long()], "sum", lengths=ok.sum(1))
+            dd = torch.zeros(n, dtype=torch.float64, device="cuda")
+            dd[row[at]] = w[at]
+            ref = R[:, c] - 0.7 * s / dd
+            assert float((Z[:, c].double() - ref).abs().max()) <= 40 * 2.0 ** -24 * 4.0
+    assert torch.equal(X, Y)
