@@ -399,5 +399,20 @@ __device__ __forceinline__ double div_by_recip(double w, double h, double r) {
 void exclusive_scan(const int32_t* d_in, int32_t* d_out, int n, cudaStream_t s, int32_t* h_total = nullptr);
 int32_t exclusive_scan_total(const int32_t* d_in, int32_t* d_out, int n, cudaStream_t s);  // the total, to the host
 int32_t read_int(const int32_t* d_p, cudaStream_t s);  // a device int, to the host (after s's earlier work)
+// Up to 16 doubles a kernel posts to this thread's mapped host block: host_post_begin before the
+// launch, host_post by one thread of the kernel, host_post_wait after it.  The same block carries
+// read_int's and the scans' counts: one at a time.
+struct HostPost {
+    int32_t* flag = nullptr;
+    double* val = nullptr;
+};
+HostPost host_post_begin();
+void host_post_wait(double* out, int k, cudaStream_t s);
+__device__ __forceinline__ void host_post(const HostPost& p, const double* v, int k) {
+    for (int q = 0; q < k; ++q) *(volatile double*)(p.val + q) = v[q];
+    __threadfence_system();
+    *(volatile int32_t*)p.flag = 1;
+    __threadfence_system();
+}
 
 }  // namespace bamg

@@ -4,6 +4,8 @@
 // independent set of the slow points joins C.  Independent sets use Luby's rule with
 // fixed SplitMix64 priorities: an undecided candidate enters when its key (priority,
 // index) beats every undecided neighbour's, after which its undecided neighbours leave.
+#include <algorithm>
+
 #include "kernels.cuh"
 
 namespace bamg {
@@ -85,34 +87,44 @@ __global__ void k_mis_remove(int n, const int32_t* __restrict__ rp, const int32_
 // after every round.
 constexpr int MIS_CHECK = 4;
 static void independent_set(int n, const int32_t* rp, const int32_t* ci, const int32_t* rpT, const int32_t* ciT,
-                            uint8_t* und, uint8_t* chosen, uint64_t seed, uint64_t stream, cudaStream_t s) {
-    TmpBuf<uint8_t> win(n, s);
-    TmpBuf<int> left(1, s);
+                            uint8_t* und, uint8_t* chosen, uint8_t* win, int* left, uint64_t seed, uint64_t stream,
+                            cudaStream_t s) {
     const unsigned g = blocks_for(n, 256);
     for (int round = 0; round <= n; round += MIS_CHECK) {
         for (int k = 0; k < MIS_CHECK; ++k) {
-            BAMG_LAUNCH(k_mis_step, g, 256, 0, s, n, rp, ci, rpT, ciT, und, win.get(), seed, stream, left.get());
-            BAMG_LAUNCH(k_mis_remove, g, 256, 0, s, n, rp, ci, rpT, ciT, und, win.get(), chosen, left.get());
+            BAMG_LAUNCH(k_mis_step, g, 256, 0, s, n, rp, ci, rpT, ciT, und, win, seed, stream, left);
+            BAMG_LAUNCH(k_mis_remove, g, 256, 0, s, n, rp, ci, rpT, ciT, und, win, chosen, left);
         }
-        int h = 0;
-        BAMG_CK(cudaMemcpyAsync(&h, left.get(), sizeof(int), cudaMemcpyDeviceToHost, s));
-        BAMG_CK(cudaStreamSynchronize(s));
-        if (h == 0) return;
+        if (read_int(left, s) == 0) return;
     }
     throw Error(BAMG_ETIMEOUT, "independent set did not terminate");
 }
 
+// u = 0 on C, the round's random start on F; in the first round (w given) also w_i = omega / b_ii
+template <typename T>
 __global__ void k_cr_start(int n, const uint8_t* __restrict__ cf, double* __restrict__ u, uint64_t seed,
-                           uint64_t stream) {
+                           uint64_t stream, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                           const T* __restrict__ bv, double omega, double* __restrict__ w) {
     pdl_begin();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) u[i] = cf[i] ? 0.0 : 1.0 + counter_uniform(seed, stream, (uint64_t)i);
+    if (i >= n) return;
+    u[i] = cf[i] ? 0.0 : 1.0 + counter_uniform(seed, stream, (uint64_t)i);
+    if (w) {
+        double d = 0.0;
+        for (int p = rp[i]; p < rp[i + 1]; ++p)
+            if (ci[p] == i) d = (double)bv[p];
+        w[i] = omega * (1.0 / d);
+    }
 }
 
+// One F-relaxation sweep.  u is 0 on C, so every entry of the row takes part: the C entries add
+// zeros, which leaves the sum exactly as it is and spares a load per entry between the index and u.
+// The quotient omega / b_ii comes from k_cr_start: an FP64 division a row and sweep took a third of
+// the sweep's time on the FP64 pipe (32 us a sweep of 2^18 rows).
 template <typename T>
 __global__ void k_frelax(int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                         const T* __restrict__ bv, const uint8_t* __restrict__ cf, const double* __restrict__ u,
-                         double* __restrict__ un, double omega) {
+                         const T* __restrict__ bv, const uint8_t* __restrict__ cf, const double* __restrict__ w,
+                         const double* __restrict__ u, double* __restrict__ un) {
     pdl_begin();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -120,44 +132,50 @@ __global__ void k_frelax(int n, const int32_t* __restrict__ rp, const int32_t* _
         un[i] = 0.0;
         return;
     }
-    double s = 0.0, d = 0.0;
-    for (int p = rp[i]; p < rp[i + 1]; ++p) {
-        const int j = ci[p];
-        if (j == i) d = (double)bv[p];
-        if (!cf[j]) s += (double)bv[p] * u[j];
+    double s = 0.0;
+    int p = rp[i];
+    const int pe = rp[i + 1];
+    for (; p + 4 <= pe; p += 4) {  // loads before their uses
+        const int j0 = ci[p], j1 = ci[p + 1], j2 = ci[p + 2], j3 = ci[p + 3];
+        const T b0 = bv[p], b1 = bv[p + 1], b2 = bv[p + 2], b3 = bv[p + 3];
+        const double u0 = u[j0], u1 = u[j1], u2 = u[j2], u3 = u[j3];
+        s += (double)b0 * u0;
+        s += (double)b1 * u1;
+        s += (double)b2 * u2;
+        s += (double)b3 * u3;
     }
-    un[i] = u[i] - (omega * (1.0 / d)) * s;
+    for (; p < pe; ++p) s += (double)bv[p] * u[ci[p]];
+    un[i] = u[i] - w[i] * s;
 }
 
 // k_frelax with G lanes per row (long rows of coarse levels): strided partial sums added
-// by a butterfly; the lane holding the diagonal contributes d, the others 0.
+// by a butterfly.
 template <typename T, int G>
 __global__ void k_frelax_grp(int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                             const T* __restrict__ bv, const uint8_t* __restrict__ cf, const double* __restrict__ u,
-                             double* __restrict__ un, double omega) {
+                             const T* __restrict__ bv, const uint8_t* __restrict__ cf, const double* __restrict__ w,
+                             const double* __restrict__ u, double* __restrict__ un) {
     pdl_begin();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int i = (int)(t / G), sub = (int)(t % G);
-    double s = 0.0, d = 0.0;
+    double s = 0.0;
     const bool live = i < n && !cf[i];
-    if (live)
-        for (int p = rp[i] + sub; p < rp[i + 1]; p += G) {
-            const int j = ci[p];
-            if (j == i) d = (double)bv[p];
-            if (!cf[j]) s += (double)bv[p] * u[j];
-        }
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, o);
-        d += __shfl_xor_sync(0xffffffffu, d, o);
+    if (live) {
+        const int pe = rp[i + 1];
+#pragma unroll 4
+        for (int p = rp[i] + sub; p < pe; p += G) s += (double)bv[p] * u[ci[p]];
     }
-    if (i < n && sub == 0) un[i] = live ? u[i] - (omega * (1.0 / d)) * s : 0.0;
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (i < n && sub == 0) un[i] = live ? u[i] - w[i] * s : 0.0;
 }
 
-__global__ void k_cr_norms(int n, const double* __restrict__ u0, const double* __restrict__ u,
-                           double* __restrict__ partial) {
+// sum u0^2 and sum u^2: per-block partials, added up by the block that finishes last (a fixed order)
+// and posted to the host.  One thread adding them one by one took 17 us for 256 blocks.
+__global__ void __launch_bounds__(256) k_cr_norms(int n, const double* __restrict__ u0, const double* __restrict__ u,
+                                                  double* partial, unsigned* __restrict__ ticket, HostPost post) {
     pdl_begin();
     __shared__ double sh[2][8];
+    __shared__ int s_last;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     double a = 0.0, b = 0.0;
     if (i < n) {
@@ -176,15 +194,35 @@ __global__ void k_cr_norms(int n, const double* __restrict__ u0, const double* _
         double t = 0.0;
         for (int w = 0; w < 8; ++w) t += sh[threadIdx.x][w];
         partial[(int64_t)blockIdx.x * 2 + threadIdx.x] = t;
+        __threadfence();
     }
-}
-__global__ void k_sum2(int nb, const double* __restrict__ partial, double* __restrict__ out) {
-    pdl_begin();
-    const int q = threadIdx.x;
-    if (q >= 2) return;
-    double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += partial[(int64_t)b * 2 + q];
-    out[q] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    a = b = 0.0;
+    for (unsigned k = threadIdx.x; k < gridDim.x; k += blockDim.x) {
+        a += __ldcg(partial + 2 * k);
+        b += __ldcg(partial + 2 * k + 1);
+    }
+    a = warp_sum(a);
+    b = warp_sum(b);
+    if (lane == 0) {
+        sh[0][wid] = a;
+        sh[1][wid] = b;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        a = b = 0.0;
+        for (int w = 0; w < 8; ++w) {
+            a += sh[0][w];
+            b += sh[1][w];
+        }
+        *ticket = 0u;
+        const double v[2] = {a, b};
+        host_post(post, v, 2);
+    }
 }
 
 __global__ void k_cr_slow(int n, const uint8_t* __restrict__ cf, const double* __restrict__ up,
@@ -213,58 +251,71 @@ int coarsen_cr(const MatView<T>& B, int level, uint64_t seed, double theta, int 
     const int n = B.n;
     const unsigned g = blocks_for(n, 256);
     const int G = lanes_per_row(n, B.nnz);
-    // transpose pattern for the undirected neighbourhoods
-    TmpBuf<int32_t> cnt(n, s), rpT(n + 1, s), cursor(n, s);
-    BAMG_CK(cudaMemsetAsync(cnt.get(), 0, sizeof(int32_t) * n, s));
-    BAMG_CK(cudaMemsetAsync(cursor.get(), 0, sizeof(int32_t) * n, s));
-    BAMG_LAUNCH(k_tcount, g, 256, 0, s, n, B.rp, B.ci, cnt.get());
-    exclusive_scan(cnt.get(), rpT.get(), n, s);
-    TmpBuf<int32_t> ciT(B.nnz > 0 ? B.nnz : 1, s);  // bound: the off-diagonal entries of B
-    BAMG_LAUNCH(k_tfill, g, 256, 0, s, n, B.rp, B.ci, rpT.get(), cursor.get(), ciT.get());
-    TmpBuf<uint8_t> und(n, s), cand(n, s);
+    // one allocation: the transposed pattern (cnt and cursor adjacent; cnt is the scan's input and the
+    // final numbering's), vectors, masks
+    size_t used = 0;
+    auto slice = [&](size_t bytes) {
+        const size_t at = used;
+        used += (bytes + 255) & ~size_t(255);
+        return at;
+    };
+    const size_t ni = sizeof(int32_t) * (size_t)n, nd = sizeof(double) * (size_t)n;
+    const size_t o_cnt = slice(2 * ni + 256), o_rpT = slice(ni + sizeof(int32_t)),
+                 o_ciT = slice(sizeof(int32_t) * (size_t)std::max(B.nnz, 1)),  // bound: the off-diagonal entries of B
+                 o_w = slice(nd), o_u0 = slice(nd), o_ua = slice(nd), o_ub = slice(nd),
+                 o_part = slice(2 * sizeof(double) * g), o_und = slice(n), o_cand = slice(n), o_win = slice(n);
+    TmpBuf<char> work(used, s);
+    char* m = work.get();
+    int32_t *cnt = (int32_t*)(m + o_cnt), *cursor = cnt + n, *rpT = (int32_t*)(m + o_rpT), *ciT = (int32_t*)(m + o_ciT);
+    unsigned* ticket = (unsigned*)(cursor + n);
+    int* left = (int*)ticket + 1;
+    double *w = (double*)(m + o_w), *u0 = (double*)(m + o_u0), *part = (double*)(m + o_part);
+    uint8_t *und = (uint8_t*)(m + o_und), *cand = (uint8_t*)(m + o_cand), *win = (uint8_t*)(m + o_win);
+    BAMG_CK(cudaMemsetAsync(cnt, 0, 2 * ni + 2 * sizeof(int32_t), s));
+    BAMG_LAUNCH(k_tcount, g, 256, 0, s, n, B.rp, B.ci, cnt);
+    exclusive_scan(cnt, rpT, n, s);
+    BAMG_LAUNCH(k_tfill, g, 256, 0, s, n, B.rp, B.ci, (const int32_t*)rpT, cursor, ciT);
     BAMG_CK(cudaMemsetAsync(cf, 0, n, s));
-    BAMG_CK(cudaMemsetAsync(und.get(), 1, n, s));
-    independent_set(n, B.rp, B.ci, rpT.get(), ciT.get(), und.get(), cf, seed, STREAM_MIS + ((uint64_t)level << 8), s);
-    TmpBuf<double> u0(n, s), ua(n, s), ub(n, s), norms(2, s), part((size_t)g * 2, s);
+    BAMG_CK(cudaMemsetAsync(und, 1, n, s));
+    independent_set(n, B.rp, B.ci, rpT, ciT, und, cf, win, left, seed, STREAM_MIS + ((uint64_t)level << 8), s);
     int rounds = 0;
     double h[2];
     for (;;) {
-        BAMG_LAUNCH(k_cr_start, g, 256, 0, s, n, cf, u0.get(), seed, STREAM_CR + ((uint64_t)level << 8) + rounds);
-        const double* cur = u0.get();
+        BAMG_LAUNCH(k_cr_start<T>, g, 256, 0, s, n, (const uint8_t*)cf, u0, seed,
+                    STREAM_CR + ((uint64_t)level << 8) + rounds, B.rp, B.ci, B.v, omega, rounds == 0 ? w : (double*)nullptr);
+        const double* cur = u0;
         double* prev = nullptr;
-        double* bufs[2] = {ua.get(), ub.get()};
+        double* bufs[2] = {(double*)(m + o_ua), (double*)(m + o_ub)};
         for (int k = 0; k < nu; ++k) {
             double* nxt = bufs[k & 1];
+            auto sweep = [&](auto kern, unsigned grid) {
+                BAMG_LAUNCH(kern, grid, 256, 0, s, n, B.rp, B.ci, B.v, (const uint8_t*)cf, (const double*)w, cur, nxt);
+            };
             const unsigned gg = blocks_for((int64_t)n * G, 256);
             switch (G) {
-                case 1: BAMG_LAUNCH(k_frelax<T>, g, 256, 0, s, n, B.rp, B.ci, B.v, cf, cur, nxt, omega); break;
-                case 4: BAMG_LAUNCH((k_frelax_grp<T, 4>), gg, 256, 0, s, n, B.rp, B.ci, B.v, cf, cur, nxt, omega); break;
-                case 8: BAMG_LAUNCH((k_frelax_grp<T, 8>), gg, 256, 0, s, n, B.rp, B.ci, B.v, cf, cur, nxt, omega); break;
-                case 16:
-                    BAMG_LAUNCH((k_frelax_grp<T, 16>), gg, 256, 0, s, n, B.rp, B.ci, B.v, cf, cur, nxt, omega);
-                    break;
-                default:
-                    BAMG_LAUNCH((k_frelax_grp<T, 32>), gg, 256, 0, s, n, B.rp, B.ci, B.v, cf, cur, nxt, omega);
+                case 1: sweep(k_frelax<T>, g); break;
+                case 4: sweep(k_frelax_grp<T, 4>, gg); break;
+                case 8: sweep(k_frelax_grp<T, 8>, gg); break;
+                case 16: sweep(k_frelax_grp<T, 16>, gg); break;
+                default: sweep(k_frelax_grp<T, 32>, gg);
             }
             prev = const_cast<double*>(cur);
             cur = nxt;
         }
-        BAMG_LAUNCH(k_cr_norms, g, 256, 0, s, n, u0.get(), cur, part.get());
-        BAMG_LAUNCH(k_sum2, 1, 32, 0, s, (int)g, part.get(), norms.get());
-        BAMG_CK(cudaMemcpyAsync(h, norms.get(), sizeof(h), cudaMemcpyDeviceToHost, s));
-        BAMG_CK(cudaStreamSynchronize(s));
+        const HostPost post = host_post_begin();
+        BAMG_LAUNCH(k_cr_norms, g, 256, 0, s, n, (const double*)u0, cur, part, ticket, post);
+        host_post_wait(h, 2, s);
         const double rho = std::pow(std::sqrt(h[1]) / std::sqrt(h[0]), 1.0 / nu);
         if (!(rho > theta) || rounds >= max_rounds || h[0] == 0.0) break;
-        BAMG_LAUNCH(k_cr_slow, g, 256, 0, s, n, cf, prev, cur, theta, cand.get());
+        BAMG_LAUNCH(k_cr_slow, g, 256, 0, s, n, (const uint8_t*)cf, (const double*)prev, cur, theta, cand);
         ++rounds;
-        independent_set(n, B.rp, B.ci, rpT.get(), ciT.get(), cand.get(), cf, seed,
+        independent_set(n, B.rp, B.ci, rpT, ciT, cand, cf, win, left, seed,
                         STREAM_MIS + ((uint64_t)level << 8) + rounds, s);
     }
-    TmpBuf<int32_t> ci32(n, s), sc(n + 1, s);
-    BAMG_LAUNCH(k_u8_to_i32, g, 256, 0, s, n, cf, ci32.get());
-    exclusive_scan(ci32.get(), sc.get(), n, s);
-    BAMG_LAUNCH(k_cidx_from_scan, g, 256, 0, s, n, cf, sc.get(), cidx);
-    *nc_out = read_int(sc.get() + n, s);
+    BAMG_LAUNCH(k_u8_to_i32, g, 256, 0, s, n, (const uint8_t*)cf, cnt);
+    exclusive_scan(cnt, rpT, n, s);
+    BAMG_LAUNCH(k_cidx_from_scan, g, 256, 0, s, n, (const uint8_t*)cf, (const int32_t*)rpT, cidx);
+    *nc_out = read_int(rpT + n, s);
     return rounds;
 }
 
@@ -298,15 +349,15 @@ void colour_classes(int n, int nnz, const int32_t* rp, const int32_t* ci, int le
     exclusive_scan(cnt.get(), rpT.get(), n, s);
     TmpBuf<int32_t> ciT(nnz > 0 ? nnz : 1, s);
     BAMG_LAUNCH(k_tfill, g, 256, 0, s, n, rp, ci, rpT.get(), cursor.get(), ciT.get());
-    TmpBuf<uint8_t> left(n, s), und(n, s), chosen(n, s);
+    TmpBuf<uint8_t> left(n, s), und(n, s), chosen(n, s), win(n, s);
     TmpBuf<int32_t> colour(n, s);
-    TmpBuf<int> rem(1, s);
+    TmpBuf<int> rem(1, s), undecided(1, s);
     BAMG_CK(cudaMemsetAsync(left.get(), 1, n, s));
     int ncol = 0;
     for (int c = 0; c < MAX_COLOURS; ++c) {
         BAMG_CK(cudaMemcpyAsync(und.get(), left.get(), n, cudaMemcpyDeviceToDevice, s));
         BAMG_CK(cudaMemsetAsync(chosen.get(), 0, n, s));
-        independent_set(n, rp, ci, rpT.get(), ciT.get(), und.get(), chosen.get(), seed,
+        independent_set(n, rp, ci, rpT.get(), ciT.get(), und.get(), chosen.get(), win.get(), undecided.get(), seed,
                         STREAM_COLOUR + ((uint64_t)level << 8) + (uint64_t)c, s);
         BAMG_CK(cudaMemsetAsync(rem.get(), 0, sizeof(int), s));
         BAMG_LAUNCH(k_colour_take, g, 256, 0, s, n, (const uint8_t*)chosen.get(), c, colour.get(), left.get(),

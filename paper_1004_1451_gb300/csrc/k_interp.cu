@@ -244,6 +244,18 @@ static void exclusive_scan_total_begin(const int32_t* d_in, int32_t* d_out, int 
 }
 static int32_t scan_total_wait(cudaStream_t s) { return host_word_wait(host_word(), s); }
 
+HostPost host_post_begin() {
+    HostWord& hw = host_word();
+    *(volatile int32_t*)hw.h = HOST_WORD_EMPTY;
+    return HostPost{hw.d, reinterpret_cast<double*>(hw.d + 16)};
+}
+void host_post_wait(double* out, int k, cudaStream_t s) {
+    const HostWord& hw = host_word();
+    host_word_wait(hw, s);
+    std::atomic_thread_fence(std::memory_order_acquire);
+    for (int q = 0; q < k; ++q) out[q] = ((volatile double*)(hw.h + 16))[q];
+}
+
 int32_t read_int(const int32_t* d_p, cudaStream_t s) {
     HostWord& hw = host_word();
     *(volatile int32_t*)hw.h = HOST_WORD_EMPTY;
