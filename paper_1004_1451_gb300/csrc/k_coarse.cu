@@ -53,8 +53,21 @@ __device__ __forceinline__ unsigned pivot_key(float mag, int row) {
     return (bits & ~63u) | (unsigned)(63 - row);
 }
 
-// Real A (F = float or double); pivots below floorv in magnitude become +-floorv.
-template <typename F>
+// x - l p: rounded once, or (TWO) after the product and after the difference, as the complex
+// arithmetic does (x - (lr pr - li pi) with li = pi = 0)
+template <bool TWO>
+__device__ __forceinline__ float sub_mul(float x, float l, float p) {
+    return TWO ? __fadd_rn(x, -__fmul_rn(l, p)) : x - l * p;
+}
+template <bool TWO>
+__device__ __forceinline__ double sub_mul(double x, double l, double p) {
+    return TWO ? __dadd_rn(x, -__dmul_rn(l, p)) : x - l * p;
+}
+
+// Real A (F = float or double); pivots below floorv in magnitude become +-floorv.  With TWO the
+// factors are block_lu_factor_cplx's for a zero imaginary part, bit for bit (up to the sign of
+// zeros): two roundings, and a pivot below floorv becomes floorv.
+template <typename F, bool TWO = false>
 __device__ void block_lu_factor(F* A, int n, int* src, F* dinv, F floorv) {
     __shared__ int step_of[CN];  // pivot step of each row, -1 while unpivoted
     __shared__ F mult[CN];
@@ -75,7 +88,7 @@ __device__ void block_lu_factor(F* A, int n, int* src, F* dinv, F floorv) {
             if (lane == 0) {
                 const int pr = 63 - (int)(best & 63u);
                 F pv = A[pr * LDP + k];
-                if (absv(pv) < floorv) pv = pv >= F(0) ? floorv : -floorv;
+                if (absv(pv) < floorv) pv = TWO || pv >= F(0) ? floorv : -floorv;
                 A[pr * LDP + k] = pv;
                 src[k] = pr;
                 dinv[k] = F(1) / pv;
@@ -97,9 +110,9 @@ __device__ void block_lu_factor(F* A, int n, int* src, F* dinv, F floorv) {
                     x[j] = row[c + 4 * j];
                 }
 #pragma unroll
-                for (int j = 0; j < 4; ++j) row[c + 4 * j] = x[j] - l * pc[j];
+                for (int j = 0; j < 4; ++j) row[c + 4 * j] = sub_mul<TWO>(x[j], l, pc[j]);
             }
-            for (; c < n; c += 4) row[c] -= l * prow[c];
+            for (; c < n; c += 4) row[c] = sub_mul<TWO>(row[c], l, prow[c]);
         }
         __syncthreads();
     }
@@ -216,7 +229,7 @@ __device__ void block_lu_factor_cplx(F* Ar, F* Ai, int n, int* src, F* dr, F* di
 // row src[i] of A and of R): the independent columns hide the latency of the shuffles.
 // Forward and back substitution eliminate one column of L (of U) at a time, as in the
 // plain algorithm; lane l holds the unknowns l and l + 32.
-template <typename F, int NC>
+template <typename F, int NC, bool TWO = false>
 __device__ void warp_lu_solve_cols(const F* A, int n, const int* src, const F* dinv, F* R, int ldr, int c0, int m) {
     const int lane = lane_id();
     const int r0 = lane < n ? src[lane] : 0, r1 = lane + 32 < n ? src[lane + 32] : 0;
@@ -234,8 +247,8 @@ __device__ void warp_lu_solve_cols(const F* A, int n, const int* src, const F* d
 #pragma unroll
         for (int j = 0; j < NC; ++j) {
             const F y = __shfl_sync(0xffffffffu, q < 32 ? x0[j] : x1[j], q & 31);
-            if (a0) x0[j] = x0[j] - l0 * y;
-            if (a1) x1[j] = x1[j] - l1 * y;
+            if (a0) x0[j] = sub_mul<TWO>(x0[j], l0, y);
+            if (a1) x1[j] = sub_mul<TWO>(x1[j], l1, y);
         }
     }
     const F d0 = lane < n ? dinv[lane] : F(0), d1 = lane + 32 < n ? dinv[lane + 32] : F(0);
@@ -250,8 +263,8 @@ __device__ void warp_lu_solve_cols(const F* A, int n, const int* src, const F* d
 #pragma unroll
         for (int j = 0; j < NC; ++j) {
             const F y = __shfl_sync(0xffffffffu, q < 32 ? x0[j] : x1[j], q & 31);
-            if (a0) x0[j] = x0[j] - u0 * y;
-            if (a1) x1[j] = x1[j] - u1 * y;
+            if (a0) x0[j] = sub_mul<TWO>(x0[j], u0, y);
+            if (a1) x1[j] = sub_mul<TWO>(x1[j], u1, y);
         }
     }
     __syncwarp();
@@ -680,6 +693,10 @@ __global__ void __launch_bounds__(CT) k_coarse_eigvals(int n, const double* __re
 // then products with K); the Rayleigh-type quotient lambda = v^H B v / v^H T v (Algorithm
 // 3's update, in complex form, accumulated in F); and the phase that makes <w, v> real and
 // positive (w_i = i + 1) with unit 2-norm.
+// A real shift (every one of a reversible chain, grid walks among them) leaves all imaginary parts
+// zero: the factorisation and the iteration then run in real arithmetic, with the roundings of the
+// complex one, so the vectors are the same.  On the FP64 pipe that is 2 operations an element
+// instead of 6, one division a pivot instead of three.
 template <typename F>
 __device__ __forceinline__ F pivot_tiny() {
     if constexpr (sizeof(F) == 8)
@@ -739,7 +756,11 @@ __global__ void __launch_bounds__(CT) k_coarse_eigvec(int n, const double* __res
     // complex LU with partial pivoting on |Re| + |Im|, rows in place: row srcp[i] holds
     // pivot row i, dr + i di = 1 / u_ii
     __shared__ int srcp[CN];
-    block_lu_factor_cplx<F>(Ar, Ai, n, srcp, dr, di, pfloor);
+    const bool real = si == F(0);  // uniform per block
+    if (real)
+        block_lu_factor<F, true>(Ar, n, srcp, dr, pfloor);
+    else
+        block_lu_factor_cplx<F>(Ar, Ai, n, srcp, dr, di, pfloor);
     // start vector in [1, 2) drawn per column (SplitMix64, stream = the column): for a
     // multiple eigenvalue (the symmetric pairs of grid walks) each column converges to
     // the projection of its own start onto the eigenspace, so the columns span it
@@ -759,10 +780,25 @@ __global__ void __launch_bounds__(CT) k_coarse_eigvec(int n, const double* __res
         // steps as products v <- K v by the block (4 threads per row); the normalisation in FP32
         F* Kr = Tm + CN * LDP;
         F* Ki = Kr + CN * LDP;
-        warp_lu_solve_cols_cplx<F, CN / (CT / 32)>(Ar, Ai, n, srcp, dr, di, Tm, Kr, Ki, wid * (CN / (CT / 32)));
+        if (real) {
+            for (int idx = tid; idx < n * n; idx += CT) {
+                const int r = idx / n, c = idx - r * n;
+                Kr[r * LDP + c] = Tm[r * LDP + c];
+            }
+            __syncthreads();
+            warp_lu_solve_cols<F, CN / (CT / 32), true>(Ar, n, srcp, dr, Kr, LDP, wid * (CN / (CT / 32)), n);
+        } else {
+            warp_lu_solve_cols_cplx<F, CN / (CT / 32)>(Ar, Ai, n, srcp, dr, di, Tm, Kr, Ki, wid * (CN / (CT / 32)));
+        }
         __syncthreads();
         for (int it = 0; it < 4; ++it) {
-            if (row < n) {
+            if (row < n && real) {
+                F a = F(0);
+                const int c1 = min(n, 16 * quarter + 16);
+                for (int c = 16 * quarter; c < c1; ++c) a = add_rn(a, mul_rn(Kr[row * LDP + c], vr[c]));
+                pre[quarter * CN + row] = a;
+                pim[quarter * CN + row] = F(0);
+            } else if (row < n) {
                 F a = F(0), b = F(0);
                 const int c1 = min(n, 16 * quarter + 16);
                 for (int c = 16 * quarter; c < c1; ++c) {
@@ -805,7 +841,7 @@ __global__ void __launch_bounds__(CT) k_coarse_eigvec(int n, const double* __res
             for (int c = 16 * quarter; c < c1; ++c) {
                 const F t = Tm[row * LDP + c];
                 a += t * vr[c];
-                b += t * vi[c];
+                if (!real) b += t * vi[c];
             }
             pre[quarter * CN + row] = a;
             pim[quarter * CN + row] = b;
@@ -830,38 +866,59 @@ __global__ void __launch_bounds__(CT) k_coarse_eigvec(int n, const double* __res
                 xr[h] = r < n ? tr[srcp[r]] : F(0);
                 xi[h] = r < n ? ti[srcp[r]] : F(0);
             }
-            for (int q = 0; q + 1 < n; ++q) {  // unit lower
-                const F yr = __shfl_sync(0xffffffffu, q < 32 ? xr[0] : xr[1], q & 31);
-                const F yi = __shfl_sync(0xffffffffu, q < 32 ? xi[0] : xi[1], q & 31);
+            if (real) {
+                for (int q = 0; q + 1 < n; ++q) {  // unit lower
+                    const F y = __shfl_sync(0xffffffffu, q < 32 ? xr[0] : xr[1], q & 31);
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int r = lane + 32 * h;
-                    if (r > q && r < n) {
-                        const F lr = Ar[fr[h] * LDP + q], li = Ai[fr[h] * LDP + q];
-                        xr[h] -= lr * yr - li * yi;
-                        xi[h] -= lr * yi + li * yr;
+                    for (int h = 0; h < 2; ++h) {
+                        const int r = lane + 32 * h;
+                        if (r > q && r < n) xr[h] = sub_mul<true>(xr[h], Ar[fr[h] * LDP + q], y);
                     }
                 }
-            }
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int r = lane + 32 * h;
-                if (r < n) {
-                    const F a = xr[h], b = xi[h];
-                    xr[h] = a * dr[r] - b * di[r];
-                    xi[h] = a * di[r] + b * dr[r];
+                for (int h = 0; h < 2; ++h)
+                    if (lane + 32 * h < n) xr[h] = xr[h] * dr[lane + 32 * h];
+                for (int q = n - 1; q > 0; --q) {  // unit upper
+                    const F y = __shfl_sync(0xffffffffu, q < 32 ? xr[0] : xr[1], q & 31);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        if (lane + 32 * h < q) xr[h] = sub_mul<true>(xr[h], Ar[fr[h] * LDP + q], y);
                 }
-            }
-            for (int q = n - 1; q > 0; --q) {  // unit upper
-                const F yr = __shfl_sync(0xffffffffu, q < 32 ? xr[0] : xr[1], q & 31);
-                const F yi = __shfl_sync(0xffffffffu, q < 32 ? xi[0] : xi[1], q & 31);
+                xi[0] = xi[1] = F(0);
+            } else {
+                for (int q = 0; q + 1 < n; ++q) {  // unit lower
+                    const F yr = __shfl_sync(0xffffffffu, q < 32 ? xr[0] : xr[1], q & 31);
+                    const F yi = __shfl_sync(0xffffffffu, q < 32 ? xi[0] : xi[1], q & 31);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int r = lane + 32 * h;
+                        if (r > q && r < n) {
+                            const F lr = Ar[fr[h] * LDP + q], li = Ai[fr[h] * LDP + q];
+                            xr[h] -= lr * yr - li * yi;
+                            xi[h] -= lr * yi + li * yr;
+                        }
+                    }
+                }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int r = lane + 32 * h;
-                    if (r < q) {
-                        const F ur = Ar[fr[h] * LDP + q], ui = Ai[fr[h] * LDP + q];
-                        xr[h] -= ur * yr - ui * yi;
-                        xi[h] -= ur * yi + ui * yr;
+                    if (r < n) {
+                        const F a = xr[h], b = xi[h];
+                        xr[h] = a * dr[r] - b * di[r];
+                        xi[h] = a * di[r] + b * dr[r];
+                    }
+                }
+                for (int q = n - 1; q > 0; --q) {  // unit upper
+                    const F yr = __shfl_sync(0xffffffffu, q < 32 ? xr[0] : xr[1], q & 31);
+                    const F yi = __shfl_sync(0xffffffffu, q < 32 ? xi[0] : xi[1], q & 31);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int r = lane + 32 * h;
+                        if (r < q) {
+                            const F ur = Ar[fr[h] * LDP + q], ui = Ai[fr[h] * LDP + q];
+                            xr[h] -= ur * yr - ui * yi;
+                            xi[h] -= ur * yi + ui * yr;
+                        }
                     }
                 }
             }
