@@ -468,11 +468,12 @@ void relax(const MatView<T>& B, const T* T_val, T* dB, T* dinvB, T* dT, const do
 template <typename T, int MODE>
 __global__ void k_colstats(int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                            const T* __restrict__ bv, const T* __restrict__ tv, const T* __restrict__ X, int ld,
-                           int col0, int nvec, double* __restrict__ partial) {
+                           int col0, int nvec, double* __restrict__ partial, unsigned* __restrict__ ticket) {
     pdl_begin();
     constexpr int W = V16<T>::W;
     extern __shared__ double sh[];
     const int ch = threadIdx.x, ry = threadIdx.y, ny = blockDim.y;
+    if (blockIdx.x == 0 && ch == 0 && ry == 0) *ticket = 0u;  // for the kernel that adds up the partials
     const int off = col0 + ch * W;
     T s0[W], s1[W];
 #pragma unroll
@@ -526,6 +527,14 @@ __global__ void k_colstats(int n, const int32_t* __restrict__ rp, const int32_t*
 }
 
 
+// Workspace of one column-statistics pair of kernels: the partials, the sums and a ticket.
+struct ColWork {
+    double *partial, *sums;
+    unsigned* ticket;
+    static size_t doubles(int nb, int width) { return (size_t)nb * width + width + 1; }
+    ColWork(double* p, int nb, int width)
+        : partial(p), sums(p + (size_t)nb * width), ticket(reinterpret_cast<unsigned*>(p + (size_t)nb * width + width)) {}
+};
 // Column statistics of Eq. (3.4) / the Rayleigh quotients as per-block partial sums
 // (nb rows of `width` values in `partial`); the consumer forms the sums with
 // colsum_partials.  Returns nb.
@@ -545,7 +554,7 @@ static int colstats_blocks(int n, int ncols, int* width) {
     return nb;
 }
 template <typename T, int MODE>
-static void colstats(const MatView<T>& B, const T* T_val, const T* X, int ld, int col0, int ncols, double* partial,
+static void colstats(const MatView<T>& B, const T* T_val, const T* X, int ld, int col0, int ncols, const ColWork& cw,
                      cudaStream_t s) {
     constexpr int W = V16<T>::W;
     const int nvec = (ncols + W - 1) / W;
@@ -555,36 +564,50 @@ static void colstats(const MatView<T>& B, const T* T_val, const T* X, int ld, in
     const int nb = colstats_blocks<T>(B.n, ncols, &width);
     size_t smem = (size_t)ny * nvec * 2 * W * sizeof(double);
     BAMG_LAUNCH((k_colstats<T, MODE>), nb, dim3(nvec, ny), smem, s, B.n, B.rp, B.ci, B.v, T_val, X, ld, col0, nvec,
-                partial);
+                cw.partial, cw.ticket);
 }
-// sums[q] for q < width from the partials, one warp per output (lanes stride the blocks,
-// then a fixed butterfly); a block of COLSUM_T threads.
-constexpr int COLSUM_T = 256;
-__device__ void colsum_partials(int nblocks, int width, const double* __restrict__ partial, double* sums) {
+// sums[q] for q < width from the partials, one warp per output (lanes stride the blocks, then a
+// fixed butterfly), COLSUM_T / 32 outputs a block of the grid.  True in every thread of the block that
+// finishes last, which sees all sums.  One block for all outputs took 16 us for 128 partials of 40
+// outputs and 32 for 512 of 48: some 900 FP64 additions of a warp, 16 cycles each on one SM's pipe.
+constexpr int COLSUM_T = 128;
+static int colsum_blocks(int width) { return (width + COLSUM_T / 32 - 1) / (COLSUM_T / 32); }
+__device__ bool colsum_partials(int nblocks, int width, const double* __restrict__ partial, double* sums,
+                                unsigned* ticket) {
+    __shared__ int s_last;
     const int lane = threadIdx.x & 31;
-    for (int q = threadIdx.x >> 5; q < width; q += COLSUM_T / 32) {
+    const int q = blockIdx.x * (COLSUM_T / 32) + (threadIdx.x >> 5);
+    if (q < width) {
         double s = 0.0;
+#pragma unroll 4
         for (int b = lane; b < nblocks; b += 32) s += partial[(int64_t)b * width + q];
         s = warp_sum(s);
-        if (lane == 0) sums[q] = s;
+        if (lane == 0) {
+            sums[q] = s;
+            __threadfence();
+        }
     }
     __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (!s_last) return false;
+    __threadfence();
+    return true;
 }
 
 // ---------------------------------------------------------------- LS weights
 // nrm[k] = ||x_k||_2 and nrm[32 + k] = 1 / nrm[k] (used by FP32 test vectors)
-__global__ void __launch_bounds__(COLSUM_T) k_weights(int ncols, int W, int nblocks, const double* __restrict__ partial,
+__global__ void __launch_bounds__(COLSUM_T) k_weights(int ncols, int W, int nblocks, const ColWork cw,
                                                         const uint8_t* __restrict__ active, double floor,
                                                         double* __restrict__ w, double* __restrict__ nrm) {
     pdl_begin();
-    __shared__ double sums[64];
-    colsum_partials(nblocks, 2 * ((ncols + W - 1) / W) * W, partial, sums);
+    if (!colsum_partials(nblocks, 2 * ((ncols + W - 1) / W) * W, cw.partial, cw.sums, cw.ticket)) return;
     if (threadIdx.x >= 32) return;
     const int k = threadIdx.x;  // one warp, ncols <= 32
     double m = 0.0, nk = 1.0;
     if (k < ncols) {
         const int ch = k / W, e = k - ch * W;
-        const double xx = sums[ch * 2 * W + e], bb = sums[ch * 2 * W + W + e];
+        const double xx = __ldcg(cw.sums + ch * 2 * W + e), bb = __ldcg(cw.sums + ch * 2 * W + W + e);
         const bool act = active ? active[k] != 0 : true;
         if (act && xx > 0.0) {
             nk = sqrt(xx);
@@ -625,24 +648,24 @@ void tv_weights(const MatView<T>& B, int ncols, int ld, int col0, const uint8_t*
     BAMG_REQUIRE(ncols >= 1 && ncols <= 32, BAMG_EINVAL, "tv_weights: 1 <= ncols <= 32");
     int width = 0;
     const int nb = colstats_blocks<T>(B.n, ncols, &width);
-    TmpBuf<double> partial((size_t)nb * width, s);
-    TmpBuf<double> nrm(64, s);
-    colstats<T, 0>(B, nullptr, X, ld, col0, ncols, partial.get(), s);
-    BAMG_LAUNCH(k_weights, 1, COLSUM_T, 0, s, ncols, W, nb, (const double*)partial.get(), d_active, floor, d_w,
-                nrm.get());
-    BAMG_LAUNCH(k_scale_cols<T>, blocks_for((int64_t)B.n * ncols, 256), 256, 0, s, B.n, X, ld, col0, ncols, nrm.get());
+    TmpBuf<double> work(64 + ColWork::doubles(nb, width), s);
+    double* nrm = work.get();
+    const ColWork cw(nrm + 64, nb, width);
+    colstats<T, 0>(B, nullptr, X, ld, col0, ncols, cw, s);
+    BAMG_LAUNCH(k_weights, colsum_blocks(width), COLSUM_T, 0, s, ncols, W, nb, cw, d_active, floor, d_w, nrm);
+    BAMG_LAUNCH(k_scale_cols<T>, blocks_for((int64_t)B.n * ncols, 256), 256, 0, s, B.n, X, ld, col0, ncols,
+                (const double*)nrm);
 }
 
 // ---------------------------------------------------------------- Rayleigh update
-__global__ void __launch_bounds__(COLSUM_T) k_rayleigh(int ncols, int W, int nblocks, const double* __restrict__ partial,
-                                                         double tol, double* __restrict__ lam, uint8_t* __restrict__ sel) {
+__global__ void __launch_bounds__(COLSUM_T) k_rayleigh(int ncols, int W, int nblocks, const ColWork cw, double tol,
+                                                         double* __restrict__ lam, uint8_t* __restrict__ sel) {
     pdl_begin();
-    __shared__ double sums[64];
-    colsum_partials(nblocks, 2 * ((ncols + W - 1) / W) * W, partial, sums);
+    if (!colsum_partials(nblocks, 2 * ((ncols + W - 1) / W) * W, cw.partial, cw.sums, cw.ticket)) return;
     const int k = threadIdx.x;
     if (k >= ncols) return;
     const int ch = k / W, e = k - ch * W;
-    const double num = sums[ch * 2 * W + e], den = sums[ch * 2 * W + W + e];
+    const double num = __ldcg(cw.sums + ch * 2 * W + e), den = __ldcg(cw.sums + ch * 2 * W + W + e);
     const double old = lam[k];
     const double nw = (k == 0) ? 0.0 : num / den;
     const double change = fabs(nw - old) / fmax(fabs(old), 1e-300);
@@ -656,9 +679,10 @@ void rayleigh_update(const MatView<T>& B, const T* T_val, const T* X, int ncols,
     constexpr int W = V16<T>::W;
     int width = 0;
     const int nb = colstats_blocks<T>(B.n, ncols, &width);
-    TmpBuf<double> partial((size_t)nb * width, s);
-    colstats<T, 1>(B, T_val, X, ld, col0, ncols, partial.get(), s);
-    BAMG_LAUNCH(k_rayleigh, 1, COLSUM_T, 0, s, ncols, W, nb, (const double*)partial.get(), tol, d_lam, d_sel);
+    TmpBuf<double> work(ColWork::doubles(nb, width), s);
+    const ColWork cw(work.get(), nb, width);
+    colstats<T, 1>(B, T_val, X, ld, col0, ncols, cw, s);
+    BAMG_LAUNCH(k_rayleigh, colsum_blocks(width), COLSUM_T, 0, s, ncols, W, nb, cw, tol, d_lam, d_sel);
 }
 
 // ---------------------------------------------------------------- injection / prolongation

@@ -301,3 +301,31 @@ def test_first_sweep_forms_the_diagonals(shift, rows_entries, n, ncols, nu):
             ref = R[:, c] - 0.7 * s / dd
             assert float((Z[:, c].double() - ref).abs().max()) <= 40 * 2.0 ** -24 * 4.0
     assert torch.equal(X, Y)
+
+
+@pytest.mark.parametrize("nx,ny,ncols", [(2, 1, 1), (17, 19, 32), (300, 250, 10), (1100, 600, 5)])
+def test_weights_over_many_partials(nx, ny, ncols):
+    """Column norms and LS weights in FP64 (one to 512 partial blocks, summed by several blocks) against
+    torch: sums of positive terms, n 2^-53 relative at most, and a quotient."""
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+
+    ptr, col, val = _walk(nx, ny)
+    n = nx * ny
+    row = torch.repeat_interleave(torch.arange(n, device="cuda"), (ptr[1:] - ptr[:-1]).long())
+    i = torch.arange(n, device="cuda")
+    rows, cols = torch.cat([row, i]), torch.cat([col.long(), i])
+    vals = torch.cat([-val, torch.ones(n, dtype=torch.float64, device="cuda")])
+    order = torch.argsort(rows * n + cols)
+    B = ((ptr + torch.arange(n + 1, device="cuda")).int(), cols[order].int(), vals[order].contiguous())
+    X = 1.0 + torch.rand(n, ncols + ncols % 2, dtype=torch.float64, device="cuda")
+    ref = X[:, :ncols] / torch.linalg.vector_norm(X[:, :ncols], dim=0)
+    count = (B[0][1:] - B[0][:-1]).long()
+    bx = torch.stack([torch.segment_reduce(B[2] * ref[:, c].contiguous()[B[1].long()], "sum", lengths=count)
+                      for c in range(ncols)], 1)
+    wr = 1.0 / bx.square().sum(0)
+    w = bamg.tv_weights(B, X, ncols)
+    tol = 64 * n * 2.0 ** -53 + 1e-14
+    assert float(((w - wr / wr.max()).abs() / (wr / wr.max())).max()) <= 1e3 * tol
+    assert float((X[:, :ncols] - ref).abs().max()) <= tol
