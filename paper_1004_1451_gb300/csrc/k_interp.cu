@@ -947,11 +947,190 @@ template <typename T, int CM>
 struct LsFit {
     alignas(16) T xi[KMAX];
     alignas(16) T xj[CM][KMAX];
+    T pad[32 / sizeof(T)];  // the four points of a warp read the same column on distinct banks
 };
 // blocks an SM: as many as leave the registers a candidate's row needs
 constexpr int lsp_blocks(int size, int nc) {
     return size == 4 ? (nc <= 8 ? 6 : nc <= 16 ? 5 : 4) : (nc <= 8 ? 4 : nc <= 16 ? 3 : 2);
 }
+// The greedy fit (Algorithm 2) of one point by GL lanes, a candidate each (ncand <= GL): i64 the
+// point, fine whether it is one to fit (ncand its candidates).  Every lane of the warp calls it.
+template <typename T, int NC, int CM, int GL>
+__device__ __forceinline__ void lsp_fit(int64_t i64, bool fine, int ncand, const int32_t* __restrict__ cidx,
+                                        const int32_t* __restrict__ cand, const T* __restrict__ X, int ncols, int ld,
+                                        const T* s_w, int mmax, int c, double ridge, bool vec, LsFit<T, CM>& sh,
+                                        int32_t* __restrict__ pcol, T* __restrict__ pval, int32_t* __restrict__ pcnt) {
+    constexpr int W = V16<T>::W;
+    const T INF = (T)INFINITY;
+    const int lane = threadIdx.x & 31, sub = lane & (GL - 1);
+    const int node = sub < ncand ? cand[i64 * mmax + sub] : -1;
+    const int ccol = node >= 0 ? cidx[node] : 0;
+    T xs[NC];
+    if (node >= 0) {
+        const T* x = X + (int64_t)node * ld;
+        if (vec) {
+#pragma unroll
+            for (int k = 0; k < NC; k += W)
+                if (k < ncols) {
+                    V16<T>::load(x + k, xs + k);
+#pragma unroll
+                    for (int e = 1; e < W; ++e)
+                        if (k + e >= ncols) xs[k + e] = T(0);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < W; ++e) xs[k + e] = T(0);
+                }
+        } else {
+#pragma unroll
+            for (int k = 0; k < NC; ++k) xs[k] = k < ncols ? x[k] : T(0);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < NC; ++k) xs[k] = T(0);
+    }
+    for (int k = sub; k < NC; k += GL) sh.xi[k] = fine && k < ncols ? X[i64 * ld + k] : T(0);
+    __syncwarp();
+    T gss = T(0), bs = T(0);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        const T wk = s_w[k], v = xs[k];
+        gss += wk * v * v;
+        bs += wk * v * sh.xi[k];
+    }
+    // greedy least squares (Algorithm 2)
+    T gsj[CM], GJJ[CM][CM], bJ[CM], pbest[CM];
+    int J[CM];
+#pragma unroll
+    for (int a = 0; a < CM; ++a) {
+        gsj[a] = bJ[a] = pbest[a] = T(0);
+        J[a] = 0x7fffffff;
+#pragma unroll
+        for (int b = 0; b < CM; ++b) GJJ[a][b] = T(0);
+    }
+    bool used = false, go = fine;
+    int nJ = 0;
+#pragma unroll
+    for (int t = 0; t < CM; ++t) {
+        if (t >= c) break;
+        T L = INF;
+        T pl[CM];
+#pragma unroll
+        for (int a = 0; a < CM; ++a) pl[a] = T(0);
+        if (go && node >= 0 && !used) {
+            T A[CM][CM], rhs[CM];
+            T tr = gss;
+#pragma unroll
+            for (int a = 0; a < CM; ++a) {
+#pragma unroll
+                for (int b = 0; b < CM; ++b) A[a][b] = (a < t && b < t) ? GJJ[a][b] : T(0);
+                rhs[a] = a < t ? bJ[a] : T(0);
+                if (a < t) tr += GJJ[a][a];
+            }
+#pragma unroll
+            for (int a = 0; a < CM; ++a) {
+                if (a < t) {
+                    A[a][t] = gsj[a];
+                    A[t][a] = gsj[a];
+                }
+            }
+            A[t][t] = gss;
+            rhs[t] = bs;
+            const T delta = (T)ridge * tr / (T)(t + 1);
+#pragma unroll
+            for (int a = 0; a < CM; ++a)
+                if (a <= t) A[a][a] += delta;
+            if (chol_solve<T, CM>(A, rhs, t + 1, pl)) {
+                T acc = T(0);
+#pragma unroll
+                for (int k = 0; k < NC; ++k) {
+                    T r = sh.xi[k] - pl[t] * xs[k];
+#pragma unroll
+                    for (int a = 0; a < CM; ++a)
+                        if (a < t) r -= pl[a] * sh.xj[a][k];
+                    acc += s_w[k] * r * r;
+                }
+                L = (acc == acc) ? acc : INF;
+            }
+        }
+        T bestL = L;
+        int bestLane = lane;
+#pragma unroll
+        for (int o = GL / 2; o > 0; o >>= 1) {
+            const T oL = __shfl_xor_sync(0xffffffffu, bestL, o);
+            const int oLane = __shfl_xor_sync(0xffffffffu, bestLane, o);
+            if (oL < bestL || (oL == bestL && oLane < bestLane)) {
+                bestL = oL;
+                bestLane = oLane;
+            }
+        }
+        go = go && bestL < INF;
+        if (!__any_sync(0xffffffffu, go)) break;
+        const T w_gss = __shfl_sync(0xffffffffu, gss, bestLane);
+        const T w_bs = __shfl_sync(0xffffffffu, bs, bestLane);
+        const int w_c = __shfl_sync(0xffffffffu, ccol, bestLane);
+        T w_g[CM], w_p[CM];
+#pragma unroll
+        for (int a = 0; a < CM; ++a) {
+            w_g[a] = __shfl_sync(0xffffffffu, gsj[a], bestLane);
+            w_p[a] = __shfl_sync(0xffffffffu, pl[a], bestLane);
+        }
+        if (go) {
+#pragma unroll
+            for (int a = 0; a < CM; ++a) {
+                if (a < t) {
+                    GJJ[t][a] = w_g[a];
+                    GJJ[a][t] = w_g[a];
+                }
+                pbest[a] = a <= t ? w_p[a] : T(0);
+            }
+            GJJ[t][t] = w_gss;
+            bJ[t] = w_bs;
+            J[t] = w_c;
+            nJ = t + 1;
+            if (lane == bestLane) {  // the winner's row, from its registers
+                used = true;
+#pragma unroll
+                for (int k = 0; k < NC; k += W) V16<T>::store(&sh.xj[t][k], xs + k);
+            }
+        }
+        __syncwarp();
+        if (t + 1 < CM && t + 1 < c) {
+            T g = T(0);
+#pragma unroll
+            for (int k = 0; k < NC; ++k) g += s_w[k] * xs[k] * sh.xj[t][k];
+            gsj[t] = g;
+        }
+    }
+    if (fine && sub == 0) {
+        T vals[CM];
+#pragma unroll
+        for (int a = 0; a < CM; ++a) vals[a] = pbest[a];
+#pragma unroll
+        for (int a = 1; a < CM; ++a)  // by coarse index; empty slots (index 0x7fffffff) last
+#pragma unroll
+            for (int b = a; b > 0; --b)
+                if (J[b - 1] > J[b]) {
+                    const int tc = J[b];
+                    J[b] = J[b - 1];
+                    J[b - 1] = tc;
+                    const T tv = vals[b];
+                    vals[b] = vals[b - 1];
+                    vals[b - 1] = tv;
+                }
+#pragma unroll
+        for (int a = 0; a < CM; ++a)
+            if (a < c) {
+                pcol[i64 * c + a] = a < nJ ? J[a] : -1;
+                pval[i64 * c + a] = a < nJ ? vals[a] : T(0);
+            }
+        pcnt[i64] = nJ;
+    }
+    __syncwarp();  // the shared memory takes the next points
+}
+
+// Four points a warp at a time: eight lanes each where none has more than eight candidates (full
+// coarsening of a grid gives two or four, an independent set of a triangulation five to eight), else two
+// by two with 16 lanes.
 template <typename T, int NC, int CM>
 __global__ void __launch_bounds__(LSP_WARPS * 32, lsp_blocks(sizeof(T), NC))
     k_ls_pair(int n, const uint8_t* __restrict__ cf, const int32_t* __restrict__ cidx, const int32_t* __restrict__ cand,
@@ -959,191 +1138,39 @@ __global__ void __launch_bounds__(LSP_WARPS * 32, lsp_blocks(sizeof(T), NC))
               const double* __restrict__ w, int mmax, int c, double ridge, bool vec, int32_t* __restrict__ pcol,
               T* __restrict__ pval, int32_t* __restrict__ pcnt) {
     pdl_begin();
-    constexpr int W = V16<T>::W;
-    __shared__ LsFit<T, CM> s_half[LSP_WARPS][2];
+    __shared__ LsFit<T, CM> s_fit[LSP_WARPS][4];
     __shared__ alignas(16) T s_w[KMAX];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane & 15, hb = lane & 16;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x < KMAX) s_w[threadIdx.x] = threadIdx.x < ncols ? (T)w[threadIdx.x] : T(0);
     __syncthreads();
-    LsFit<T, CM>& sh = s_half[wid][hb >> 4];
-    const T INF = (T)INFINITY;
-    const int64_t pairs = ((int64_t)n + 1) / 2, stride = (int64_t)gridDim.x * LSP_WARPS;
+    const int64_t quads = ((int64_t)n + 3) / 4, stride = (int64_t)gridDim.x * LSP_WARPS;
 #pragma unroll 1
-    for (int64_t q = (int64_t)blockIdx.x * LSP_WARPS + wid; q < pairs; q += stride) {
-        const int64_t i64 = 2 * q + (hb >> 4);
-        const int ncand = i64 < n ? ncands[i64] : -1;
-        const bool fine = ncand >= 0;
-        if (i64 < n && !fine && cf[i64]) {  // a coarse point's unit row
+    for (int64_t q = (int64_t)blockIdx.x * LSP_WARPS + wid; q < quads; q += stride) {
+        const int64_t i = 4 * q + (lane >> 3);
+        const int m = i < n ? ncands[i] : -1;
+        if (i < n && m < 0 && cf[i]) {  // a coarse point's unit row
+            const int sub = lane & 7;
             if (sub < c) {
-                pcol[i64 * c + sub] = sub == 0 ? cidx[i64] : -1;
-                pval[i64 * c + sub] = sub == 0 ? T(1) : T(0);
+                pcol[i * c + sub] = sub == 0 ? cidx[i] : -1;
+                pval[i * c + sub] = sub == 0 ? T(1) : T(0);
             }
-            if (sub == 0) pcnt[i64] = 1;
+            if (sub == 0) pcnt[i] = 1;
         }
-        if (!__any_sync(0xffffffffu, fine)) continue;
-        const int node = sub < ncand ? cand[i64 * mmax + sub] : -1;
-        const int ccol = node >= 0 ? cidx[node] : 0;
-        T xs[NC];
-        if (node >= 0) {
-            const T* x = X + (int64_t)node * ld;
-            if (vec) {
-#pragma unroll
-                for (int k = 0; k < NC; k += W)
-                    if (k < ncols) {
-                        V16<T>::load(x + k, xs + k);
-#pragma unroll
-                        for (int e = 1; e < W; ++e)
-                            if (k + e >= ncols) xs[k + e] = T(0);
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < W; ++e) xs[k + e] = T(0);
-                    }
-            } else {
-#pragma unroll
-                for (int k = 0; k < NC; ++k) xs[k] = k < ncols ? x[k] : T(0);
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < NC; ++k) xs[k] = T(0);
+        const unsigned any = __ballot_sync(0xffffffffu, m >= 0);
+        if (!any) continue;
+        if (!__any_sync(0xffffffffu, m > 8)) {
+            lsp_fit<T, NC, CM, 8>(i, m >= 0, m, cidx, cand, X, ncols, ld, s_w, mmax, c, ridge, vec, s_fit[wid][lane >> 3],
+                                  pcol, pval, pcnt);
+            continue;
         }
-        for (int k = sub; k < NC; k += 16) sh.xi[k] = fine && k < ncols ? X[i64 * ld + k] : T(0);
-        __syncwarp();
-        T gss = T(0), bs = T(0);
-#pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            const T wk = s_w[k], v = xs[k];
-            gss += wk * v * v;
-            bs += wk * v * sh.xi[k];
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            if (!((any >> (16 * h)) & 0xffffu)) continue;
+            const int g = 2 * h + (lane >> 4);
+            const int mg = __shfl_sync(0xffffffffu, m, 8 * g);
+            lsp_fit<T, NC, CM, 16>(4 * q + g, mg >= 0, mg, cidx, cand, X, ncols, ld, s_w, mmax, c, ridge, vec,
+                                   s_fit[wid][g], pcol, pval, pcnt);
         }
-        // greedy least squares (Algorithm 2)
-        T gsj[CM], GJJ[CM][CM], bJ[CM], pbest[CM];
-        int J[CM];
-#pragma unroll
-        for (int a = 0; a < CM; ++a) {
-            gsj[a] = bJ[a] = pbest[a] = T(0);
-            J[a] = 0x7fffffff;
-#pragma unroll
-            for (int b = 0; b < CM; ++b) GJJ[a][b] = T(0);
-        }
-        bool used = false, go = fine;
-        int nJ = 0;
-#pragma unroll
-        for (int t = 0; t < CM; ++t) {
-            if (t >= c) break;
-            T L = INF;
-            T pl[CM];
-#pragma unroll
-            for (int a = 0; a < CM; ++a) pl[a] = T(0);
-            if (go && node >= 0 && !used) {
-                T A[CM][CM], rhs[CM];
-                T tr = gss;
-#pragma unroll
-                for (int a = 0; a < CM; ++a) {
-#pragma unroll
-                    for (int b = 0; b < CM; ++b) A[a][b] = (a < t && b < t) ? GJJ[a][b] : T(0);
-                    rhs[a] = a < t ? bJ[a] : T(0);
-                    if (a < t) tr += GJJ[a][a];
-                }
-#pragma unroll
-                for (int a = 0; a < CM; ++a) {
-                    if (a < t) {
-                        A[a][t] = gsj[a];
-                        A[t][a] = gsj[a];
-                    }
-                }
-                A[t][t] = gss;
-                rhs[t] = bs;
-                const T delta = (T)ridge * tr / (T)(t + 1);
-#pragma unroll
-                for (int a = 0; a < CM; ++a)
-                    if (a <= t) A[a][a] += delta;
-                if (chol_solve<T, CM>(A, rhs, t + 1, pl)) {
-                    T acc = T(0);
-#pragma unroll
-                    for (int k = 0; k < NC; ++k) {
-                        T r = sh.xi[k] - pl[t] * xs[k];
-#pragma unroll
-                        for (int a = 0; a < CM; ++a)
-                            if (a < t) r -= pl[a] * sh.xj[a][k];
-                        acc += s_w[k] * r * r;
-                    }
-                    L = (acc == acc) ? acc : INF;
-                }
-            }
-            T bestL = L;
-            int bestLane = lane;
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) {
-                const T oL = __shfl_xor_sync(0xffffffffu, bestL, o);
-                const int oLane = __shfl_xor_sync(0xffffffffu, bestLane, o);
-                if (oL < bestL || (oL == bestL && oLane < bestLane)) {
-                    bestL = oL;
-                    bestLane = oLane;
-                }
-            }
-            go = go && bestL < INF;
-            if (!__any_sync(0xffffffffu, go)) break;
-            const T w_gss = __shfl_sync(0xffffffffu, gss, bestLane);
-            const T w_bs = __shfl_sync(0xffffffffu, bs, bestLane);
-            const int w_c = __shfl_sync(0xffffffffu, ccol, bestLane);
-            T w_g[CM], w_p[CM];
-#pragma unroll
-            for (int a = 0; a < CM; ++a) {
-                w_g[a] = __shfl_sync(0xffffffffu, gsj[a], bestLane);
-                w_p[a] = __shfl_sync(0xffffffffu, pl[a], bestLane);
-            }
-            if (go) {
-#pragma unroll
-                for (int a = 0; a < CM; ++a) {
-                    if (a < t) {
-                        GJJ[t][a] = w_g[a];
-                        GJJ[a][t] = w_g[a];
-                    }
-                    pbest[a] = a <= t ? w_p[a] : T(0);
-                }
-                GJJ[t][t] = w_gss;
-                bJ[t] = w_bs;
-                J[t] = w_c;
-                nJ = t + 1;
-                if (lane == bestLane) {  // the winner's row, from its registers
-                    used = true;
-#pragma unroll
-                    for (int k = 0; k < NC; k += W) V16<T>::store(&sh.xj[t][k], xs + k);
-                }
-            }
-            __syncwarp();
-            if (t + 1 < CM && t + 1 < c) {
-                T g = T(0);
-#pragma unroll
-                for (int k = 0; k < NC; ++k) g += s_w[k] * xs[k] * sh.xj[t][k];
-                gsj[t] = g;
-            }
-        }
-        if (fine && sub == 0) {
-            T vals[CM];
-#pragma unroll
-            for (int a = 0; a < CM; ++a) vals[a] = pbest[a];
-#pragma unroll
-            for (int a = 1; a < CM; ++a)  // by coarse index; empty slots (index 0x7fffffff) last
-#pragma unroll
-                for (int b = a; b > 0; --b)
-                    if (J[b - 1] > J[b]) {
-                        const int tc = J[b];
-                        J[b] = J[b - 1];
-                        J[b - 1] = tc;
-                        const T tv = vals[b];
-                        vals[b] = vals[b - 1];
-                        vals[b - 1] = tv;
-                    }
-#pragma unroll
-            for (int a = 0; a < CM; ++a)
-                if (a < c) {
-                    pcol[i64 * c + a] = a < nJ ? J[a] : -1;
-                    pval[i64 * c + a] = a < nJ ? vals[a] : T(0);
-                }
-            pcnt[i64] = nJ;
-        }
-        __syncwarp();  // the halves' shared memory takes the next pair
     }
 }
 
@@ -1192,7 +1219,7 @@ int interp_ls(int n, int nnz, const int32_t* rp, const int32_t* ci, const T* bv,
         else
             search(k_ls_search<16, 1>, 2 * LSP_WARPS, (int64_t)nnz <= 4 * (int64_t)n ? 2 : 3);
         const unsigned grid =
-            (unsigned)std::min<int64_t>(((int64_t)n + 2 * LSP_WARPS - 1) / (2 * LSP_WARPS), (int64_t)nsm * 12);
+            (unsigned)std::min<int64_t>(((int64_t)n + 4 * LSP_WARPS - 1) / (4 * LSP_WARPS), (int64_t)nsm * 12);
         constexpr int W = V16<T>::W;
         const bool vec = ld % W == 0 && ((uintptr_t)X & 15) == 0;
         auto go = [&](auto kern) {

@@ -252,7 +252,7 @@ def test_odd_sweep_counts_write_every_row(dtype, nx, ny, ncols):
 
 @pytest.mark.parametrize("shift", [False, True])
 @pytest.mark.parametrize("rows_entries,n,ncols,nu", [(3, 1, 4, 1), (5, 1000, 10, 2), (5, 400001, 16, 3), (14, 3001, 7, 2),
-                                                     (14, 300000, 8, 1)])
+                                                     (14, 300000, 12, 1)])
 def test_first_sweep_forms_the_diagonals(shift, rows_entries, n, ncols, nu):
     """FP32 sweeps whose first one reads the diagonals off the rows, against sweeps one call at a time
     with the diagonals at hand (relax_noalloc where it fits, else single-sweep calls): same bits, the
