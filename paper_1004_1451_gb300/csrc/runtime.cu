@@ -1701,7 +1701,9 @@ int bamg_solve_batch(int nchains, const bamg_csr* As, const int* r, const int* l
         return BAMG_EINVAL;
     }
     if (nchains == 0) return BAMG_OK;
-    if (nworkers <= 0) nworkers = std::min(16, std::max(1, (nchains + 3) / 4));
+    // a thread per chain up to 16: 12 chains of 32..60 squared states in FP64 took 10.8 ms on 3 threads and
+    // 5.9 on 12, 32 chains 15.1 on 8 and 14.6 on 16, 96 chains 55.7 on 8 and 50.0 on 16
+    if (nworkers <= 0) nworkers = std::min(16, nchains);
     nworkers = std::min(nworkers, nchains);
     // largest chains first: the queue ends with the short jobs
     std::vector<int> order(nchains);
