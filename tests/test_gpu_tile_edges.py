@@ -329,3 +329,45 @@ def test_weights_over_many_partials(nx, ny, ncols):
     tol = 64 * n * 2.0 ** -53 + 1e-14
     assert float(((w - wr / wr.max()).abs() / (wr / wr.max())).max()) <= 1e3 * tol
     assert float((X[:, :ncols] - ref).abs().max()) <= tol
+
+
+@pytest.mark.parametrize("kind,n", [("path", 2), ("path", 5000), ("grid", 70000), ("star", 3000), ("dense", 700)])
+def test_independent_set_is_the_greedy_one(kind, n):
+    """The splitting before any relaxation round (max_rounds 0) is the greedy independent set by
+    descending (priority, index): long chains of waiting neighbours, more than 64 neighbours a state
+    (their states are then looked up again), rows of one direction only."""
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+    from oracle import bamg as ob
+
+    rng = np.random.default_rng(n)
+    if kind == "path":
+        a, b = np.arange(n - 1), np.arange(1, n)
+    elif kind == "grid":
+        i = np.arange(n)
+        a, b = np.concatenate([i[:-1], i[:-250]]), np.concatenate([i[1:], i[250:]])
+    elif kind == "star":
+        a, b = np.concatenate([np.zeros(n - 1, int), np.ones(n - 2, int)]), np.concatenate([np.arange(1, n), np.arange(2, n)])
+    else:
+        a = np.repeat(np.arange(n), 60)
+        b = rng.integers(0, n, a.size)
+    import scipy.sparse as sp
+
+    A = sp.csr_matrix((np.full(a.size, -0.01), (a, b)), shape=(n, n))  # edges stored one way
+    A.setdiag(1.0)
+    A = sp.csr_matrix(A)
+    A.sort_indices()
+    B = (torch.tensor(A.indptr.astype(np.int32), device="cuda"), torch.tensor(A.indices.astype(np.int32), device="cuda"),
+         torch.tensor(A.data, device="cuda"))
+    cf, _, nc, _ = bamg.coarsen_cr(B, 3, 11, max_rounds=0)
+    pri = ob.counter_u64(11, (1 << 23) + (3 << 8), np.arange(n, dtype=np.uint64))
+    S = sp.csr_matrix(A + A.T)
+    want = np.zeros(n, dtype=bool)
+    gone = np.zeros(n, dtype=bool)
+    for i in sorted(range(n), key=lambda k: (int(pri[k]), k), reverse=True):
+        if not gone[i]:
+            want[i] = True
+            gone[S.indices[S.indptr[i]:S.indptr[i + 1]]] = True
+            gone[i] = True
+    assert np.array_equal(cf.cpu().numpy().astype(bool), want) and nc == want.sum()
