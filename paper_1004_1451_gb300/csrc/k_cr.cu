@@ -39,67 +39,95 @@ __device__ __forceinline__ bool beats(uint64_t pi, int i, uint64_t pj, int j) { 
 // started, long chains) the next launch settles.  Rounds as two kernels each, four rounds between the
 // host's checks, took 8 launches and 35 us where one and 10 us do (65,536 states).
 // st: 1 undecided candidate, 0 no candidate or out, 2 in.
+//
+// G lanes share a row on levels of long rows (lanes_per_row): one lane looking at a row's 30 to 70
+// neighbours, one dependent load after the other, took most of the sets' time (46 us a set on average over
+// a planar chain of 2^18 states; 24 on its long-row levels with the lanes).
 constexpr int MIS_LOOKS = 24;
+template <int G>
 __global__ void k_mis(int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                       const int32_t* __restrict__ rpT, const int32_t* __restrict__ ciT, uint8_t* st,
                       uint8_t* __restrict__ chosen, uint64_t seed, uint64_t stream, int* __restrict__ left) {
     pdl_begin();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    constexpr unsigned ALL = 0xffffffffu;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (int)(t / G), sub = (int)(t % G);
     volatile uint8_t* vst = st;
-    if (i >= n || vst[i] != 1) return;
+    bool done = i >= n || vst[i] != 1;  // the same in a row's lanes: only they change its state
+    if (G == 1 ? done : !__any_sync(ALL, !done)) return;
+    // true if p is in any of the row's lanes (all lanes of the warp take part)
+    auto any = [&](bool p) {
+        if constexpr (G == 1) return p;
+        return ((__ballot_sync(ALL, p) >> ((threadIdx.x & 31) & ~(G - 1))) & (ALL >> (32 - G))) != 0;
+    };
     const uint64_t pi = counter_u64(seed, stream, (uint64_t)i);
-    const int a = rp[i], na = rp[i + 1] - a, b = rpT[i], tot = na + rpT[i + 1] - b;
+    const int a = done ? 0 : rp[i], na = done ? 0 : rp[i + 1] - a, b = done ? 0 : rpT[i],
+              tot = done ? 0 : na + rpT[i + 1] - b;
     auto neighbour = [&](int k) { return k < na ? ci[a + k] : ciT[b + k - na]; };
-    unsigned long long beat = 0ull;  // the undecided neighbours that beat i, among the first 64
+    unsigned long long beat = 0ull;  // the undecided neighbours that beat i, among this lane's first 64
     bool out = false, wait = false;
-    for (int k = 0; k < tot && !out; ++k) {
+    for (int k = sub; k < tot && !out; k += G) {
         const int j = neighbour(k);
         const int s = j != i ? vst[j] : 0;
         if (s == 0 || beats(pi, i, counter_u64(seed, stream, (uint64_t)j), j)) continue;
         out = s == 2;
         wait = true;
-        if (k < 64) beat |= 1ull << k;
+        if (k < 64 * G) beat |= 1ull << (k / G);
     }
     // settled in the loop, not after it: lanes of the same warp wait for one another
     auto settle = [&] {
-        if (out) {
-            vst[i] = 0;
-        } else if (!wait) {
-            vst[i] = 2;
-            chosen[i] = 1;
-        }
-        return out || !wait;
+        const bool o = any(out), w = any(wait);
+        if (done) return;
+        done = o || !w;
+        if (!done || sub != 0) return;
+        vst[i] = o ? 0 : 2;
+        if (!o) chosen[i] = 1;
     };
-    bool done = settle();
-    for (int look = 0; look < MIS_LOOKS && !done; ++look) {
-        wait = false;
-        for (unsigned long long m = beat; m && !out; m &= m - 1) {
-            const int k = __ffsll((long long)m) - 1, s = vst[neighbour(k)];
-            if (s == 0)
-                beat &= ~(1ull << k);
-            else if (s == 2)
-                out = true;
-            else
+    settle();
+    for (int look = 0; look < MIS_LOOKS; ++look) {
+        if (G == 1 ? done : !__any_sync(ALL, !done)) break;
+        out = wait = false;
+        if (!done) {
+            for (unsigned long long m = beat; m && !out; m &= m - 1) {
+                const int k = __ffsll((long long)m) - 1, s = vst[neighbour(sub + k * G)];
+                if (s == 0)
+                    beat &= ~(1ull << k);
+                else if (s == 2)
+                    out = true;
+                else
+                    wait = true;
+            }
+            for (int k = sub + 64 * G; k < tot && !out; k += G) {
+                const int j = neighbour(k);
+                const int s = j != i ? vst[j] : 0;
+                if (s == 0 || beats(pi, i, counter_u64(seed, stream, (uint64_t)j), j)) continue;
+                out = s == 2;
                 wait = true;
+            }
         }
-        for (int k = 64; k < tot && !out; ++k) {
-            const int j = neighbour(k);
-            const int s = j != i ? vst[j] : 0;
-            if (s == 0 || beats(pi, i, counter_u64(seed, stream, (uint64_t)j), j)) continue;
-            out = s == 2;
-            wait = true;
-        }
-        done = settle();
+        settle();
     }
-    if (!done) atomicAdd(left, 1);
+    if (!done && sub == 0) atomicAdd(left, 1);
 }
 
 // chosen |= independent set of the candidates (und: 1 on entry; consumed)
-static void independent_set(int n, const int32_t* rp, const int32_t* ci, const int32_t* rpT, const int32_t* ciT,
-                            uint8_t* und, uint8_t* chosen, int* left, uint64_t seed, uint64_t stream, cudaStream_t s) {
+static void independent_set(int n, int nnz, const int32_t* rp, const int32_t* ci, const int32_t* rpT,
+                            const int32_t* ciT, uint8_t* und, uint8_t* chosen, int* left, uint64_t seed, uint64_t stream,
+                            cudaStream_t s) {
+    const int G = lanes_per_row(n, nnz);
     for (int round = 0; round <= n; ++round) {  // every launch settles at least one
         BAMG_CK(cudaMemsetAsync(left, 0, sizeof(int), s));
-        BAMG_LAUNCH(k_mis, blocks_for(n, 256), 256, 0, s, n, rp, ci, rpT, ciT, und, chosen, seed, stream, left);
+        auto go = [&](auto kern) {
+            BAMG_LAUNCH(kern, blocks_for((int64_t)n * G, 256), 256, 0, s, n, rp, ci, rpT, ciT, und, chosen, seed, stream,
+                        left);
+        };
+        switch (G) {
+            case 1: go(k_mis<1>); break;
+            case 4: go(k_mis<4>); break;
+            case 8: go(k_mis<8>); break;
+            case 16: go(k_mis<16>); break;
+            default: go(k_mis<32>);
+        }
         if (read_int(left, s) == 0) return;
     }
     throw Error(BAMG_ETIMEOUT, "independent set did not terminate");
@@ -282,7 +310,7 @@ int coarsen_cr(const MatView<T>& B, int level, uint64_t seed, double theta, int 
     BAMG_LAUNCH(k_tfill, g, 256, 0, s, n, B.rp, B.ci, (const int32_t*)rpT, cursor, ciT);
     BAMG_CK(cudaMemsetAsync(cf, 0, n, s));
     BAMG_CK(cudaMemsetAsync(und, 1, n, s));
-    independent_set(n, B.rp, B.ci, rpT, ciT, und, cf, left, seed, STREAM_MIS + ((uint64_t)level << 8), s);
+    independent_set(n, B.nnz, B.rp, B.ci, rpT, ciT, und, cf, left, seed, STREAM_MIS + ((uint64_t)level << 8), s);
     int rounds = 0;
     double h[2];
     for (;;) {
@@ -314,7 +342,7 @@ int coarsen_cr(const MatView<T>& B, int level, uint64_t seed, double theta, int 
         if (!(rho > theta) || rounds >= max_rounds || h[0] == 0.0) break;
         BAMG_LAUNCH(k_cr_slow, g, 256, 0, s, n, (const uint8_t*)cf, (const double*)prev, cur, theta, cand);
         ++rounds;
-        independent_set(n, B.rp, B.ci, rpT, ciT, cand, cf, left, seed,
+        independent_set(n, B.nnz, B.rp, B.ci, rpT, ciT, cand, cf, left, seed,
                         STREAM_MIS + ((uint64_t)level << 8) + rounds, s);
     }
     BAMG_LAUNCH(k_u8_to_i32, g, 256, 0, s, n, (const uint8_t*)cf, cnt);
@@ -362,7 +390,7 @@ void colour_classes(int n, int nnz, const int32_t* rp, const int32_t* ci, int le
     for (int c = 0; c < MAX_COLOURS; ++c) {
         BAMG_CK(cudaMemcpyAsync(und.get(), left.get(), n, cudaMemcpyDeviceToDevice, s));
         BAMG_CK(cudaMemsetAsync(chosen.get(), 0, n, s));
-        independent_set(n, rp, ci, rpT.get(), ciT.get(), und.get(), chosen.get(), undecided.get(), seed,
+        independent_set(n, nnz, rp, ci, rpT.get(), ciT.get(), und.get(), chosen.get(), undecided.get(), seed,
                         STREAM_COLOUR + ((uint64_t)level << 8) + (uint64_t)c, s);
         BAMG_CK(cudaMemsetAsync(rem.get(), 0, sizeof(int), s));
         BAMG_LAUNCH(k_colour_take, g, 256, 0, s, n, (const uint8_t*)chosen.get(), c, colour.get(), left.get(),

@@ -331,11 +331,13 @@ def test_weights_over_many_partials(nx, ny, ncols):
     assert float((X[:, :ncols] - ref).abs().max()) <= tol
 
 
-@pytest.mark.parametrize("kind,n", [("path", 2), ("path", 5000), ("grid", 70000), ("star", 3000), ("dense", 700)])
+@pytest.mark.parametrize("kind,n", [("path", 2), ("path", 5000), ("grid", 70000), ("star", 3000), ("dense", 700),
+                                    ("hub", 2000), (30, 900), (150, 301)])
 def test_independent_set_is_the_greedy_one(kind, n):
     """The splitting before any relaxation round (max_rounds 0) is the greedy independent set by
     descending (priority, index): long chains of waiting neighbours, more than 64 neighbours a state
-    (their states are then looked up again), rows of one direction only."""
+    (their states are then looked up again), rows of one direction only, every number of lanes a row
+    (by the mean row length; a hub's row is longer than its lanes remember)."""
     import torch
 
     import paper_1004_1451_gb300 as bamg
@@ -350,8 +352,10 @@ def test_independent_set_is_the_greedy_one(kind, n):
     elif kind == "star":
         a, b = np.concatenate([np.zeros(n - 1, int), np.ones(n - 2, int)]), np.concatenate([np.arange(1, n), np.arange(2, n)])
     else:
-        a = np.repeat(np.arange(n), 60)
+        a = np.repeat(np.arange(n), {"dense": 60, "hub": 14}.get(kind, kind))
         b = rng.integers(0, n, a.size)
+        if kind == "hub":
+            a, b = np.concatenate([a, np.full(n - 1, n - 1)]), np.concatenate([b, np.arange(n - 1)])
     import scipy.sparse as sp
 
     A = sp.csr_matrix((np.full(a.size, -0.01), (a, b)), shape=(n, n))  # edges stored one way
