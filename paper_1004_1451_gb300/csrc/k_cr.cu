@@ -150,8 +150,13 @@ __global__ void k_cr_start(int n, const uint8_t* __restrict__ cf, double* __rest
     }
 }
 
-// One F-relaxation sweep.  u is 0 on C, so every entry of the row takes part: the C entries add
-// zeros, which leaves the sum exactly as it is and spares a load per entry between the index and u.
+// s + b u; a point of C (u = +0) takes no part, whatever the entry's value
+__device__ __forceinline__ double cr_term(double s, double b, double u) {
+    return __double_as_longlong(u) != 0 ? s + b * u : s;
+}
+
+// One F-relaxation sweep.  u is 0 on C and tells the C entries of the row: no load of the flag between
+// the index and u.
 // The quotient omega / b_ii comes from k_cr_start: an FP64 division a row and sweep took a third of
 // the sweep's time on the FP64 pipe (32 us a sweep of 2^18 rows).
 template <typename T>
@@ -172,12 +177,12 @@ __global__ void k_frelax(int n, const int32_t* __restrict__ rp, const int32_t* _
         const int j0 = ci[p], j1 = ci[p + 1], j2 = ci[p + 2], j3 = ci[p + 3];
         const T b0 = bv[p], b1 = bv[p + 1], b2 = bv[p + 2], b3 = bv[p + 3];
         const double u0 = u[j0], u1 = u[j1], u2 = u[j2], u3 = u[j3];
-        s += (double)b0 * u0;
-        s += (double)b1 * u1;
-        s += (double)b2 * u2;
-        s += (double)b3 * u3;
+        s = cr_term(s, (double)b0, u0);
+        s = cr_term(s, (double)b1, u1);
+        s = cr_term(s, (double)b2, u2);
+        s = cr_term(s, (double)b3, u3);
     }
-    for (; p < pe; ++p) s += (double)bv[p] * u[ci[p]];
+    for (; p < pe; ++p) s = cr_term(s, (double)bv[p], u[ci[p]]);
     un[i] = u[i] - w[i] * s;
 }
 
@@ -195,7 +200,7 @@ __global__ void k_frelax_grp(int n, const int32_t* __restrict__ rp, const int32_
     if (live) {
         const int pe = rp[i + 1];
 #pragma unroll 4
-        for (int p = rp[i] + sub; p < pe; p += G) s += (double)bv[p] * u[ci[p]];
+        for (int p = rp[i] + sub; p < pe; p += G) s = cr_term(s, (double)bv[p], u[ci[p]]);
     }
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);

@@ -375,3 +375,33 @@ def test_independent_set_is_the_greedy_one(kind, n):
             gone[S.indices[S.indptr[i]:S.indptr[i + 1]]] = True
             gone[i] = True
     assert np.array_equal(cf.cpu().numpy().astype(bool), want) and nc == want.sum()
+
+
+@pytest.mark.parametrize("per_row", [4, 20])
+def test_entries_of_coarse_columns_take_no_part(per_row):
+    """F-relaxation leaves out the columns of C: an infinite entry there changes no splitting (one lane
+    and several lanes a row).  The first set does not depend on the values, so its columns are known."""
+    import scipy.sparse as sp
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+
+    n = 1500
+    rng = np.random.default_rng(per_row)
+    A = sp.random(n, n, density=per_row / n, random_state=rng, format="csr")
+    A.data[:] = -1.0
+    A = sp.csr_matrix(A + A.T)
+    A.setdiag(0.0)
+    A.setdiag(-np.asarray(A.sum(1)).ravel() + 0.01)
+    A = sp.csr_matrix(A)
+    A.sort_indices()
+    rp, ci = (torch.tensor(v.astype(np.int32), device="cuda") for v in (A.indptr, A.indices))
+    val = torch.tensor(A.data, device="cuda")
+    first = bamg.coarsen_cr((rp, ci, val), 0, 5, max_rounds=0)[0].bool()
+    row = torch.repeat_interleave(torch.arange(n, device="cuda"), (rp[1:] - rp[:-1]).long())
+    hit = first[ci.long()] & ~first[row]
+    want, _, nc, rounds = bamg.coarsen_cr((rp, ci, val), 0, 5, theta=0.3)
+    assert rounds > 0
+    for bad in (float("inf"), float("nan")):
+        got, _, nc2, rounds2 = bamg.coarsen_cr((rp, ci, torch.where(hit, torch.full_like(val, bad), val)), 0, 5, theta=0.3)
+        assert torch.equal(got, want) and nc2 == nc and rounds2 == rounds
