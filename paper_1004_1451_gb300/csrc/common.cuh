@@ -289,7 +289,7 @@ struct ArenaScope {  // sets tmp_arena() for a scope and releases the arena's ch
 };
 
 // Stream-ordered temporary: a slice of the current StackArena when it serves this stream,
-// else cudaMallocAsync / cudaFreeAsync.
+// else a block of the pool.
 template <typename T>
 struct TmpBuf {
     T* p = nullptr;

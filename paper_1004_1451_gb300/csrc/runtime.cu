@@ -1701,14 +1701,29 @@ int bamg_solve_batch(int nchains, const bamg_csr* As, const int* r, const int* l
         return BAMG_EINVAL;
     }
     if (nchains == 0) return BAMG_OK;
-    // a thread per chain up to 16: 12 chains of 32..60 squared states in FP64 took 10.8 ms on 3 threads and
-    // 5.9 on 12, 32 chains 15.1 on 8 and 14.6 on 16, 96 chains 55.7 on 8 and 50.0 on 16
-    if (nworkers <= 0) nworkers = std::min(16, nchains);
+    const bool choose = nworkers <= 0;
+    if (choose) nworkers = 16;
     nworkers = std::min(nworkers, nchains);
     // largest chains first: the queue ends with the short jobs
     std::vector<int> order(nchains);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return As[a].n > As[b].n; });
+    if (choose) {
+        // a thread per chain up to 16: 12 chains of 32..60 squared states in FP64 took 10.8 ms on 3 threads
+        // and 5.9 on 12, 32 chains 15.1 on 8 and 14.6 on 16, 96 chains 55.7 on 8 and 50.0 on 16.  More than
+        // a thread per four chains only while the largest chains together (Krylov and test vectors in
+        // FP64, some ten copies of the matrix) stay below 16 GiB, so that what fitted the device with fewer
+        // in flight does not overflow it: chains of that size fill the GPU by themselves.
+        double bytes = 0.0;
+        int fit = 0;
+        for (; fit < nworkers; ++fit) {
+            const int k = order[fit];
+            const double m = std::min(std::max(opts[k].gmres_m, 1), GMRES_MMAX);
+            bytes += As[k].n * (16.0 * (m + 2) + 40.0 * std::max(r[k], 0) + 400.0) + 160.0 * As[k].nnz;
+            if (!(bytes < 16.0 * (1ull << 30))) break;
+        }
+        nworkers = std::max(fit, std::min(nworkers, std::max(1, (nchains + 3) / 4)));
+    }
     std::atomic<int> next{0};
     std::mutex mu;
     int first_code = BAMG_OK;
