@@ -45,9 +45,10 @@ __device__ __forceinline__ bool beats(uint64_t pi, int i, uint64_t pj, int j) { 
 // a planar chain of 2^18 states; 24 on its long-row levels with the lanes).
 constexpr int MIS_LOOKS = 24;
 template <int G>
-__global__ void k_mis(int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                      const int32_t* __restrict__ rpT, const int32_t* __restrict__ ciT, uint8_t* st,
-                      uint8_t* __restrict__ chosen, uint64_t seed, uint64_t stream, int* __restrict__ left) {
+__global__ void __launch_bounds__(256, 8)
+    k_mis(int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci, const int32_t* __restrict__ rpT,
+          const int32_t* __restrict__ ciT, uint8_t* st, uint8_t* __restrict__ chosen, uint64_t seed, uint64_t stream,
+          int* __restrict__ left) {
     pdl_begin();
     constexpr unsigned ALL = 0xffffffffu;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -66,14 +67,25 @@ __global__ void k_mis(int n, const int32_t* __restrict__ rp, const int32_t* __re
     auto neighbour = [&](int k) { return k < na ? ci[a + k] : ciT[b + k - na]; };
     unsigned long long beat = 0ull;  // the undecided neighbours that beat i, among this lane's first 64
     bool out = false, wait = false;
-    for (int k = sub; k < tot && !out; k += G) {
-        const int j = neighbour(k);
-        const int s = j != i ? vst[j] : 0;
-        if (s == 0 || beats(pi, i, counter_u64(seed, stream, (uint64_t)j), j)) continue;
-        out = s == 2;
-        wait = true;
-        if (k < 64 * G) beat |= 1ull << (k / G);
-    }
+    // four neighbours at a time: their states are loaded without waiting for one another
+    constexpr int U = 4;
+    auto scan = [&](int k0) {
+        for (int k = k0; k < tot && !out; k += U * G) {
+            int j[U], q[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) j[u] = k + u * G < tot ? neighbour(k + u * G) : i;
+#pragma unroll
+            for (int u = 0; u < U; ++u) q[u] = j[u] != i ? vst[j[u]] : 0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (q[u] == 0 || beats(pi, i, counter_u64(seed, stream, (uint64_t)j[u]), j[u])) continue;
+                out |= q[u] == 2;
+                wait = true;
+                if (k + u * G < 64 * G) beat |= 1ull << ((k + u * G) / G);
+            }
+        }
+    };
+    scan(sub);
     // settled in the loop, not after it: lanes of the same warp wait for one another
     auto settle = [&] {
         const bool o = any(out), w = any(wait);
@@ -88,22 +100,23 @@ __global__ void k_mis(int n, const int32_t* __restrict__ rp, const int32_t* __re
         if (G == 1 ? done : !__any_sync(ALL, !done)) break;
         out = wait = false;
         if (!done) {
-            for (unsigned long long m = beat; m && !out; m &= m - 1) {
-                const int k = __ffsll((long long)m) - 1, s = vst[neighbour(sub + k * G)];
-                if (s == 0)
-                    beat &= ~(1ull << k);
-                else if (s == 2)
-                    out = true;
-                else
-                    wait = true;
+            for (unsigned long long m = beat; m && !out;) {
+                int k[U], q[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    k[u] = m ? __ffsll((long long)m) - 1 : -1;
+                    m &= m - 1;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) q[u] = k[u] >= 0 ? vst[neighbour(sub + k[u] * G)] : 0;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (q[u] == 0 && k[u] >= 0) beat &= ~(1ull << k[u]);
+                    out |= q[u] == 2;
+                    wait |= q[u] == 1;
+                }
             }
-            for (int k = sub + 64 * G; k < tot && !out; k += G) {
-                const int j = neighbour(k);
-                const int s = j != i ? vst[j] : 0;
-                if (s == 0 || beats(pi, i, counter_u64(seed, stream, (uint64_t)j), j)) continue;
-                out = s == 2;
-                wait = true;
-            }
+            scan(sub + 64 * G);
         }
         settle();
     }
