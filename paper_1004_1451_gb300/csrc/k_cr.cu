@@ -37,7 +37,7 @@ __device__ __forceinline__ bool beats(uint64_t pi, int i, uint64_t pj, int j) { 
 // again at the neighbours that beat it (their states change once, and only from undecided) until its
 // own is settled, at most MIS_LOOKS times; what is left undecided (neighbours whose blocks had not
 // started, long chains) the next launch settles.  Rounds as two kernels each, four rounds between the
-// host's checks, took 8 launches and 35 us where one and 10 us do (65,536 states).
+// host's checks, took 8 launches and 46 us where one and 24 us do (planar walk of 65,536 states).
 // st: 1 undecided candidate, 0 no candidate or out, 2 in.
 //
 // G lanes share a row on levels of long rows (lanes_per_row): one lane looking at a row's 30 to 70
@@ -67,7 +67,9 @@ __global__ void __launch_bounds__(256, 8)
     auto neighbour = [&](int k) { return k < na ? ci[a + k] : ciT[b + k - na]; };
     unsigned long long beat = 0ull;  // the undecided neighbours that beat i, among this lane's first 64
     bool out = false, wait = false;
-    // four neighbours at a time: their states are loaded without waiting for one another
+    // four neighbours at a time: their states are loaded without waiting for one another (one at a time the
+    // set took 30 us).  More lanes a row than lanes_per_row took 12, but the looks then ran out before the
+    // chains of waiting rows had settled: the second launch, or four times the looks, cost more (10 us a call).
     constexpr int U = 4;
     auto scan = [&](int k0) {
         for (int k = k0; k < tot && !out; k += U * G) {
