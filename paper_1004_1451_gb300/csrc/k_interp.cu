@@ -1524,7 +1524,7 @@ __global__ void k_gal_compact(int nc, const int32_t* __restrict__ poff, const in
 // row of 115 products with a few lanes in each; a row now takes as many as its longest sum (about 30).
 // Rows are handled by a first kernel with room for GAL_CAP_S products per warp (most rows); longer
 // rows go to a list that a second kernel accumulates in a hash table (below), and beyond its capacity
-// by ranges of J.
+// by blocks of columns.
 constexpr int GAL_WARPS_S = 4;
 constexpr int GAL_CAP_S = 256;  // a power of two: also the slots of the row's J table
 constexpr int GAL_CAP_LOG = 8;
@@ -1715,9 +1715,76 @@ __global__ void __launch_bounds__(GAL_WARPS_S * 32)
 // then find or claim their J in an open-addressing table (GAL_HSLOTS slots), the lanes
 // that share a J in a chunk are summed by the lowest one in lane order, so every J
 // accumulates its products in definition order.  The table's entries are finally sorted
-// by J.  A row with more distinct J than half the table is summed by ranges of J.
+// by J.  A row with more distinct J than half the table is summed by blocks of them (gal_row_blocks).
 constexpr int GAL_HSLOTS = 2048;
 constexpr int GAL_STAGE = 32 * 4;  // products of one batch of pairs (caliber <= 4)
+
+// The table's occupied slots by J: skeys[e] = (J, slot) for e below the number of them, which is returned.
+__device__ __forceinline__ int gal_sort_slots(const int* hkey, unsigned long long* skeys) {
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    int u = 0;
+    for (int e0 = 0; e0 < GAL_HSLOTS; e0 += 32) {
+        const int e = e0 + lane;
+        const bool occ = hkey[e] >= 0;
+        const unsigned bal = __ballot_sync(0xffffffffu, occ);
+        if (occ) skeys[u + __popc(bal & lt)] = ((unsigned long long)(unsigned)hkey[e] << 32) | (unsigned)e;
+        u += __popc(bal);
+    }
+    __syncwarp();
+    int N = 32;
+    while (N < u) N <<= 1;
+    for (int e = u + lane; e < N; e += 32) skeys[e] = ~0ull;
+    __syncwarp();
+    for (int k = 2; k <= N; k <<= 1) {
+        for (int jj = k >> 1; jj > 0; jj >>= 1) {
+            for (int e = lane; e < N; e += 32) {
+                const int pe = e ^ jj;
+                if (pe > e) {
+                    const unsigned long long x = skeys[e], y = skeys[pe];
+                    const bool up = (e & k) == 0;
+                    if ((x > y) == up) {
+                        skeys[e] = y;
+                        skeys[pe] = x;
+                    }
+                }
+            }
+            __syncwarp();
+        }
+    }
+    return u;
+}
+// The first u sorted slots to the row's entries from position `at` on; o: the row's product offset.
+template <typename T>
+__device__ __forceinline__ void gal_write_slots(const GalArgs<T>& a, int o, int at, int u, const T* hvb,
+                                                const T* hvt, const unsigned long long* skeys) {
+    for (int e = threadIdx.x & 31; e < u; e += 32) {
+        const unsigned long long kk = skeys[e];
+        const int slot = (int)(kk & 0xffffffffu);
+        a.uJ[o + at + e] = (int32_t)(kk >> 32);
+        a.ubv[o + at + e] = hvb[slot];
+        a.utv[o + at + e] = hvt[slot];
+    }
+}
+// J's slot, claimed if it is not there (linear probing; unrolled, it cost the rows of one
+// table 8%); -1 when the table is full.
+__device__ __forceinline__ int gal_slot(int* hkey, int J, bool& claimed) {
+    unsigned h = ((unsigned)J * 2654435761u) & (GAL_HSLOTS - 1);
+#pragma unroll 1
+    for (int probe = 0; probe < GAL_HSLOTS; ++probe) {
+        const int k = hkey[h];
+        if (k == J) return (int)h;
+        if (k == -1) {
+            const int prev = atomicCAS(&hkey[h], -1, J);
+            if (prev == -1 || prev == J) {
+                claimed = prev == -1;
+                return (int)h;
+            }
+        }
+        h = (h + 1) & (GAL_HSLOTS - 1);
+    }
+    return -1;
+}
 
 template <typename T>
 __device__ bool gal_row_hash(const GalArgs<T>& a, int I, int* hkey, T* hvb, T* hvt, int* sJ, T* sb_, T* st_,
@@ -1777,25 +1844,7 @@ __device__ bool gal_row_hash(const GalArgs<T>& a, int I, int* hkey, T* hvb, T* h
             const bool leader = e < nb && (grp & lt) == 0u;
             bool claimed = false;
             if (leader) {
-                // find or claim the slot of J (linear probing)
-                unsigned h = ((unsigned)J * 2654435761u) & (GAL_HSLOTS - 1);
-                int slot = -1;
-                for (int probe = 0; probe < GAL_HSLOTS; ++probe) {
-                    const int k = hkey[h];
-                    if (k == J) {
-                        slot = (int)h;
-                        break;
-                    }
-                    if (k == -1) {
-                        const int prev = atomicCAS(&hkey[h], -1, J);
-                        if (prev == -1 || prev == J) {
-                            slot = (int)h;
-                            claimed = prev == -1;
-                            break;
-                        }
-                    }
-                    h = (h + 1) & (GAL_HSLOTS - 1);
-                }
+                const int slot = gal_slot(hkey, J, claimed);
                 if (slot >= 0) {
                     T vb = hvb[slot], vt = hvt[slot];
                     unsigned m = grp;
@@ -1812,113 +1861,136 @@ __device__ bool gal_row_hash(const GalArgs<T>& a, int I, int* hkey, T* hvb, T* h
             used += __popc(__ballot_sync(0xffffffffu, claimed));
             __syncwarp();
         }
-        if (used > GAL_HSLOTS / 2) return false;  // too many distinct J: by ranges of J
+        if (used > GAL_HSLOTS / 2) return false;  // too many distinct J: by blocks of them
     }
-    // compact the occupied slots, sort by J, write the row
-    int u = 0;
-    for (int e0 = 0; e0 < GAL_HSLOTS; e0 += 32) {
-        const int e = e0 + lane;
-        const bool occ = hkey[e] >= 0;
-        const unsigned bal = __ballot_sync(0xffffffffu, occ);
-        if (occ) skeys[u + __popc(bal & lt)] = ((unsigned long long)(unsigned)hkey[e] << 32) | (unsigned)e;
-        u += __popc(bal);
-    }
-    __syncwarp();
-    int N = 32;
-    while (N < u) N <<= 1;
-    for (int e = u + lane; e < N; e += 32) skeys[e] = ~0ull;
-    __syncwarp();
-    for (int k = 2; k <= N; k <<= 1) {
-        for (int jj = k >> 1; jj > 0; jj >>= 1) {
-            for (int e = lane; e < N; e += 32) {
-                const int pe = e ^ jj;
-                if (pe > e) {
-                    const unsigned long long x = skeys[e], y = skeys[pe];
-                    const bool up = (e & k) == 0;
-                    if ((x > y) == up) {
-                        skeys[e] = y;
-                        skeys[pe] = x;
-                    }
-                }
-            }
-            __syncwarp();
-        }
-    }
-    for (int e = lane; e < u; e += 32) {
-        const unsigned long long kk = skeys[e];
-        const int slot = (int)(kk & 0xffffffffu);
-        a.uJ[o + e] = (int32_t)(kk >> 32);
-        a.ubv[o + e] = hvb[slot];
-        a.utv[o + e] = hvt[slot];
-    }
+    const int u = gal_sort_slots(hkey, skeys);
+    gal_write_slots(a, o, 0, u, hvb, hvt, skeys);
     if (lane == 0) a.ucnt[I] = u;
     __syncwarp();
     return true;
 }
 
-// A row of any length: the products with J in [lo, lo + GAL_HSLOTS) are added in definition order
-// into a table indexed by J - lo, lo starting at the row's smallest J not yet done; each range's
-// entries come out in order of J.
+// A row of any length, in passes over its products: a pass sums those with J from lo on, as gal_row_hash
+// does, and whenever three quarters of the table are taken keeps the lower half of its columns (hi: the
+// first one it gave up, so every J in [lo, hi) has all its products in the table); the next pass begins at
+// hi.  What bounds it is the chain of loads and shared-memory operations of the one warp, so the passes
+// count: each takes 768 to 1664 columns, whatever the gaps between them.  Ranges of 2048 consecutive J, a range's
+// products all added by one lane, took a pass for every range that the row touches: rows of 1,204 columns
+// scattered over 100,000 took 9.0 ms in FP32 and 9.3 in FP64, now 0.38 and 0.39; over 1,500 (one range)
+// 0.34 and 0.50, now 0.33 and 0.34; rows of 7,800 columns among 10,000 7.0 and 8.1, now 4.5 and 4.6.
 template <typename T>
-__device__ void gal_row_ranges(const GalArgs<T>& a, int I, int* seen, T* tvb, T* tvt) {
+__device__ void gal_row_blocks(const GalArgs<T>& a, int I, int* hkey, T* hvb, T* hvt, int* sJ, T* sb_, T* st_,
+                               unsigned long long* skeys) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const int o = a.poff[I], q0 = a.qrp[I], q1 = a.qrp[I + 1];
+    auto clear = [&] {  // -0: a slot's first product comes out as it is, its sign included
+        for (int e = lane; e < GAL_HSLOTS; e += 32) {
+            hkey[e] = -1;
+            hvb[e] = T(-0.0);
+            hvt[e] = T(-0.0);
+        }
+        __syncwarp();
+    };
     int done = 0, lo = 0;  // entries written; J below lo are done
     for (;;) {
-        int mn = 0x7fffffff;  // the smallest J >= lo
-        for (int q = q0; q < q1; ++q) {
-            const int i = a.qci[q];
-            for (int p = a.rp[i] + lane; p < a.rp[i + 1]; p += 32) {
-                const int j = a.ci[p];
-                for (int sl = 0; sl < a.pcnt[j]; ++sl) {
+        int hi = 0x7fffffff, used = 0;
+        clear();
+        for (int qc = q0; qc < q1; qc += 32) {  // the Q row's entries in chunks of 32, their pairs in batches of 32
+            const int qq = qc + lane;
+            const int ii = qq < q1 ? a.qci[qq] : 0;
+            const int rb = qq < q1 ? a.rp[ii] : 0;
+            const int rl = qq < q1 ? a.rp[ii + 1] - rb : 0;
+            int rinc = rl;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, rinc, d);
+                if (lane >= d) rinc += v;
+            }
+            const int npairs = __shfl_sync(0xffffffffu, rinc, 31);
+            for (int f0 = 0; f0 < npairs; f0 += 32) {
+                const int f = f0 + lane;
+                int k = 0;  // the chunk entry holding pair f: the first with rinc > f
+#pragma unroll
+                for (int st = 16; st >= 1; st >>= 1) {
+                    const int ic = __shfl_sync(0xffffffffu, rinc, k + st - 1);
+                    if (ic <= f) k += st;
+                }
+                k = min(k, 31);
+                const int i = __shfl_sync(0xffffffffu, ii, k);
+                const int p = __shfl_sync(0xffffffffu, rb, k) + f - __shfl_sync(0xffffffffu, rinc - rl, k);
+                const int j = f < npairs ? a.ci[p] : 0;
+                const int m = f < npairs ? a.pcnt[j] : 0;
+                int cnt = 0;  // the pair's products of this pass
+                for (int sl = 0; sl < m; ++sl) {
                     const int J = a.pcol[(int64_t)j * a.c + sl];
-                    if (J >= lo && J < mn) mn = J;
+                    cnt += J >= lo && J < hi;
+                }
+                int incl = cnt;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, incl, d);
+                    if (lane >= d) incl += v;
+                }
+                const int nb = __shfl_sync(0xffffffffu, incl, 31);
+                if (cnt > 0) {  // staged in definition order
+                    const T qv = a.qv[qc + k];
+                    const T qb = mul_rn(qv, a.bv[p]);
+                    const T qt = a.tv ? mul_rn(qv, a.tv[p]) : (j == i ? qv : T(0));
+                    int e = incl - cnt;
+                    for (int sl = 0; sl < m; ++sl) {
+                        const int J = a.pcol[(int64_t)j * a.c + sl];
+                        if (J < lo || J >= hi) continue;
+                        const T pv = a.pval[(int64_t)j * a.c + sl];
+                        sJ[e] = J;
+                        sb_[e] = mul_rn(qb, pv);
+                        st_[e] = mul_rn(qt, pv);
+                        ++e;
+                    }
+                }
+                __syncwarp();
+                for (int e0 = 0; e0 < nb; e0 += 32) {
+                    const int e = e0 + lane;
+                    const int J = e < nb ? sJ[e] : -1 - lane;
+                    const unsigned grp = __match_any_sync(0xffffffffu, J);
+                    bool claimed = false;
+                    if (e < nb && (grp & lt) == 0u) {
+                        const int slot = gal_slot(hkey, J, claimed);  // at most 1536 + 128 are taken
+                        T vb = hvb[slot], vt = hvt[slot];
+                        for (unsigned g = grp; g; g &= g - 1u) {  // the group's products in lane order
+                            const int l2 = e0 + __ffs(g) - 1;
+                            vb = add_rn(vb, sb_[l2]);
+                            vt = add_rn(vt, st_[l2]);
+                        }
+                        hvb[slot] = vb;
+                        hvt[slot] = vt;
+                    }
+                    used += __popc(__ballot_sync(0xffffffffu, claimed));
+                    __syncwarp();
+                }
+                if (used > GAL_HSLOTS / 4 * 3) {  // keep the lower half: through the row's own place, and back
+                    const int mid = gal_sort_slots(hkey, skeys) / 2;
+                    hi = (int)(skeys[mid] >> 32);
+                    gal_write_slots(a, o, done, mid, hvb, hvt, skeys);
+                    __syncwarp();
+                    clear();
+                    for (int e = lane; e < mid; e += 32) {  // each lane what it has written itself
+                        bool c = false;
+                        const int slot = gal_slot(hkey, a.uJ[o + done + e], c);
+                        hvb[slot] = a.ubv[o + done + e];
+                        hvt[slot] = a.utv[o + done + e];
+                    }
+                    used = mid;
+                    __syncwarp();
                 }
             }
         }
-        mn = __reduce_min_sync(0xffffffffu, mn);
-        if (mn == 0x7fffffff) break;
-        lo = mn;
-        for (int e = lane; e < GAL_HSLOTS; e += 32) {
-            seen[e] = 0;
-            tvb[e] = T(0);
-            tvt[e] = T(0);
-        }
+        const int u = gal_sort_slots(hkey, skeys);
+        gal_write_slots(a, o, done, u, hvb, hvt, skeys);
+        done += u;
         __syncwarp();
-        for (int q = q0; q < q1; ++q) {
-            const int i = a.qci[q];
-            const T qq = a.qv[q];
-            for (int p = a.rp[i]; p < a.rp[i + 1] && lane == 0; ++p) {  // (rows this long are rare)
-                const int j = a.ci[p];
-                const T qb = mul_rn(qq, a.bv[p]), qt = a.tv ? mul_rn(qq, a.tv[p]) : (j == i ? qq : T(0));
-                for (int sl = 0; sl < a.pcnt[j]; ++sl) {
-                    const int J = a.pcol[(int64_t)j * a.c + sl];
-                    if (J < lo || J - lo >= GAL_HSLOTS) continue;
-                    const T pv = a.pval[(int64_t)j * a.c + sl];
-                    const T vb = mul_rn(qb, pv), vt = mul_rn(qt, pv);
-                    const bool first = seen[J - lo] == 0;
-                    tvb[J - lo] = first ? vb : add_rn(tvb[J - lo], vb);
-                    tvt[J - lo] = first ? vt : add_rn(tvt[J - lo], vt);
-                    seen[J - lo] = 1;
-                }
-            }
-        }
-        __syncwarp();
-        for (int e0 = 0; e0 < GAL_HSLOTS; e0 += 32) {
-            const int e = e0 + lane;
-            const unsigned bal = __ballot_sync(0xffffffffu, seen[e] != 0);
-            if (seen[e]) {
-                const int at = o + done + __popc(bal & lt);
-                a.uJ[at] = lo + e;
-                a.ubv[at] = tvb[e];
-                a.utv[at] = tvt[e];
-            }
-            done += __popc(bal);
-        }
-        __syncwarp();
-        if (lo > 0x7fffffff - GAL_HSLOTS) break;
-        lo += GAL_HSLOTS;
+        if (hi == 0x7fffffff) break;
+        lo = hi;
     }
     if (lane == 0) a.ucnt[I] = done;
     __syncwarp();
@@ -1940,7 +2012,8 @@ __global__ void __launch_bounds__(32) k_gal_large(const __grid_constant__ GalArg
     const int cnt = *nlist;
     for (int k = blockIdx.x; k < cnt; k += gridDim.x) {
         const int I = list[k];
-        if (!gal_row_hash<T>(a, I, hkey, hvb, hvt, sJ, sb_, st_, skeys)) gal_row_ranges<T>(a, I, hkey, hvb, hvt);
+        if (!gal_row_hash<T>(a, I, hkey, hvb, hvt, sJ, sb_, st_, skeys))
+            gal_row_blocks<T>(a, I, hkey, hvb, hvt, sJ, sb_, st_, skeys);
     }
 }
 
