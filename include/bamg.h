@@ -185,9 +185,10 @@ enum { BAMG_X_GUESS = 1, BAMG_X_HOST = 2, BAMG_NORM_L2 = 4 };
 int bamg_solve(bamg_handle* h, double* x, int flags, double tol, bamg_stats* st);
 
 /* Batched form: sets up and solves nchains independent chains to ||B x||_1/||x||_1 <= tol
- * and frees them, with nworkers host threads (0: one per chain, at most 16, fewer for
- * chains of many GB), each driving its own non-blocking stream; chains are taken largest
- * first from a shared queue, so the small latency-bound kernels of several chains overlap on the GPU.
+ * and frees them, with nworkers host threads (0: one per chain, at most 16, down to one per
+ * four chains where those in flight would take half of the free memory or 16 GiB), each
+ * driving its own non-blocking stream; chains are taken largest first from a shared queue, so
+ * the small latency-bound kernels of several chains overlap on the GPU.
  * As[k], r[k], levels[k], opts[k] as for bamg_setup (opts[k].stream is ignored);
  * xs[k]: n_k doubles for the result, device memory unless flags has BAMG_X_HOST
  * (BAMG_X_GUESS is not accepted).  st (may be NULL) receives one entry per chain.

@@ -15,6 +15,7 @@
 #include <thread>
 #include <type_traits>
 
+#include "batch_plan.cuh"
 #include "gmres_state.cuh"
 #include "kernels.cuh"
 
@@ -81,6 +82,20 @@ static cudaMemPool_t mem_pool() {
     return pool;
 }
 void pool_alloc(void** p, size_t bytes, cudaStream_t s) { BAMG_CK(cudaMallocFromPoolAsync(p, bytes, mem_pool(), s)); }
+
+// Bytes that allocations on the current device can still have: what the device has free and what the pool
+// holds unused (0 where the runtime does not say; throws nothing).
+static size_t memory_at_hand() {
+    int dev = 0;
+    size_t free = 0, total = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaMemGetInfo(&free, &total) != cudaSuccess) return 0;
+    const cudaMemPool_t pool = dev >= 0 && dev < 64 ? g_pool[dev].load() : nullptr;
+    uint64_t reserved = 0, used = 0;
+    if (pool && cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
+        free += reserved - used;
+    return free;
+}
 
 // The private streams of solvers that are gone, with their fence events: up to STREAMS_KEPT per
 // device (creating them takes some 50 us a solver).
@@ -1701,29 +1716,18 @@ int bamg_solve_batch(int nchains, const bamg_csr* As, const int* r, const int* l
         return BAMG_EINVAL;
     }
     if (nchains == 0) return BAMG_OK;
-    const bool choose = nworkers <= 0;
-    if (choose) nworkers = 16;
-    nworkers = std::min(nworkers, nchains);
     // largest chains first: the queue ends with the short jobs
     std::vector<int> order(nchains);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return As[a].n > As[b].n; });
-    if (choose) {
-        // a thread per chain up to 16: 12 chains of 32..60 squared states in FP64 took 10.8 ms on 3 threads
-        // and 5.9 on 12, 32 chains 15.1 on 8 and 14.6 on 16, 96 chains 55.7 on 8 and 50.0 on 16.  More than
-        // a thread per four chains only while the largest chains together (Krylov and test vectors in
-        // FP64, some ten copies of the matrix) stay below 16 GiB, so that what fitted the device with fewer
-        // in flight does not overflow it: chains of that size fill the GPU by themselves.
-        double bytes = 0.0;
-        int fit = 0;
-        for (; fit < nworkers; ++fit) {
-            const int k = order[fit];
-            const double m = std::min(std::max(opts[k].gmres_m, 1), GMRES_MMAX);
-            bytes += As[k].n * (16.0 * (m + 2) + 40.0 * std::max(r[k], 0) + 400.0) + 160.0 * As[k].nnz;
-            if (!(bytes < 16.0 * (1ull << 30))) break;
-        }
-        nworkers = std::max(fit, std::min(nworkers, std::max(1, (nchains + 3) / 4)));
+    if (nworkers <= 0) {
+        std::vector<BatchChain> chains;
+        for (int k : order)
+            chains.push_back({As[k].n, As[k].nnz, r[k], std::min(opts[k].gmres_m, GMRES_MMAX), opts[k].caliber,
+                              opts[k].precision == BAMG_PREC_FP64, opts[k].interp == BAMG_INTERP_LEARNED});
+        nworkers = batch_workers(chains, (double)memory_at_hand());
     }
+    nworkers = std::min(nworkers, nchains);
     std::atomic<int> next{0};
     std::mutex mu;
     int first_code = BAMG_OK;
