@@ -309,7 +309,8 @@ __device__ __forceinline__ void net_lda(uint32_t (&a)[4], const __nv_bfloat16* t
                  : "r"((unsigned)__cvta_generic_to_shared(p)));
 }
 // The warp's 32 columns (from c0) of a row tile in the A-operand layout, to the tile in shared
-// memory and to rows ra, rb of a row-major bf16 matrix
+// memory and to rows ra, rb of a row-major bf16 matrix (OUT)
+template <bool OUT = true>
 __device__ __forceinline__ void step_put(__nv_bfloat16* tile, __nv_bfloat16* __restrict__ O, const uint32_t (&H)[2][4],
                                          int c0, int64_t ra, int64_t rb, bool va, bool vb, int g, int t) {
 #pragma unroll
@@ -321,8 +322,8 @@ __device__ __forceinline__ void step_put(__nv_bfloat16* tile, __nv_bfloat16* __r
                 *reinterpret_cast<uint32_t*>(tile + g * NET_LD2 + c) = H[k][2 * e];
                 *reinterpret_cast<uint32_t*>(tile + (g + 8) * NET_LD2 + c) = H[k][2 * e + 1];
             }
-            if (va) *reinterpret_cast<uint32_t*>(O + ra * MLP_H + c) = H[k][2 * e];
-            if (vb) *reinterpret_cast<uint32_t*>(O + rb * MLP_H + c) = H[k][2 * e + 1];
+            if (OUT && va) *reinterpret_cast<uint32_t*>(O + ra * MLP_H + c) = H[k][2 * e];
+            if (OUT && vb) *reinterpret_cast<uint32_t*>(O + rb * MLP_H + c) = H[k][2 * e + 1];
         }
 }
 // relu(acc + bias) of the warp's 32 columns, rounded
@@ -360,9 +361,11 @@ __device__ __forceinline__ void step_mask(uint32_t (&O)[2][4], const float (&acc
 // memory: a batch of 4096 rows has only 256 tiles, and one warp through all the products of a
 // tile took 13 us of dependent instructions.  `early`: X was complete before the preceding kernel
 // began, so the first feature tile is fetched while that one still runs.
+//
+// KEEP: the rounded gradients are left in memory beside the unrounded ones (gradients() chooses).
 constexpr int STEP_GROUPS = 2, STEP_WARPS = 4 * STEP_GROUPS;
 struct StepOut {
-    __nv_bfloat16 *H1, *H2, *D1, *D2, *D3;  // activations and rounded gradients, M x 128 (D3: M x 16)
+    __nv_bfloat16 *H1, *H2, *D1, *D2, *D3;  // activations and rounded gradients, M x 128 (D3: M x 16; D with KEEP)
     float *F1, *F2, *F3;                    // the gradients unrounded
     float* G;                               // the flat gradient
     double* loss;
@@ -380,6 +383,7 @@ __device__ __forceinline__ void step_fetch(float* buf, const float* __restrict__
                                            int w, int lane) {
     if (r0 + 4 * w < M) net_fetch<4>(buf + 4 * w * NET_LDX, X, r0 + 4 * w, M, wide, lane);
 }
+template <bool KEEP>
 __global__ void __launch_bounds__(STEP_WARPS * 32)
     k_mlp_step(int64_t M, const float* __restrict__ X, const float* __restrict__ Tg, const __nv_bfloat16* __restrict__ Wb,
                const float* __restrict__ P, const StepOut out, bool early) {
@@ -460,11 +464,11 @@ __global__ void __launch_bounds__(STEP_WARPS * 32)
             if (w == 0) {
                 const int c = n * 8 + 2 * t;
                 if (va) {
-                    *reinterpret_cast<uint32_t*>(out.D3 + ra * MLP_S + c) = D3[2 * n];
+                    if (KEEP) *reinterpret_cast<uint32_t*>(out.D3 + ra * MLP_S + c) = D3[2 * n];
                     *reinterpret_cast<float2*>(out.F3 + ra * MLP_S + c) = make_float2(d[0], d[1]);
                 }
                 if (vb) {
-                    *reinterpret_cast<uint32_t*>(out.D3 + rb * MLP_S + c) = D3[2 * n + 1];
+                    if (KEEP) *reinterpret_cast<uint32_t*>(out.D3 + rb * MLP_S + c) = D3[2 * n + 1];
                     *reinterpret_cast<float2*>(out.F3 + rb * MLP_S + c) = make_float2(d[2], d[3]);
                 }
             }
@@ -480,7 +484,7 @@ __global__ void __launch_bounds__(STEP_WARPS * 32)
             mma_bf16(acc[n + 1], D3[0], D3[1], D3[2], D3[3], b[2], b[3]);
         }
         step_mask(D, acc, H2, out.F2, c0, ra, rb, va, vb, t);
-        step_put(h1t, out.D2, D, c0, ra, rb, va, vb, g, t);  // over H1: every warp has read it
+        step_put<KEEP>(h1t, out.D2, D, c0, ra, rb, va, vb, g, t);  // over H1: every warp has read it
         step_sync(group);
 #pragma unroll
         for (int k = 0; k < MLP_H / 16; ++k) net_lda(A[k], h1t, k, lane);
@@ -498,7 +502,7 @@ __global__ void __launch_bounds__(STEP_WARPS * 32)
                 mma_bf16(acc[n + 1], A[k][0], A[k][1], A[k][2], A[k][3], b[2], b[3]);
             }
         step_mask(D, acc, H1, out.F1, c0, ra, rb, va, vb, t);
-        step_put(nullptr, out.D1, D, c0, ra, rb, va, vb, g, t);
+        if (KEEP) step_put(nullptr, out.D1, D, c0, ra, rb, va, vb, g, t);
         // the next tile's H1 goes over D2 after the barrier at its start
     }
     if (w == 0) {
@@ -542,6 +546,21 @@ __device__ __forceinline__ void wg_stage(__nv_bfloat16* s, const __nv_bfloat16* 
             net_cp16(s + r * LDS + c, src + (m0 + r) * LDG + c0 + c);
         else
             *reinterpret_cast<uint4*>(s + r * LDS + c) = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+// the same from FP32, rounded here
+template <int C, int LDG, int LDS>
+__device__ __forceinline__ void wg_stage(__nv_bfloat16* s, const float* __restrict__ src, int c0, int64_t m0, int cnt) {
+    constexpr int Q = C / 4;
+#pragma unroll
+    for (int e = threadIdx.x; e < WG_MC * Q; e += WG_WARPS * 32) {
+        const int r = e / Q, c = 4 * (e - r * Q);
+        uint2 v = make_uint2(0u, 0u);
+        if (r < cnt) {
+            const float4 f = *reinterpret_cast<const float4*>(src + (m0 + r) * LDG + c0 + c);
+            v = make_uint2(pack_bf16(f.x, f.y), pack_bf16(f.z, f.w));
+        }
+        *reinterpret_cast<uint2*>(s + r * LDS + c) = v;
     }
 }
 // the warp's tile of MT m16 (all of the slab) x 2 n8 outputs, k columns from kc
@@ -616,6 +635,7 @@ __device__ __forceinline__ void wg_colsum8(float* s, int64_t M, int N, int n0, c
     }
     __syncthreads();
 }
+template <bool KEEP>
 __global__ void __launch_bounds__(WG_WARPS * 32, 2)
     k_mlp_wgrad(int64_t M, int64_t rows, const float* __restrict__ X, const StepOut in) {
     pdl_begin();
@@ -650,10 +670,12 @@ __global__ void __launch_bounds__(WG_WARPS * 32, 2)
     for (int64_t m0 = m_begin; m0 < m_end; m0 += WG_MC) {
         const int cnt = (int)(m_end - m0 < WG_MC ? m_end - m0 : WG_MC);
         if (job < 4) {
-            wg_stage<32, MLP_H, WG_LDD>(sD, in.D2, 32 * job, m0, cnt);
+            if constexpr (KEEP) wg_stage<32, MLP_H, WG_LDD>(sD, in.D2, 32 * job, m0, cnt);
+            else wg_stage<32, MLP_H, WG_LDD>(sD, in.F2, 32 * job, m0, cnt);
             wg_stage<MLP_H, MLP_H, WG_LDX>(sX, in.H1, 0, m0, cnt);
         } else if (job < 8) {
-            wg_stage<32, MLP_H, WG_LDD>(sD, in.D1, 32 * (job - 4), m0, cnt);
+            if constexpr (KEEP) wg_stage<32, MLP_H, WG_LDD>(sD, in.D1, 32 * (job - 4), m0, cnt);
+            else wg_stage<32, MLP_H, WG_LDD>(sD, in.F1, 32 * (job - 4), m0, cnt);
             constexpr int Q = MLP_F / 2;
 #pragma unroll 14
             for (int e = threadIdx.x; e < WG_MC * Q; e += WG_WARPS * 32) {
@@ -661,7 +683,8 @@ __global__ void __launch_bounds__(WG_WARPS * 32, 2)
                 *reinterpret_cast<uint32_t*>(sX + r * WG_LDX + c) = r < cnt ? load_pair(X + (m0 + r) * MLP_F + c) : 0u;
             }
         } else {
-            wg_stage<MLP_S, MLP_S, WG_LDD>(sD, in.D3, 0, m0, cnt);
+            if constexpr (KEEP) wg_stage<MLP_S, MLP_S, WG_LDD>(sD, in.D3, 0, m0, cnt);
+            else wg_stage<MLP_S, MLP_S, WG_LDD>(sD, in.F3, 0, m0, cnt);
             wg_stage<MLP_H, MLP_H, WG_LDX>(sX, in.H2, 0, m0, cnt);
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
@@ -742,17 +765,25 @@ void mlp_get(const Model* m, float* h_params, cudaStream_t s) {
     BAMG_CK(cudaStreamSynchronize(s));
 }
 
-// Activations and gradients (rounded and not) of one batch of rows, and the loss sum.
+// Activations and gradients (rounded and not) of one batch of rows, and the loss sum: 2144 bytes a row up to
+// KEEP_ROWS (0.6 GB).  A larger batch leaves the rounded gradients out, 1600 bytes a row, and k_mlp_wgrad
+// rounds the others as it reads them: the same bits, and no more traffic (what the step kernel does not
+// write, k_mlp_wgrad reads).  4,000,000 rows took 8160 MiB and 21.6 ms with them, 6080 MiB and 20.3 ms without;
+// 262,145 rows 1.19 ms and 1.09.  (Slices of 262,144 rows instead: 600 MiB, but 25.1 ms.)
+constexpr int64_t KEEP_ROWS = 1 << 18;
 struct MlpWork {
     DevBuf<__nv_bfloat16> H1, H2, D1, D2, D3;
     DevBuf<float> F1, F2, F3;
     DevBuf<double> loss;
-    explicit MlpWork(int64_t rows) {
+    bool keep;  // the rounded gradients have a place of their own
+    explicit MlpWork(int64_t rows) : keep(rows <= KEEP_ROWS) {
         H1.alloc(rows * MLP_H);
         H2.alloc(rows * MLP_H);
-        D1.alloc(rows * MLP_H);
-        D2.alloc(rows * MLP_H);
-        D3.alloc(rows * MLP_S);
+        if (keep) {
+            D1.alloc(rows * MLP_H);
+            D2.alloc(rows * MLP_H);
+            D3.alloc(rows * MLP_S);
+        }
         F1.alloc(rows * MLP_H);
         F2.alloc(rows * MLP_H);
         F3.alloc(rows * MLP_S);
@@ -787,20 +818,25 @@ void mlp_forward(const Model* m, int64_t rows, const float* feat, float* Y, cuda
 }
 
 // Gradients of the batch loss added to m->G; the loss sum into w.loss.
-static void gradients(Model* m, int64_t rows, const float* feat, const float* target, MlpWork& w, bool early,
-                      cudaStream_t s) {
+template <bool KEEP>
+static void gradients_as(Model* m, int64_t rows, const float* feat, const float* target, MlpWork& w, bool early,
+                         cudaStream_t s) {
     static std::atomic<bool> allowed[256] = {}, allowed_w[256] = {};
-    const int nsm = net_device(k_mlp_step, sizeof(StepSmem), allowed);
-    net_device(k_mlp_wgrad, WG_SMEM, allowed_w);
+    const int nsm = net_device(k_mlp_step<KEEP>, sizeof(StepSmem), allowed);
+    net_device(k_mlp_wgrad<KEEP>, WG_SMEM, allowed_w);
     const StepOut out{w.H1.get(), w.H2.get(), w.D1.get(), w.D2.get(), w.D3.get(),
                       w.F1.get(), w.F2.get(), w.F3.get(), m->G.get(), w.loss.get()};
-    BAMG_LAUNCH(k_mlp_step, (unsigned)std::min<int64_t>(nsm, (rows + 15) / 16), STEP_WARPS * 32, sizeof(StepSmem), s,
-                rows, feat, target, (const __nv_bfloat16*)m->Wb.get(), (const float*)m->P.get(), out, early);
+    BAMG_LAUNCH(k_mlp_step<KEEP>, (unsigned)std::min<int64_t>(nsm, (rows + 15) / 16), STEP_WARPS * 32, sizeof(StepSmem),
+                s, rows, feat, target, (const __nv_bfloat16*)m->Wb.get(), (const float*)m->P.get(), out, early);
     // up to two blocks per SM over the jobs, in whole chunks of rows
     const int64_t chunks = (rows + WG_MC - 1) / WG_MC, per = (chunks * WG_JOBS + 2 * nsm - 1) / (2 * nsm);
     const int64_t br = per * WG_MC;
-    BAMG_LAUNCH(k_mlp_wgrad, dim3((unsigned)((rows + br - 1) / br), WG_JOBS), WG_WARPS * 32, WG_SMEM, s, rows, br, feat,
-                out);
+    BAMG_LAUNCH(k_mlp_wgrad<KEEP>, dim3((unsigned)((rows + br - 1) / br), WG_JOBS), WG_WARPS * 32, WG_SMEM, s, rows, br,
+                feat, out);
+}
+static void gradients(Model* m, int64_t rows, const float* feat, const float* target, MlpWork& w, bool early,
+                      cudaStream_t s) {
+    (w.keep ? gradients_as<true> : gradients_as<false>)(m, rows, feat, target, w, early, s);
 }
 
 double mlp_gradients(Model* m, int64_t rows, const float* feat, const float* target, float* h_grad, cudaStream_t s) {

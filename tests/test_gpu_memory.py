@@ -70,3 +70,68 @@ def test_batch_leaves_fewer_in_flight_where_memory_is_short():
         assert all(s["status"] == 0 for s in stats)
         assert all(float((x - want).abs().sum()) <= 1e-3 and torch.equal(x, xs[0]) for x in xs)
         del xs
+
+
+def _features(rows):
+    import torch
+
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    feat = torch.randn(rows, 112, device="cuda", generator=g)
+    feat[:, 0:96:6] = (torch.rand(rows, 16, device="cuda", generator=g) < 0.7).float()
+    return feat, torch.randn(rows, 16, device="cuda", generator=g)
+
+
+def test_gradients_of_a_large_batch_in_little_memory():
+    """A batch of 4,000,000 rows with 7 GiB free beside its features: activations and gradients take 6104 MiB as long
+    as every number is kept once, 8160 with the rounded gradients beside the unrounded ones."""
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+
+    rows = 4000000
+    feat, target = _features(rows)
+    m = bamg.Model(3)
+    m.gradients(feat[:300000], target[:300000])  # loads the kernels
+    with _Only(7 << 30):
+        g, loss = m.gradients(feat, target)
+    d = torch.cat([m.forward(c) for c in feat.split(500000)]).double() - target
+    d *= feat[:, 0:96:6] > 0
+    assert loss == pytest.approx(float(d.square().sum()) / rows, rel=1e-6)
+    # 15,625 additions a partial sum and 13 to join the 256 of a column, each to 2^-24 of the sum of magnitudes
+    err = (torch.tensor(g[-16:], dtype=torch.float64) - (2 * d.sum(0) / rows).cpu()).abs()
+    assert bool((err <= (15625 + 13) * 2.0 ** -24 * (2 * d.abs().sum(0) / rows).cpu()).all())
+
+
+@pytest.mark.parametrize("rows", [2 ** 18, 2 ** 18 + 1, 2 ** 18 + 256 * 7 + 17])
+def test_gradients_where_the_rounded_ones_are_not_kept(rows):
+    """On both sides of the row count from which the rounded gradients have no place of their own, against the network
+    with the same roundings in 64 bits: a bf16 rounding that falls the other way moves an entry by at most 2^-8 of
+    itself, so each gradient by at most 2^-8 of its norm."""
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+
+    def bf(x):
+        return x.to(torch.bfloat16).double()
+
+    feat, target = _features(rows)
+    m = bamg.Model(3)
+    p = torch.tensor(m.get(), device="cuda").double()
+    p += 0.02 * torch.rand(p.shape, generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    m.set(p.cpu().numpy())
+    p = p.float().double()
+    W1, b1, W2, b2, W3, b3 = (t for t in torch.split(p, [128 * 112, 128, 128 * 128, 128, 16 * 128, 16]))
+    W1, W2, W3 = W1.view(128, 112), W2.view(128, 128), W3.view(16, 128)
+    x = bf(feat)
+    h1 = bf((x @ bf(W1).T + b1).relu().float())
+    h2 = bf((h1 @ bf(W2).T + b2).relu().float())
+    d3 = 2 * ((h2 @ bf(W3).T + b3) - target) * (feat[:, 0:96:6] > 0) / rows
+    d2 = (bf(d3.float()) @ bf(W3)) * (h2 > 0)
+    d1 = (bf(d2.float()) @ bf(W2)) * (h1 > 0)
+    want = [bf(d1.float()).T @ x, d1.sum(0), bf(d2.float()).T @ h1, d2.sum(0), bf(d3.float()).T @ h2, d3.sum(0)]
+    g, _ = m.gradients(feat, target)
+    at = 0
+    for w in want:
+        part = torch.tensor(g[at:at + w.numel()], device="cuda").double().view(w.shape)
+        at += w.numel()
+        assert float((part - w).norm()) <= 2.0 ** -8 * float(w.norm())
