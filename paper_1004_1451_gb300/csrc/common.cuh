@@ -27,6 +27,7 @@ void set_last_error(const std::string& msg);
     do {                                                                                           \
         cudaError_t e_ = (call);                                                                   \
         if (e_ != cudaSuccess) {                                                                   \
+            cudaGetLastError(); /* this call's answer, not the next launch's */                     \
             throw ::bamg::Error(e_ == cudaErrorMemoryAllocation ? BAMG_ENOMEM : BAMG_ECUDA,        \
                                 std::string(#call) + ": " + cudaGetErrorString(e_));               \
         }                                                                                          \

@@ -135,3 +135,26 @@ def test_gradients_where_the_rounded_ones_are_not_kept(rows):
         part = torch.tensor(g[at:at + w.numel()], device="cuda").double().view(w.shape)
         at += w.numel()
         assert float((part - w).norm()) <= 2.0 ** -8 * float(w.norm())
+
+
+def test_calls_after_one_that_ran_out_of_memory():
+    """A call that the device has no memory for says so; the calls after it, on the same thread, run."""
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+
+    big, _ = _walk(1400, 1400)
+    small, want = _walk(60, 50)
+    opts = {"grid": (60, 50), "precision": "fp64"}
+    bamg.solve_batch([small], 8, 20, 1e-10, opts=opts)  # loads the kernels
+    with _Only(1 << 30):
+        with pytest.raises(bamg.BamgError) as e:
+            bamg.Solver(*big, r=8, levels=20, grid=(1400, 1400), precision="fp64")
+        assert e.value.code == -4
+        x, _ = bamg.Solver(*small, r=8, levels=20, **opts).solve(1e-10)
+        assert float((x - want).abs().sum()) <= 1e-6
+        with pytest.raises(bamg.BamgError) as e:
+            bamg.solve_batch([small, big, small], 8, 20, 1e-10, workers=1,
+                             opts=[opts, {"grid": (1400, 1400), "precision": "fp64"}, opts])
+        assert e.value.code == -4 and [s["status"] for s in e.value.stats] == [0, -4, 0]
+        assert torch.equal(e.value.xs[0], e.value.xs[2]) and float((e.value.xs[0] - want).abs().sum()) <= 1e-6
