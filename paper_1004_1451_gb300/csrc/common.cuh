@@ -4,10 +4,12 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <iterator>
 #include <map>
+#include <set>
 #include <stdexcept>
 #include <string>
-#include <unordered_map>
+#include <utility>
 #include <vector>
 
 #include "../../include/bamg.h"
@@ -98,39 +100,78 @@ void pool_trim();  // of the current device
 // back into a free list (at once, for buffers are reused in the order of the solver's streams, which
 // are fenced against one another).  A setup allocates some 200 of them, at 2 us each, and at 30 us with
 // eight host threads in the allocator at a time.  Blocks above MAX_SLICE come from the pool
-// directly.  The chunks are freed with the solver.
+// directly.  The chunks are freed with the solver, so what they hold beyond its buffers is a live handle's
+// cost: the first has the size that the owner expects, each later one a sixth of what is there; a free slice
+// larger than asked for gives up its rest, and neighbours that are free join.  (Chunks from 2 MiB doubling up to 32 and whole slices
+// up to twice the size: 62 MiB of chunks for 27 of buffers on 200 x 200 states in FP64, now 33.)
 struct DevArena {
-    static constexpr size_t MAX_SLICE = size_t(4) << 20, FIRST_CHUNK = size_t(2) << 20, MAX_CHUNK = size_t(32) << 20;
+    static constexpr size_t MAX_SLICE = size_t(4) << 20, MIN_CHUNK = size_t(512) << 10, MAX_CHUNK = size_t(24) << 20;
     struct Chunk {
         char* base;
         size_t cap, top;
         cudaStream_t s;
     };
+    struct Slice {
+        size_t bytes;
+        size_t chunk;
+        bool free;
+    };
     std::vector<Chunk> chunks;
-    std::multimap<size_t, char*> free_;
-    std::unordered_map<char*, size_t> size_;
+    std::map<char*, Slice> slices;              // every slice, in the order of addresses
+    std::set<std::pair<size_t, char*>> unused;  // the free ones by size
+    size_t held = 0, first = 0;
+    void expect(size_t bytes) { first = bytes < MAX_CHUNK ? (bytes + 255) & ~size_t(255) : MAX_CHUNK; }
     void* alloc(size_t bytes, cudaStream_t s) {
         bytes = (bytes + 255) & ~size_t(255);
-        auto it = free_.lower_bound(bytes);
-        if (it != free_.end() && it->first <= 2 * bytes) {
+        const auto it = unused.lower_bound({bytes, nullptr});
+        if (it != unused.end()) {
             char* p = it->second;
-            free_.erase(it);
+            unused.erase(it);
+            Slice& sl = slices.at(p);
+            sl.free = false;
+            if (sl.bytes > bytes) {
+                slices.emplace(p + bytes, Slice{sl.bytes - bytes, sl.chunk, true});
+                unused.insert({sl.bytes - bytes, p + bytes});
+                sl.bytes = bytes;
+            }
             return p;
         }
         if (chunks.empty() || chunks.back().top + bytes > chunks.back().cap) {
-            const size_t next = chunks.empty() ? FIRST_CHUNK : 2 * chunks.back().cap;
-            const size_t cap = next < MAX_CHUNK ? next : MAX_CHUNK;
+            const size_t next = chunks.empty() ? first : (held / 6 + 255) & ~size_t(255);
+            const size_t cap = next < MIN_CHUNK ? MIN_CHUNK : next < MAX_CHUNK ? next : MAX_CHUNK;
             Chunk c{nullptr, cap > bytes ? cap : bytes, 0, s};
             pool_alloc((void**)&c.base, c.cap, s);
             chunks.push_back(c);
+            held += c.cap;
         }
         Chunk& c = chunks.back();
         char* p = c.base + c.top;
         c.top += bytes;
-        size_[p] = bytes;
+        slices.emplace(p, Slice{bytes, chunks.size() - 1, false});
         return p;
     }
-    void free(void* p) { free_.emplace(size_.at((char*)p), (char*)p); }
+    void free(void* q) {
+        auto it = slices.find((char*)q);
+        it->second.free = true;
+        const auto join = [&](std::map<char*, Slice>::iterator lo, std::map<char*, Slice>::iterator hi) {
+            lo->second.bytes += hi->second.bytes;
+            slices.erase(hi);
+        };
+        const auto next = std::next(it);
+        if (next != slices.end() && next->second.free && next->second.chunk == it->second.chunk) {
+            unused.erase({next->second.bytes, next->first});
+            join(it, next);
+        }
+        if (it != slices.begin()) {
+            const auto prev = std::prev(it);
+            if (prev->second.free && prev->second.chunk == it->second.chunk) {
+                unused.erase({prev->second.bytes, prev->first});
+                join(prev, it);
+                it = prev;
+            }
+        }
+        unused.insert({it->second.bytes, it->first});
+    }
     DevArena() = default;
     ~DevArena() {
         for (Chunk& c : chunks) cudaFreeAsync(c.base, c.s);

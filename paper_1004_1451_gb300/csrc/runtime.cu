@@ -789,6 +789,11 @@ struct Solver : SolverBase {
             ~Untrace() { p = nullptr; }
         } untrace_{trace};
         levels_max = levels;
+        {   // what the small buffers of this setup and its solve add up to: the Krylov vectors, and test vectors, rows
+            // of P and matrices of all levels (within 1% on chains of 200 to 65,536 states where all are small)
+            const double n = A->n, m = std::min(std::max(o.gmres_m, 1), GMRES_MMAX), w = sizeof(T);
+            darena.expect((size_t)(n * ((m + 1) * 8 + m * w + 160 + w * (29 + 1.5 * r_)) + A->nnz * (57 + 21.5 * w)));
+        }
         read_input(A, r_);
         const int n = A->n;
         tr.mark("input");

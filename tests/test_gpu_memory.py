@@ -158,3 +158,53 @@ def test_calls_after_one_that_ran_out_of_memory():
                              opts=[opts, {"grid": (1400, 1400), "precision": "fp64"}, opts])
         assert e.value.code == -4 and [s["status"] for s in e.value.stats] == [0, -4, 0]
         assert torch.equal(e.value.xs[0], e.value.xs[2]) and float((e.value.xs[0] - want).abs().sum()) <= 1e-6
+
+
+@pytest.mark.parametrize("nx,ny,count,mib", [(20, 10, 200, 1.0), (64, 64, 100, 9.2), (200, 200, 40, 89.0)])
+def test_a_kept_handle_holds_little_beyond_its_buffers(nx, ny, count, mib):
+    """Device memory of a hierarchy that has solved: its buffers (0.4, 7.4 and 73 MiB in FP64) and a quarter more, with what
+    the pool rounds up to shared by all."""
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+
+    A, _ = _walk(nx, ny)
+
+    def make():
+        s = bamg.Solver(*A, r=8, levels=20, grid=(nx, ny), precision="fp64")
+        s.solve(1e-8)
+        return s
+
+    make().close()
+    bamg.release_memory()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    handles = [make() for _ in range(count)]
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    held = free - torch.cuda.mem_get_info()[0]
+    for s in handles:
+        s.close()
+    bamg.release_memory()
+    assert held <= (count * mib + 64) * 2 ** 20
+
+
+def test_a_handle_does_not_grow_with_the_cycles_of_its_setup():
+    """Setups of more cycles rebuild the coarse operators more often in the same memory."""
+    import torch
+
+    import paper_1004_1451_gb300 as bamg
+
+    A, _ = _walk(64, 64)
+    held = []
+    for cycles in (2, 16):
+        bamg.release_memory()
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        handles = [bamg.Solver(*A, r=8, levels=20, grid=(64, 64), precision="fp64", setup_cycles=cycles) for _ in range(64)]
+        torch.cuda.synchronize()
+        held.append(free - torch.cuda.mem_get_info()[0])
+        for s in handles:
+            s.close()
+    bamg.release_memory()
+    assert held[1] <= held[0] + (32 << 20)
