@@ -772,6 +772,13 @@ struct Solver : SolverBase {
         BAMG_REQUIRE(!(h_err & 1), BAMG_EOVERFLOW, "neighbourhood search: a fine point needs more than 2048 recorded states");
     }
 
+    // What the small buffers of a hierarchy and its solve add up to: the Krylov vectors, and test vectors, rows of P and
+    // matrices of all levels (within 1% on chains of 200 to 65,536 states where all are small).
+    void expect_memory(double n, double nnz, int ncols) {
+        const double m = std::min(std::max(o.gmres_m, 1), GMRES_MMAX), w = sizeof(T);
+        darena.expect((size_t)(n * ((m + 1) * 8 + m * w + 160 + w * (29 + 1.5 * ncols)) + nnz * (57 + 21.5 * w)));
+    }
+
     // Bootstrap setup: o.setup_cycles MLE cycles, then the rebuild, B_L^+ and the initial
     // guess.  With `mle_tol` > 0 (the stand-alone MLE of Section 4.1) the cycles go on
     // until the state vector approximation meets the tolerance (2-norm ratio when
@@ -789,11 +796,7 @@ struct Solver : SolverBase {
             ~Untrace() { p = nullptr; }
         } untrace_{trace};
         levels_max = levels;
-        {   // what the small buffers of this setup and its solve add up to: the Krylov vectors, and test vectors, rows
-            // of P and matrices of all levels (within 1% on chains of 200 to 65,536 states where all are small)
-            const double n = A->n, m = std::min(std::max(o.gmres_m, 1), GMRES_MMAX), w = sizeof(T);
-            darena.expect((size_t)(n * ((m + 1) * 8 + m * w + 160 + w * (29 + 1.5 * r_)) + A->nnz * (57 + 21.5 * w)));
-        }
+        expect_memory(A->n, A->nnz, r_);
         read_input(A, r_);
         const int n = A->n;
         tr.mark("input");
@@ -862,6 +865,7 @@ struct Solver : SolverBase {
     // --------------------------------------------------------------- import
     void import(int nlev, const bamg_level_in* in, const double* h_pinv, const double* h_x_init) {
         AllocStream as_(s, &darena);
+        expect_memory(in[0].n, in[0].nnz, 0);
         lv.clear();
         for (int l = 0; l < nlev; ++l) {
             auto L = std::make_unique<LevelT<T>>();
