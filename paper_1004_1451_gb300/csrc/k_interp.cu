@@ -769,10 +769,11 @@ __global__ void __launch_bounds__(WARPS * 32, (WARPS > 1 && sizeof(T) == 4) ? 8 
     }
 }
 
-// ---------------------------------------------------------------- two points a warp
-// The fit without optional outputs, in two kernels: the neighbourhood searches, then the greedy
-// fits.  Each half of a warp takes one point, 16 lanes for the at most 16 candidates.  Same candidates
-// and the same arithmetic per candidate as ls_point, so the same rows bit for bit.
+// ---------------------------------------------------------------- several points a warp
+// The fit without optional outputs, in two kernels: the neighbourhood searches (half a warp a point, on
+// long rows a whole one), then the greedy fits (four points a warp with eight lanes each, or two with 16, a
+// candidate a lane).  Same candidates and the same arithmetic per candidate as ls_point, so the same rows
+// bit for bit.
 //
 // What bounds them: instruction issue and the chain of dependent loads (every operand sits in L1 or
 // L2).  One warp a point with half its lanes idle in the fit took 2240 warp instructions a fine point
@@ -1226,6 +1227,11 @@ int interp_ls(int n, int nnz, const int32_t* rp, const int32_t* ci, const T* bv,
             BAMG_LAUNCH(kern, grid, LSP_WARPS * 32, 0, s, n, cf, cidx, (const int32_t*)cand,
                         (const int32_t*)ncand, X, ncols, ld, d_w, mmax, c, ridge, vec, pcol, pval, pcnt);
         };
+        // A fit of NC columns and CM slots: up to two slots (the default) by the columns there are, because a
+        // lane's row in registers sets the blocks an SM (2^18 points, FP32: 263 us with 8 columns, 363 with
+        // 32).  Three or four slots take one form: its systems, not its columns, take the time in FP32 (404 us
+        // with 8 columns, 423 with 32; 462 and 489 with four), and in FP64 8 columns cost what 32 do
+        // (3.3 and 4.8 ms), which is still less than a point a warp took (5.3 and 7.4 ms; FP32 0.85 and 0.97).
         if (c <= 2) {
             if (ncols <= 8) go(k_ls_pair<T, 8, 2>);
             else if (ncols <= 16) go(k_ls_pair<T, 16, 2>);
@@ -2018,8 +2024,9 @@ __global__ void __launch_bounds__(32) k_gal_large(const __grid_constant__ GalArg
 }
 
 // The number of entries of B_c alone (the sizing call): every row's distinct J, counted by inserting
-// them into a table of GAL_SYM_S slots a warp (a row that fills three quarters of it goes to `list`),
-// or of GAL_SYM_L slots a block; a row that fills that too sets *over.
+// them into a table of GAL_SYM_S slots a warp, or for the rows it lists of GAL_SYM_L slots a block.  A table
+// gives up when a probe has passed a quarter of its slots (with J that spread, when it is nearly full): the
+// row is listed, or sets *over, after which the products are formed and counted.
 constexpr int GAL_SYM_S = 512, GAL_SYM_L = 8192;
 constexpr int GAL_SYM_SUMS = 64;  // partial totals, a sector apart: one address would take every row in turn
 template <int HS, int THREADS>

@@ -5,11 +5,12 @@
 // beta2 = 0.999, eps = 1e-8, He-uniform initialisation from SplitMix64) are those of the
 // interface declared in include/bamg.h.
 //
-// All products run on the tensor cores (mma.sync m16n8k16, bf16 in, FP32 accumulate): one
-// warp takes 16 rows through all layers, the weights staged once per block in shared
-// memory with a padded row stride.  The training backward's products (input gradients
-// through the ReLU masks, weight gradients summed over the batch) use the same instruction
-// with the incoming gradient rounded to bf16; bias gradients and Adam stay in FP32.
+// All products run on the tensor cores (mma.sync m16n8k16, bf16 in, FP32 accumulate), the
+// weights staged once per block in shared memory with a padded row stride: in the forward pass
+// one warp takes 16 rows through all layers, in a training step four warps do.  The training
+// backward's products (input gradients through the ReLU masks, weight gradients summed over the
+// batch) use the same instruction with the incoming gradient rounded to bf16; bias gradients and
+// Adam stay in FP32.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -279,11 +280,11 @@ __global__ void __launch_bounds__(NET_WARPS * 32)
 
 // ------------------------------------------------------------------ backward
 // A training step is two kernels and the optimiser.  k_mlp_step takes a row tile through the
-// forward pass, the masked loss and the input gradients in one warp: the gradient that enters a
-// product is rounded to bf16 like the forward's inputs, which again turns an accumulator into the
-// next product's A operand in place.  It leaves H1, H2 and the rounded gradients in memory (bf16)
-// for the weight gradients and the unrounded gradients (FP32) for the bias gradients (k_mlp_wgrad, all
-// layers in one launch), and adds up the loss.
+// forward pass, the masked loss and the input gradients in four warps, which pass it on through
+// shared memory; the gradient that enters a product is rounded to bf16 like the forward's inputs.  It
+// leaves H1, H2 and (up to KEEP_ROWS rows) the rounded gradients in memory (bf16) for the weight gradients
+// and the unrounded gradients (FP32) for the bias gradients (k_mlp_wgrad, all layers in one launch),
+// and adds up the loss.
 //
 // What bounds it: launches and latency (a batch of 4096 rows is 0.9 GFLOP and 6 MB; 10 us of
 // dependent instructions in k_mlp_step and 6 in k_mlp_wgrad, tensor pipe below 10%).  It took 14
