@@ -102,8 +102,9 @@ void pool_trim();  // of the current device
 // eight host threads in the allocator at a time.  Blocks above MAX_SLICE come from the pool
 // directly.  The chunks are freed with the solver, so what they hold beyond its buffers is a live handle's
 // cost: the first has the size that the owner expects, each later one a sixth of what is there; a free slice
-// larger than asked for gives up its rest, and neighbours that are free join.  (Chunks from 2 MiB doubling up to 32 and whole slices
-// up to twice the size: 62 MiB of chunks for 27 of buffers on 200 x 200 states in FP64, now 33.)
+// larger than asked for gives up its rest, and neighbours that are free join.  (With chunks from 2 MiB
+// doubling up to 32 and whole slices up to twice the size, 62 MiB of chunks held 27 of buffers on
+// 200 x 200 states in FP64, now 33.)
 struct DevArena {
     static constexpr size_t MAX_SLICE = size_t(4) << 20, MIN_CHUNK = size_t(512) << 10, MAX_CHUNK = size_t(24) << 20;
     struct Chunk {
@@ -137,6 +138,12 @@ struct DevArena {
             return p;
         }
         if (chunks.empty() || chunks.back().top + bytes > chunks.back().cap) {
+            if (!chunks.empty() && chunks.back().top < chunks.back().cap) {  // its rest, for smaller buffers
+                Chunk& c = chunks.back();
+                slices.emplace(c.base + c.top, Slice{c.cap - c.top, chunks.size() - 1, true});
+                unused.insert({c.cap - c.top, c.base + c.top});
+                c.top = c.cap;
+            }
             const size_t next = chunks.empty() ? first : (held / 6 + 255) & ~size_t(255);
             const size_t cap = next < MIN_CHUNK ? MIN_CHUNK : next < MAX_CHUNK ? next : MAX_CHUNK;
             Chunk c{nullptr, cap > bytes ? cap : bytes, 0, s};
